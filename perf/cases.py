@@ -54,11 +54,11 @@ def listed():
         _coupled("channel_ragged_ladd_f32", 141, 83, 119, "f32", 4, "clustered", (8, 32), (6.0, 9.0), 20, bb="ladd",
                  periodic="x", force=2e-6),
         # the settling tank, in both storages it is run with
-        _coupled("tank_f32", 256, 256, 512, "f32", 3, "cobble", (24, 40), (12.0, 20.0), 10),
-        _coupled("tank_f16", 256, 256, 512, "f16", 3, "cobble", (24, 40), (12.0, 20.0), 10),
+        _coupled("tank_f32", 256, 256, 512, "f32", 3, "cobble", (24, 40), (12.0, 20.0), 20),
+        _coupled("tank_f16", 256, 256, 512, "f16", 3, "cobble", (24, 40), (12.0, 20.0), 20),
         # the suspension of 300 particles: the largest lattice
-        _coupled("suspension_f32", 512, 512, 512, "f32", 300, "clustered", (8, 64), (8.0, 16.0), 5),
-        _coupled("suspension_bf16", 512, 512, 512, "bf16", 300, "clustered", (8, 64), (8.0, 16.0), 5),
+        _coupled("suspension_f32", 512, 512, 512, "f32", 300, "clustered", (8, 64), (8.0, 16.0), 10),
+        _coupled("suspension_bf16", 512, 512, 512, "bf16", 300, "clustered", (8, 64), (8.0, 16.0), 10),
         # a pair of grains in a channel with the paper's 100 DEM substeps per lattice step
         _coupled("pair_substeps_f32", 128, 128, 256, "f32", 2, "clustered", (16, 32), (9.0, 12.0), 5, substeps=100),
         # the packed bed: contacts alone
@@ -315,6 +315,7 @@ def prepare(case, seed):
         _flow(case, rng, lambda i, dev: pop[i].copy_(_stored(case, i, dev)))
         _add(sim, shapes, st)
         _hold_states(state, st)
+        state["zero"] = torch.zeros((), dtype=ELEMENT[case["storage"]], device="cuda")
         torch.cuda.synchronize()
         state["sim"] = sim
     elif kind == "bed":
@@ -363,7 +364,10 @@ def run(state):
                 if n:
                     # values at solid nodes are unspecified: the fluid's alone
                     owner = _view(v.owner, sim.shape, "<i4")
-                    out["populations"] = torch.where(owner == -1, pop, torch.zeros((), dtype=pop.dtype, device="cuda"))
+                    fluid, masked = owner == -1, torch.empty(pop.shape, dtype=pop.dtype, device="cuda")
+                    for i in range(19):  # plane by plane: contiguous, without an index per element
+                        torch.where(fluid, pop[i], state["zero"], out=masked[i])
+                    out["populations"] = masked
                     out["owner"] = owner.clone()
                     out["classes"] = _view(v.node_class, sim.shape, "|u1").clone()
                 else:

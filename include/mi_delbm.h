@@ -396,8 +396,8 @@ mi_status mi_mass_properties_noalloc(const double *balls_dev, int n_balls, doubl
  * Errors: MI_EINVAL (enable not 0, 1 or 2). */
 mi_status mi_delbm_set_graphs(mi_delbm *h, int enable);
 
-/* Choose the launch shapes of the bulk kernel (threads per block along x,
- * from 32/64/128/256) and of the list kernels (blocks per SM for the wall
+/* Choose the launch shapes of the bulk kernel (threads per block, from
+ * 32/64/128/256) and of the list kernels (blocks per SM for the wall
  * fraction, refill and boundary-node kernels, from 2/4/8/16/32; the links'
  * bounce-back and the boundary nodes are timed together) by timing each candidate
  * with CUDA events on the handle's stream, and use the fastest from then on.
@@ -452,13 +452,13 @@ enum {
 mi_status mi_delbm_set_momentum_rules(mi_delbm *h, int flags);
 
 /* Set the launch shapes directly (what mi_delbm_autotune chooses): bulk
- * kernel threads per block along x (32..256, a multiple of 32; at most 128
- * with pairs), rows per thread (1 or 2), paired nodes (0: no; 1 or 2: two
- * x-adjacent nodes per thread with paired accesses, used only when nx is
- * even; for 16-bit storages 1 and 2 select a 64- or 80-register budget;
- * 3: four x-adjacent nodes per thread with 64-bit accesses, 16-bit storages
- * with nx a multiple of 4 only, else the one-node kernel), list-kernel
- * blocks per SM (1..64).  Results do not depend on them. */
+ * kernel threads per block (32..256, a multiple of 32; at most 128 with
+ * pairs), rows per thread (1 or 2: accepted, both run one row), paired nodes
+ * (0: no; 1 or 2: two x-adjacent nodes per thread with paired accesses and a
+ * 64- or 80-register budget; 3: four x-adjacent nodes per thread with 64-bit
+ * accesses; used for 16-bit storages only, 1 and 2 with nx even and 3 with nx
+ * a multiple of 4, else the one-node kernel), list-kernel blocks per SM
+ * (1..64).  Results do not depend on them. */
 mi_status mi_delbm_set_tuning(mi_delbm *h, int bulk_block_x, int bulk_rows, int bulk_pairs, int list_blocks_per_sm);
 
 /* The launch shapes in use (any pointer may be NULL). */

@@ -385,7 +385,6 @@ mi_status mi_delbm::phase_bulk() {
   L.storage = cfg.storage;
   L.forcing = forcing();
   L.block_x = tune.bulk_block_x;
-  L.rows = tune.bulk_rows;
   L.pairs = tune.bulk_pairs != 0;
   L.pair_mode = tune.bulk_pairs;
   return launch_phase(this, stream, MI_PHASE_BULK, "k_bulk", [&] { return launch_bulk(L, stream); });
@@ -904,7 +903,7 @@ mi_status mi_delbm_create(const mi_delbm_config* cfg, mi_delbm** out) {
     mi_delbm_destroy(h);
     return MI_ECUDA;
   }
-  h->tune.bulk_block_x = cfg->nx >= 256 ? 128 : (cfg->nx >= 128 ? 64 : 32);
+  h->tune.bulk_block_x = 64;  // the one-node kernel's best from 64^3 to 512^3
   h->tune.bulk_rows = 1;
   h->tune.bulk_pairs = 0;
   if (cfg->storage != MI_STORE_F32 && cfg->nx % 4 == 0) {
@@ -1369,26 +1368,22 @@ extern "C" mi_status mi_delbm_autotune(mi_delbm* h, const char* cache_path, int*
     L.storage = h->cfg.storage;
     L.forcing = h->forcing();
     float best = 1e30f;
-    // variants: 1 row, 2 rows, paired nodes (two register budgets for 16-bit
-    // storages), four nodes per thread (16-bit storages)
-    for (int variant = 0; variant < 5; ++variant) {
-      const int pairs = variant >= 2 ? variant - 1 : 0;
-      if (pairs && (h->cfg.nx % 2) != 0) continue;
-      if (pairs >= 2 && h->cfg.storage == MI_STORE_F32) continue;
+    // variants: one node, paired nodes (16-bit storages, two register budgets),
+    // four nodes per thread (16-bit storages)
+    for (int pairs = 0; pairs < 4; ++pairs) {
+      if (pairs && (h->cfg.storage == MI_STORE_F32 || (h->cfg.nx % 2) != 0)) continue;
       if (pairs == 3 && (h->cfg.nx % 4) != 0) continue;
       for (int bx : {32, 64, 128, 256}) {
-        const int span = pairs == 3 ? 4 * bx : pairs ? 2 * bx : bx;
-        if (bx > 32 && span / 2 >= h->cfg.nx) break;
-        if (pairs && bx > 128) break;
+        const int span = pairs == 3 ? 4 * bx : 2 * bx;
+        if (pairs && ((bx > 32 && span / 2 >= h->cfg.nx) || bx > 128)) break;
         L.block_x = bx;
-        L.rows = variant == 1 ? 2 : 1;
         L.pairs = pairs != 0;
         L.pair_mode = pairs;
         const float ms = h->time_launches(5, [&] { return launch_bulk(L, h->stream); });
         if (ms > 0.f && ms < best) {
           best = ms;
           t.bulk_block_x = bx;
-          t.bulk_rows = L.rows;
+          t.bulk_rows = 1;
           t.bulk_pairs = pairs;
         }
       }

@@ -10,49 +10,145 @@
 // misaligned by one element for the 10 directions with e_x != 0; the L1/L2
 // absorb the sector overlap so DRAM sees each element once), FP32 collision,
 // 19 streaming stores.  Algorithmic traffic: 19 * 2 * sizeof(storage) bytes
-// per node update (+1 byte of node class when particles are present).
+// per node update.
 #include <climits>
 #include "mi_internal.cuh"
 
 namespace mi {
 
-// BGK collision on deviations h_i = f_i - w_i and store of the result.
+// Division of a 32-bit index by a constant of the launch: q = floor(c / d) by
+// a multiplication (Granlund and Montgomery 1994: with l = ceil(log2 d) and
+// m = floor(2^32 (2^l - d) / d) + 1, t = floor(m c / 2^32),
+// q = (t + (c - t) / 2) / 2^(l - 1)).
+struct FastDiv {
+  unsigned m, s1, s2;
+  __device__ __forceinline__ unsigned div(unsigned c) const {
+    const unsigned t = __umulhi(m, c);
+    return (t + ((c - t) >> s1)) >> s2;
+  }
+};
+static FastDiv fast_div(unsigned d) {
+  unsigned l = 0;
+  while (l < 32 && (1ull << l) < d) ++l;
+  return {(unsigned)((((1ull << l) - d) << 32) / d + 1), l > 1 ? 1u : l, l > 1 ? l - 1 : 0u};
+}
+
+// One or two nodes per value: the collision is written once over V = float (one
+// node) or V = F32x2 (two nodes, packed FP32 pairs: one instruction for both).
+// Every operation is a single rounding in both, so a node's result does not
+// depend on which of the two computed it.
+struct F32x2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vset(float s, float) { return s; }
+__device__ __forceinline__ F32x2 pack(float lo, float hi) {
+  F32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack(F32x2 a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vfma(F32x2 a, F32x2 b, F32x2 c) {
+  F32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vadd(F32x2 a, F32x2 b) {
+  F32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vsub(F32x2 a, F32x2 b) {
+  F32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vmul(F32x2 a, F32x2 b) {
+  F32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vset(float s, F32x2) { return pack(s, s); }
+
+// 1 / rho: the hardware approximation and one Newton step by FMA (no slow path)
+__device__ __forceinline__ float rcp_start(float a) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return r;
+}
+__device__ __forceinline__ F32x2 rcp_start(F32x2 a) {
+  const float2 v = unpack(a);
+  return pack(rcp_start(v.x), rcp_start(v.y));
+}
+
+// BGK collision on deviations h_i = f_i - w_i.
 //   rho = 1 + sum h_i, j = sum e_i h_i (sum w_i = 1, sum w_i e_i = 0)
 //   f_eq,i - w_i = w_i (rho - 1) + w_i rho (3 e.u + 4.5 (e.u)^2 - 1.5 u.u)
-//   h+_i = h_i + omega (f_eq,i - w_i - h_i)   [+ Guo source]
-template <bool FORCE>
-__device__ __forceinline__ void collide_inplace(float (&h)[19], const CollideParams& P) {
-  float drho = 0.f;
+//   h+_i = (1 - omega) h_i + omega (f_eq,i - w_i)   [+ Guo source]
+// A direction and its opposite (2k - 1, 2k) share the even part of f_eq and
+// take its odd part with either sign, and the moments come from their sums
+// and differences: about 130 operations a node, where forming each direction
+// by itself took 260.
+template <bool FORCE, class V>
+__device__ __forceinline__ void collide_inplace(V (&h)[19], const CollideParams& P) {
+  V s[10], d[10];  // pair k: h[2k - 1] + h[2k], h[2k - 1] - h[2k]
 #pragma unroll
-  for (int i = 0; i < 19; ++i) drho += h[i];
-  const float jx = (h[1] - h[2]) + (h[7] - h[8]) + (h[9] - h[10]) + (h[11] - h[12]) + (h[13] - h[14]);
-  const float jy = (h[3] - h[4]) + (h[7] - h[8]) + (h[10] - h[9]) + (h[15] - h[16]) + (h[17] - h[18]);
-  const float jz = (h[5] - h[6]) + (h[11] - h[12]) + (h[14] - h[13]) + (h[15] - h[16]) + (h[18] - h[17]);
-  const float rho = 1.0f + drho;
-  const float irho = 1.0f / rho;
-  float ux, uy, uz;
-  if (FORCE) {
-    ux = (jx + 0.5f * P.force[0]) * irho;
-    uy = (jy + 0.5f * P.force[1]) * irho;
-    uz = (jz + 0.5f * P.force[2]) * irho;
-  } else {
-    ux = jx * irho;
-    uy = jy * irho;
-    uz = jz * irho;
+  for (int k = 1; k < 10; ++k) {
+    s[k] = vadd(h[2 * k - 1], h[2 * k]);
+    d[k] = vsub(h[2 * k - 1], h[2 * k]);
   }
-  const float usq15 = 1.5f * (ux * ux + uy * uy + uz * uz);
+  const V drho = vadd(vadd(vadd(h[0], vadd(s[1], s[2])), vadd(s[3], vadd(s[4], s[5]))),
+                      vadd(vadd(s[6], s[7]), vadd(s[8], s[9])));
+  V u[3];
+  u[0] = vadd(vadd(d[1], vadd(d[4], d[5])), vadd(d[6], d[7]));
+  u[1] = vadd(vadd(d[2], vsub(d[4], d[5])), vadd(d[8], d[9]));
+  u[2] = vadd(vadd(d[3], vsub(d[6], d[7])), vsub(d[8], d[9]));
+  const V one = vset(1.0f, drho);
+  const V rho = vadd(one, drho);
+  V r = rcp_start(rho);
+  r = vfma(r, vfma(vsub(vset(0.0f, r), rho), r, one), r);
+  if (FORCE)
+    for (int a = 0; a < 3; ++a) u[a] = vadd(u[a], vset(0.5f * P.force[a], r));
+  for (int a = 0; a < 3; ++a) u[a] = vmul(u[a], r);
+  const V usq = vfma(u[0], u[0], vfma(u[1], u[1], vmul(u[2], u[2])));
   const float om = P.omega;
+  const V keep = vset(1.0f - om, r);
+  const V base = vfma(vmul(vset(-1.5f, r), rho), usq, drho);  // drho - 1.5 rho u.u
+  V uF;
+  if (FORCE) uF = vfma(vset(P.force[0], r), u[0], vfma(vset(P.force[1], r), u[1], vmul(vset(P.force[2], r), u[2])));
+  {
+    V e0 = vmul(vset(om * wq(0), r), base);
+    if (FORCE) e0 = vfma(vset(-3.0f * (1.0f - 0.5f * om) * wq(0), r), uF, e0);
+    h[0] = vfma(keep, h[0], e0);
+  }
+  const V basea = vmul(vset(om * wq(1), r), base), based = vmul(vset(om * wq(7), r), base);
+  const V k2a = vmul(vset(4.5f * om * wq(1), r), rho), k2d = vmul(vset(4.5f * om * wq(7), r), rho);
+  const V k1a = vmul(vset(3.0f * om * wq(1), r), rho), k1d = vmul(vset(3.0f * om * wq(7), r), rho);
 #pragma unroll
-  for (int i = 0; i < 19; ++i) {
-    const float eu = cx(i) * ux + cy(i) * uy + cz(i) * uz;
-    const float feq_dev = wq(i) * (drho + rho * (3.0f * eu + 4.5f * eu * eu - usq15));
-    float hp = h[i] + om * (feq_dev - h[i]);
+  for (int k = 1; k < 10; ++k) {
+    const int i = 2 * k - 1;
+    // e_i . u: the first non-zero component of every odd direction is +1
+    const V eu = k <= 3 ? u[k - 1]
+                        : (cx(i) ? (cy(i) ? (cy(i) > 0 ? vadd(u[0], u[1]) : vsub(u[0], u[1]))
+                                          : (cz(i) > 0 ? vadd(u[0], u[2]) : vsub(u[0], u[2])))
+                                 : (cz(i) > 0 ? vadd(u[1], u[2]) : vsub(u[1], u[2])));
+    V even = vfma(vmul(k <= 3 ? k2a : k2d, eu), eu, k <= 3 ? basea : based);
+    V odd = vmul(k <= 3 ? k1a : k1d, eu);
     if (FORCE) {
+      const float g = (1.0f - 0.5f * om) * wq(i);
       const float eF = cx(i) * P.force[0] + cy(i) * P.force[1] + cz(i) * P.force[2];
-      const float uF = ux * P.force[0] + uy * P.force[1] + uz * P.force[2];
-      hp += (1.0f - 0.5f * om) * wq(i) * (3.0f * (eF - uF) + 9.0f * eu * eF);
+      even = vadd(even, vfma(vset(9.0f * g * eF, r), eu, vmul(vset(-3.0f * g, r), uF)));
+      odd = vadd(odd, vset(3.0f * g * eF, r));
     }
-    h[i] = hp;
+    h[i] = vfma(keep, h[i], vadd(even, odd));
+    h[i + 1] = vfma(keep, h[i + 1], vsub(even, odd));
   }
 }
 
@@ -65,36 +161,55 @@ __device__ __forceinline__ void collide_store(float (&h)[19], typename Store<ST>
 }
 
 // Pull streaming (with halfway bounce-back at domain walls) of node (x, y, z),
-// c its linear index: the 19 incoming deviations h_i = f_i - w_i.
+// c its linear index: the 19 incoming deviations h_i = f_i - w_i.  At a face
+// the source index is selected (the far end of a periodic axis, or the node's
+// own opposite population at a wall) before one load per direction, so all 19
+// loads are in flight together: with a branch per direction they were waited
+// for one after another, and every warp that holds a row's end paid for it.
 template <int ST>
 __device__ __forceinline__ void pull_node(const typename Store<ST>::T* __restrict__ A, const LatticeGeom& g,
                                           const CollideParams& P, int x, int y, int z, long long c, float (&h)[19]) {
+  const int nxy = g.nx * g.ny;
+  // per axis: source offset and wall flag for e = +1 (source below) and e = -1
+  const bool lo[3] = {x == 0, y == 0, z == 0}, hi[3] = {x == g.nx - 1, y == g.ny - 1, z == g.nz - 1};
+  const int n[3] = {g.nx, g.ny, g.nz}, step[3] = {1, g.nx, nxy};
+  int om[3], op[3];
+  bool wm[3], wp[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    wm[a] = lo[a] && !g.periodic[a];
+    wp[a] = hi[a] && !g.periodic[a];
+    om[a] = lo[a] ? (n[a] - 1) * step[a] : -step[a];
+    op[a] = hi[a] ? -(n[a] - 1) * step[a] : step[a];
+  }
+#pragma unroll
+  for (int i = 0; i < 19; ++i) {
+    const int e[3] = {cx(i), cy(i), cz(i)};
+    const bool bx = e[0] == 1 ? wm[0] : (e[0] == -1 ? wp[0] : false);
+    const bool by = e[1] == 1 ? wm[1] : (e[1] == -1 ? wp[1] : false);
+    const bool bz = e[2] == 1 ? wm[2] : (e[2] == -1 ? wp[2] : false);
+    const bool wall = bx | by | bz;
+    int off = 0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) off += e[a] == 1 ? om[a] : (e[a] == -1 ? op[a] : 0);
+    const long long at = wall ? opp(i) * g.plane + c : i * g.plane + (c + off);
+    h[i] = Store<ST>::dev(A + at, i);  // w_opp = w_i
+    // halfway bounce-back: f_in,i(x) = f+_opp(i)(x) + 6 w_i rho0 e_i.u_wall; a
+    // corner crossing is attributed to x, then y, then z
+    if (i && wall)
+      h[i] += bx ? P.bb_wall[e[0] == 1 ? 0 : 1][i] : (by ? P.bb_wall[e[1] == 1 ? 2 : 3][i] : P.bb_wall[e[2] == 1 ? 4 : 5][i]);
+  }
+}
+
+// The same away from the faces: constant offsets.
+template <int ST>
+__device__ __forceinline__ void pull_interior(const typename Store<ST>::T* __restrict__ A, const LatticeGeom& g,
+                                              long long c, float (&h)[19]) {
   const long long nxy = (long long)g.nx * g.ny;
-  const bool interior = (x > 0) & (x < g.nx - 1) & (y > 0) & (y < g.ny - 1) & (z > 0) & (z < g.nz - 1);
-  if (interior) {
 #pragma unroll
-    for (int i = 0; i < 19; ++i) {
-      const long long off = cx(i) + (long long)g.nx * cy(i) + nxy * cz(i);
-      h[i] = Store<ST>::dev(A + i * g.plane + (c - off), i);
-    }
-  } else {
-#pragma unroll
-    for (int i = 0; i < 19; ++i) {
-      int sx = x - cx(i), sy = y - cy(i), sz = z - cz(i);
-      int face = -1;  // a corner crossing is attributed to x, then y, then z
-      if (sz < 0) { if (g.periodic[2]) sz += g.nz; else face = 4; }
-      else if (sz >= g.nz) { if (g.periodic[2]) sz -= g.nz; else face = 5; }
-      if (sy < 0) { if (g.periodic[1]) sy += g.ny; else face = 2; }
-      else if (sy >= g.ny) { if (g.periodic[1]) sy -= g.ny; else face = 3; }
-      if (sx < 0) { if (g.periodic[0]) sx += g.nx; else face = 0; }
-      else if (sx >= g.nx) { if (g.periodic[0]) sx -= g.nx; else face = 1; }
-      if (face < 0) {
-        h[i] = Store<ST>::dev(A + i * g.plane + (sx + (long long)g.nx * sy + nxy * sz), i);
-      } else {
-        // halfway bounce-back: f_in,i(x) = f+_opp(i)(x) + 6 w_i rho0 e_i.u_wall (w_opp = w_i)
-        h[i] = Store<ST>::dev(A + opp(i) * g.plane + c, opp(i)) + P.bb_wall[face][i];
-      }
-    }
+  for (int i = 0; i < 19; ++i) {
+    const long long off = cx(i) + (long long)g.nx * cy(i) + nxy * cz(i);
+    h[i] = Store<ST>::dev(A + i * g.plane + (c - off), i);
   }
 }
 
@@ -108,95 +223,53 @@ __device__ __forceinline__ void update_node(const typename Store<ST>::T* __restr
   collide_store<ST, FORCE>(h, B, g.plane, c, P);
 }
 
-// Every node of the lattice, ROWS consecutive rows (y) per thread: all pulls
-// of a thread are issued before its collisions, so that 16-bit storages keep
-// as many bytes in flight as FP32.  With particles this runs concurrently with
+// Every node of the lattice, a thread per node, the blocks over the linear node
+// index (x fastest): a warp's 32 nodes are one aligned stretch of every plane
+// whatever nx is, and no lane idles at a row's end.  A warp that holds no face
+// node takes the constant offsets, any other the selecting pull for all its
+// lanes, so no warp runs both.  With particles this runs concurrently with
 // the particle phases: boundary nodes are rewritten afterwards by k_boundary,
 // solid nodes hold unspecified values, and the nodes next to a node uncovered
 // this step (whose refilled populations this kernel may not have seen) are
 // recomputed by k_near.  Nodes anywhere else have no solid or uncovered
 // neighbour, so their update here is final.
-template <int ST, bool FORCE, int ROWS>
+//
+// Bound by HBM: FP32 alone, 256 x 256 x 512 in 0.798 ms = 6.39 TB/s (0.94 of a
+// copy), 512^3 in 3.06 ms = 6.67 TB/s (0.98), 141 x 83 x 119 in 38 us.  With
+// rows as blocks, a branch per direction at the faces and the collision formed
+// direction by direction these took 0.955 ms, 3.53 ms and 74 us.  Blocks of 64
+// threads measured best from 64^3 to 512^3 (32: up to 3 % more, 256: 4 %).
+template <int ST, bool FORCE>
 __global__ void __launch_bounds__(256) k_bulk(const typename Store<ST>::T* __restrict__ A,
                                               typename Store<ST>::T* __restrict__ B, LatticeGeom g,
-                                              CollideParams P) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y0 = blockIdx.y * ROWS, z = blockIdx.z;
-  if (x >= g.nx) return;
-  float h[ROWS][19];
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r)
-    if (y0 + r < g.ny) pull_node<ST>(A, g, P, x, y0 + r, z, x + (long long)g.nx * (y0 + r + (long long)g.ny * z), h[r]);
-#pragma unroll
-  for (int r = 0; r < ROWS; ++r)
-    if (y0 + r < g.ny) collide_store<ST, FORCE>(h[r], B, g.plane, x + (long long)g.nx * (y0 + r + (long long)g.ny * z), P);
+                                              CollideParams P, FastDiv by_nx, FastDiv by_ny, unsigned ncell) {
+  const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
+  if (c >= ncell) return;
+  const unsigned row = by_nx.div(c), zu = by_ny.div(row);
+  const int x = (int)(c - row * (unsigned)g.nx), y = (int)(row - zu * (unsigned)g.ny), z = (int)zu;
+  const bool interior = (x > 0) & (x < g.nx - 1) & (y > 0) & (y < g.ny - 1) & (z > 0) & (z < g.nz - 1);
+  float h[19];
+  if (__all_sync(__activemask(), interior)) pull_interior<ST>(A, g, c, h);
+  else pull_node<ST>(A, g, P, x, y, z, c, h);
+  collide_store<ST, FORCE>(h, B, g.plane, c, P);
 }
 
-template <int ST, bool FORCE, int ROWS>
+template <int ST, bool FORCE>
 static cudaError_t launch_bulk_t(const BulkLaunch& L, cudaStream_t s) {
   using T = typename Store<ST>::T;
-  const int bx = L.block_x;
-  dim3 grid((L.g.nx + bx - 1) / bx, (L.g.ny + ROWS - 1) / ROWS, L.g.nz);
-  k_bulk<ST, FORCE, ROWS><<<grid, bx, 0, s>>>(static_cast<const T*>(L.A), static_cast<T*>(L.B), L.g, L.p);
+  const unsigned n = (unsigned)((long long)L.g.nx * L.g.ny * L.g.nz), bx = (unsigned)L.block_x;
+  k_bulk<ST, FORCE><<<n / bx + (n % bx ? 1u : 0u), bx, 0, s>>>(static_cast<const T*>(L.A), static_cast<T*>(L.B), L.g,
+                                                               L.p, fast_div((unsigned)L.g.nx), fast_div((unsigned)L.g.ny), n);
   return cudaGetLastError();
 }
 
-// Every node, two x-adjacent nodes (x0, x0 + 1), x0 even, per thread: the
+// 16-bit storages, two x-adjacent nodes (x0, x0 + 1), x0 even, per thread: the
 // pulls of the 9 directions with e_x = 0 are one paired load each; for
 // e_x = +1 (-1) the pair is completed by the high (low) element of the
 // previous (next) lane's paired load, fetched by a shuffle (a scalar load at
-// the warp's edge).  Both collisions store paired.  Nodes on the lattice's
-// boundary rows and edge columns are pulled again by the general path.  The
-// same concurrency contract as k_bulk.  Requires nx even.
-template <int ST, bool FORCE>
-__global__ void __launch_bounds__(128) k_bulk_pairs(const typename Store<ST>::T* __restrict__ A,
-                                                    typename Store<ST>::T* __restrict__ B, LatticeGeom g,
-                                                    CollideParams P) {
-  using T = typename Store<ST>::T;
-  using PR = Pair<ST>;
-  const int lane = threadIdx.x & 31;
-  const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = blockIdx.y, z = blockIdx.z;
-  const bool active = x0 < g.nx;
-  const int xc = active ? x0 : g.nx - 2;  // idle lanes still take part in the shuffles
-  float h0[19], h1[19];
-#pragma unroll
-  for (int i = 0; i < 19; ++i) {
-    const int ys = min(max(y - cy(i), 0), g.ny - 1), zs = min(max(z - cz(i), 0), g.nz - 1);
-    const T* row = A + i * g.plane + ((long long)zs * g.ny + ys) * g.nx;
-    const typename PR::P v = PR::load(row + xc);
-    if (cx(i) == 0) {
-      h0[i] = PR::lo(v, i);
-      h1[i] = PR::hi(v, i);
-    } else if (cx(i) == 1) {  // node x0 pulls from x0 - 1
-      const typename PR::P u = PR::shfl_up(v);
-      float prev = PR::hi(u, i);
-      if (lane == 0) prev = xc > 0 ? Store<ST>::dev(row + xc - 1, i) : 0.f;
-      h0[i] = prev;
-      h1[i] = PR::lo(v, i);
-    } else {  // node x0 + 1 pulls from x0 + 2
-      const typename PR::P u = PR::shfl_down(v);
-      float next = PR::lo(u, i);
-      if (lane == 31) next = xc + 2 < g.nx ? Store<ST>::dev(row + xc + 2, i) : 0.f;
-      h0[i] = PR::hi(v, i);
-      h1[i] = next;
-    }
-  }
-  if (!active) return;
-  const long long c0 = x0 + (long long)g.nx * (y + (long long)g.ny * z);
-  const bool rows_interior = (y > 0) & (y < g.ny - 1) & (z > 0) & (z < g.nz - 1);
-  if (!rows_interior || x0 == 0) pull_node<ST>(A, g, P, x0, y, z, c0, h0);
-  if (!rows_interior || x0 + 1 == g.nx - 1) pull_node<ST>(A, g, P, x0 + 1, y, z, c0 + 1, h1);
-  collide_inplace<FORCE>(h0, P);
-  collide_inplace<FORCE>(h1, P);
-#pragma unroll
-  for (int i = 0; i < 19; ++i) PR::put(B + i * g.plane + c0, i, h0[i], h1[i]);
-}
-
-// 16-bit storages: the same paired scheme with both nodes' incoming and
-// outgoing values kept packed, one 32-bit register per direction for the two
-// nodes, so that a thread needs about as many registers as the scalar kernel
-// and a warp keeps twice the bytes in flight.
+// the warp's edge).  The values stay packed, one 32-bit register per direction
+// for the two nodes.  Nodes on the lattice's boundary rows and edge columns
+// are pulled again by the general path.  Requires nx even.
 template <int ST, bool FORCE, int MINB>
 __global__ void __launch_bounds__(128, MINB) k_bulk_pairs16(const typename Store<ST>::T* __restrict__ A,
                                                          typename Store<ST>::T* __restrict__ B, LatticeGeom g,
@@ -365,22 +438,17 @@ __global__ void __launch_bounds__(128, FORCE ? 3 : 5) k_bulk_quad16(const typena
 
 template <int ST, bool FORCE>
 static cudaError_t launch_bulk_pairs_t(const BulkLaunch& L, cudaStream_t s) {
-  using T = typename Store<ST>::T;
+  constexpr int S16 = ST == MI_STORE_F32 ? MI_STORE_F16_DEV : ST;
+  using T16 = typename Store<S16>::T;
   const int bx = L.block_x;
   const int npair = L.g.nx / 2;
   dim3 grid((npair + bx - 1) / bx, L.g.ny, L.g.nz);
-  if (ST == MI_STORE_F32)
-    k_bulk_pairs<ST, FORCE><<<grid, bx, 0, s>>>(static_cast<const T*>(L.A), static_cast<T*>(L.B), L.g, L.p);
-  else {
-    constexpr int S16 = ST == MI_STORE_F32 ? MI_STORE_F16_DEV : ST;
-    using T16 = typename Store<S16>::T;
-    if (L.pair_mode == 2)
-      k_bulk_pairs16<S16, FORCE, 6><<<grid, bx, 0, s>>>(reinterpret_cast<const T16*>(L.A), reinterpret_cast<T16*>(L.B),
-                                                        L.g, L.p);
-    else
-      k_bulk_pairs16<S16, FORCE, 8><<<grid, bx, 0, s>>>(reinterpret_cast<const T16*>(L.A), reinterpret_cast<T16*>(L.B),
-                                                        L.g, L.p);
-  }
+  if (L.pair_mode == 2)
+    k_bulk_pairs16<S16, FORCE, 6><<<grid, bx, 0, s>>>(reinterpret_cast<const T16*>(L.A), reinterpret_cast<T16*>(L.B),
+                                                      L.g, L.p);
+  else
+    k_bulk_pairs16<S16, FORCE, 8><<<grid, bx, 0, s>>>(reinterpret_cast<const T16*>(L.A), reinterpret_cast<T16*>(L.B),
+                                                      L.g, L.p);
   return cudaGetLastError();
 }
 
@@ -400,10 +468,9 @@ template <int ST>
 static cudaError_t launch_bulk_st(const BulkLaunch& L, cudaStream_t s) {
   if (ST != MI_STORE_F32 && L.pair_mode == 3 && L.g.nx % 4 == 0 && L.g.nx >= 4)
     return L.forcing ? launch_bulk_quad_t<ST, true>(L, s) : launch_bulk_quad_t<ST, false>(L, s);
-  if (L.pairs && L.pair_mode != 3 && L.g.nx % 2 == 0 && L.g.nx >= 2)
+  if (ST != MI_STORE_F32 && L.pairs && L.pair_mode != 3 && L.g.nx % 2 == 0 && L.g.nx >= 2)
     return L.forcing ? launch_bulk_pairs_t<ST, true>(L, s) : launch_bulk_pairs_t<ST, false>(L, s);
-  if (L.rows == 2) return L.forcing ? launch_bulk_t<ST, true, 2>(L, s) : launch_bulk_t<ST, false, 2>(L, s);
-  return L.forcing ? launch_bulk_t<ST, true, 1>(L, s) : launch_bulk_t<ST, false, 1>(L, s);
+  return L.forcing ? launch_bulk_t<ST, true>(L, s) : launch_bulk_t<ST, false>(L, s);
 }
 
 cudaError_t launch_bulk(const BulkLaunch& L, cudaStream_t s) {

@@ -1018,7 +1018,7 @@ def run_mine(args):
     used = tuning if tuning else sim.get_tuning()
     quad = storage != 0 and used.get("bulk_pairs") == 3 and nx % 4 == 0
     traffic = BULK_TRAFFIC.get((storage, quad)) if (nx, ny, nz) == (256, 256, 512) else None
-    bulk_name = ("k_bulk_quad16 (D3Q19 stream-collide, four nodes per thread)" if quad
+    bulk_name = ("k_bulk16 (D3Q19 stream-collide, four nodes per thread)" if quad
                  else "k_bulk (D3Q19 stream-collide of every node)")
 
     # end to end through the public API: per step, upload of the particle

@@ -454,11 +454,10 @@ mi_status mi_delbm_set_momentum_rules(mi_delbm *h, int flags);
 /* Set the launch shapes directly (what mi_delbm_autotune chooses): bulk
  * kernel threads per block (32..256, a multiple of 32; at most 128 with
  * pairs), rows per thread (1 or 2: accepted, both run one row), paired nodes
- * (0: no; 1 or 2: two x-adjacent nodes per thread with paired accesses and a
- * 64- or 80-register budget; 3: four x-adjacent nodes per thread with 64-bit
- * accesses; used for 16-bit storages only, 1 and 2 with nx even and 3 with nx
- * a multiple of 4, else the one-node kernel), list-kernel blocks per SM
- * (1..64).  Results do not depend on them. */
+ * (0: no; 1 or 2: two x-adjacent nodes per thread with 32-bit accesses; 3:
+ * four x-adjacent nodes per thread with 64-bit accesses; used for 16-bit
+ * storages only, 1 and 2 with nx even and 3 with nx a multiple of 4, else the
+ * one-node kernel), list-kernel blocks per SM (1..64).  Results do not depend on them. */
 mi_status mi_delbm_set_tuning(mi_delbm *h, int bulk_block_x, int bulk_rows, int bulk_pairs, int list_blocks_per_sm);
 
 /* The launch shapes in use (any pointer may be NULL). */

@@ -376,6 +376,9 @@ mi_status mi_delbm::phase_contact(cudaStream_t st) {
   return launch_phase(this, st, MI_PHASE_CONTACT, "k_contacts", [&] { return launch_contacts(L, st); });
 }
 
+// x-adjacent nodes per thread of a tuning's bulk_pairs (0: one, 1 and 2: two, 3: four)
+static int bulk_nodes(int pairs) { return pairs == 3 ? 4 : (pairs ? 2 : 1); }
+
 mi_status mi_delbm::phase_bulk() {
   BulkLaunch L;
   L.A = pop[cur];
@@ -385,8 +388,7 @@ mi_status mi_delbm::phase_bulk() {
   L.storage = cfg.storage;
   L.forcing = forcing();
   L.block_x = tune.bulk_block_x;
-  L.pairs = tune.bulk_pairs != 0;
-  L.pair_mode = tune.bulk_pairs;
+  L.nodes = bulk_nodes(tune.bulk_pairs);
   return launch_phase(this, stream, MI_PHASE_BULK, "k_bulk", [&] { return launch_bulk(L, stream); });
 }
 
@@ -906,10 +908,14 @@ mi_status mi_delbm_create(const mi_delbm_config* cfg, mi_delbm** out) {
   h->tune.bulk_block_x = 64;  // the one-node kernel's best from 64^3 to 512^3
   h->tune.bulk_rows = 1;
   h->tune.bulk_pairs = 0;
-  if (cfg->storage != MI_STORE_F32 && cfg->nx % 4 == 0) {
-    // 16-bit storages: four nodes per thread with 64-bit accesses
-    h->tune.bulk_pairs = 3;
-    h->tune.bulk_block_x = cfg->nx >= 256 ? 64 : 32;
+  if (cfg->storage != MI_STORE_F32) {
+    // 16-bit storages: four nodes per thread (64-bit accesses) when nx allows
+    // and the lattice has enough nodes to fill the chip with a quarter of the
+    // threads (64^3: 13.8 us against 8.6 with two nodes, 128^3: 34.5 against
+    // 33.1, 160^3: equal, 192^3: 94.7 against 98.4, 192 x 192 x 768: 346
+    // against 370), else two
+    if (cfg->nx % 4 == 0 && ncell >= (1 << 22)) h->tune.bulk_pairs = 3;
+    else if (cfg->nx % 2 == 0) h->tune.bulk_pairs = 1;
   }
   {
     int sms = 0;
@@ -1368,17 +1374,14 @@ extern "C" mi_status mi_delbm_autotune(mi_delbm* h, const char* cache_path, int*
     L.storage = h->cfg.storage;
     L.forcing = h->forcing();
     float best = 1e30f;
-    // variants: one node, paired nodes (16-bit storages, two register budgets),
-    // four nodes per thread (16-bit storages)
-    for (int pairs = 0; pairs < 4; ++pairs) {
+    // variants: one node, and for 16-bit storages two and four nodes per thread
+    for (int pairs : {0, 1, 3}) {
       if (pairs && (h->cfg.storage == MI_STORE_F32 || (h->cfg.nx % 2) != 0)) continue;
       if (pairs == 3 && (h->cfg.nx % 4) != 0) continue;
       for (int bx : {32, 64, 128, 256}) {
-        const int span = pairs == 3 ? 4 * bx : 2 * bx;
-        if (pairs && ((bx > 32 && span / 2 >= h->cfg.nx) || bx > 128)) break;
+        if (pairs && bx > 128) break;
         L.block_x = bx;
-        L.pairs = pairs != 0;
-        L.pair_mode = pairs;
+        L.nodes = bulk_nodes(pairs);
         const float ms = h->time_launches(5, [&] { return launch_bulk(L, h->stream); });
         if (ms > 0.f && ms < best) {
           best = ms;

@@ -263,90 +263,27 @@ static cudaError_t launch_bulk_t(const BulkLaunch& L, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// 16-bit storages, two x-adjacent nodes (x0, x0 + 1), x0 even, per thread: the
-// pulls of the 9 directions with e_x = 0 are one paired load each; for
-// e_x = +1 (-1) the pair is completed by the high (low) element of the
-// previous (next) lane's paired load, fetched by a shuffle (a scalar load at
-// the warp's edge).  The values stay packed, one 32-bit register per direction
-// for the two nodes.  Nodes on the lattice's boundary rows and edge columns
-// are pulled again by the general path.  Requires nx even.
-template <int ST, bool FORCE, int MINB>
-__global__ void __launch_bounds__(128, MINB) k_bulk_pairs16(const typename Store<ST>::T* __restrict__ A,
-                                                         typename Store<ST>::T* __restrict__ B, LatticeGeom g,
-                                                         CollideParams P) {
-  using T = typename Store<ST>::T;
-  const int lane = threadIdx.x & 31;
-  const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = blockIdx.y, z = blockIdx.z;
-  const bool active = x0 < g.nx;
-  const int xc = active ? x0 : g.nx - 2;
-  unsigned in[19];  // low half: node x0, high half: node x0 + 1
-#pragma unroll
-  for (int i = 0; i < 19; ++i) {
-    const int ys = min(max(y - cy(i), 0), g.ny - 1), zs = min(max(z - cz(i), 0), g.nz - 1);
-    const unsigned short* row =
-        reinterpret_cast<const unsigned short*>(A + i * g.plane + ((long long)zs * g.ny + ys) * g.nx);
-    const unsigned v = __ldg(reinterpret_cast<const unsigned*>(row + xc));
-    if (cx(i) == 0) {
-      in[i] = v;
-    } else if (cx(i) == 1) {
-      const unsigned u = __shfl_up_sync(0xffffffffu, v, 1);
-      unsigned prev = u >> 16;
-      if (lane == 0) prev = xc > 0 ? (unsigned)__ldg(row + xc - 1) : 0u;
-      in[i] = prev | (v << 16);
-    } else {
-      const unsigned u = __shfl_down_sync(0xffffffffu, v, 1);
-      unsigned next = u & 0xFFFFu;
-      if (lane == 31) next = xc + 2 < g.nx ? (unsigned)__ldg(row + xc + 2) : 0u;
-      in[i] = (v >> 16) | (next << 16);
-    }
-  }
-  if (!active) return;
-  const long long c0 = x0 + (long long)g.nx * (y + (long long)g.ny * z);
-  const bool rows_interior = (y > 0) & (y < g.ny - 1) & (z > 0) & (z < g.nz - 1);
-  unsigned out[19];
-  {
-    float h[19];
-    if (!rows_interior || x0 == 0) {
-      pull_node<ST>(A, g, P, x0, y, z, c0, h);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 19; ++i) h[i] = dev16<ST>((unsigned short)(in[i] & 0xFFFFu));
-    }
-    collide_inplace<FORCE>(h, P);
-#pragma unroll
-    for (int i = 0; i < 19; ++i) out[i] = pack16<ST>(h[i]);
-  }
-  {
-    float h[19];
-    if (!rows_interior || x0 + 1 == g.nx - 1) {
-      pull_node<ST>(A, g, P, x0 + 1, y, z, c0 + 1, h);
-    } else {
-#pragma unroll
-      for (int i = 0; i < 19; ++i) h[i] = dev16<ST>((unsigned short)(in[i] >> 16));
-    }
-    collide_inplace<FORCE>(h, P);
-#pragma unroll
-    for (int i = 0; i < 19; ++i) out[i] |= (unsigned)pack16<ST>(h[i]) << 16;
-  }
-#pragma unroll
-  for (int i = 0; i < 19; ++i) __stcs(reinterpret_cast<unsigned*>(B + i * g.plane + c0), out[i]);
-}
-
-// 16-bit storages: four x-adjacent nodes (x0 .. x0 + 3, x0 a multiple of 4)
-// per thread.  Each pull is one aligned 64-bit load per direction when e_x = 0;
-// for e_x = +1 (-1) the four shifted elements x0 - 1 .. x0 + 2 (x0 + 1 ..
-// x0 + 4) are the quad's own aligned 64-bit word plus the aligned 32-bit
-// word beside it, joined by two byte permutes.  The 16-bit values stay packed
-// in registers until each node's collision, and every direction is stored as
-// one 64-bit streaming store: a 16-bit storage moves half the bytes of FP32
-// per instruction, and the wider accesses keep the instruction count per
-// byte near that of the FP32 kernel.  The quads at the x faces stay on this
-// path (no warp mixes paths): the word beside them comes from the other end
-// of the row when x is periodic, else the face node's pulled value is
-// replaced after unpacking by its halfway bounce-back.  Rows on the y and z
-// faces (whole warps) take the general per-node path.  The same concurrency
-// contract as k_bulk.  Requires nx % 4 == 0.
+// 16-bit storages: W = 2 or 4 x-adjacent nodes per thread (x0 .. x0 + W - 1, x0
+// a multiple of W), the blocks over the linear groups of W nodes.  A direction
+// with e_x = 0 is one aligned 32- or 64-bit load; for e_x = +1 (-1) the shifted
+// elements are the thread's own aligned word plus the one element beside it,
+// joined by shifts and a byte permute.  The values stay packed two to a
+// register until the collision, which takes two nodes at a time in packed FP32
+// pairs, and every direction is one aligned streaming store.  Groups at the x
+// faces stay on this path (no warp mixes paths): the element beside them comes
+// from the other end of the row when x is periodic, else the face node's
+// pulled value is replaced after unpacking by its halfway bounce-back.  Rows
+// on the y and z faces take the general per-node path.  The same concurrency
+// contract as k_bulk.  Requires nx % W == 0.
+//
+// Bound by HBM: 256 x 256 x 512 FP16 in 0.394 ms = 6.48 TB/s (0.95 of a copy),
+// 512^3 in 1.59 ms, four nodes per thread.  With unpacked FP32 arithmetic, rows
+// as blocks and branches per direction at the faces these took 0.522 and 1.99
+// ms: that kernel waited for instruction issue.  Two nodes per thread reach 0.449
+// ms (more instructions a byte) but, with twice the threads, win on small
+// lattices: 64^3 in 8 against 12 us; the one-node kernel takes 0.598 ms.  Five
+// blocks of 128 threads per SM (96 registers, a few spilled) measured 7 % faster
+// than four (128 registers).
 template <int ST> __device__ __forceinline__ float2 unpack2(unsigned w);
 template <> __device__ __forceinline__ float2 unpack2<MI_STORE_F16_DEV>(unsigned w) {
   return __half22float2(*reinterpret_cast<const __half2*>(&w));
@@ -364,118 +301,117 @@ template <> __device__ __forceinline__ unsigned pack2<MI_STORE_BF16_DEV>(float a
   return *reinterpret_cast<const unsigned*>(&v);
 }
 
-template <int ST, bool FORCE>
-__global__ void __launch_bounds__(128, FORCE ? 3 : 5) k_bulk_quad16(const typename Store<ST>::T* __restrict__ A,
-                                                     typename Store<ST>::T* __restrict__ B, LatticeGeom g,
-                                                     CollideParams P) {
-  const int x0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x);
-  const int y = blockIdx.y, z = blockIdx.z;
-  if (x0 >= g.nx) return;
-  const long long c0 = x0 + (long long)g.nx * (y + (long long)g.ny * z);
+// W 16-bit elements in W / 2 words, one aligned access
+template <int W> struct Words;
+template <> struct Words<2> {
+  unsigned w[1];
+  __device__ __forceinline__ void load(const unsigned short* p) { w[0] = __ldg(reinterpret_cast<const unsigned*>(p)); }
+  __device__ __forceinline__ void store(unsigned short* p) const { __stcs(reinterpret_cast<unsigned*>(p), w[0]); }
+};
+template <> struct Words<4> {
+  unsigned w[2];
+  __device__ __forceinline__ void load(const unsigned short* p) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2*>(p));
+    w[0] = v.x;
+    w[1] = v.y;
+  }
+  __device__ __forceinline__ void store(unsigned short* p) const {
+    __stcs(reinterpret_cast<uint2*>(p), make_uint2(w[0], w[1]));
+  }
+};
+
+template <int ST, bool FORCE, int W>
+__global__ void __launch_bounds__(128, W == 4 ? (FORCE ? 4 : 5) : (FORCE ? 6 : 7))
+    k_bulk16(const typename Store<ST>::T* __restrict__ A, typename Store<ST>::T* __restrict__ B, LatticeGeom g,
+             CollideParams P, FastDiv by_groups, FastDiv by_ny, unsigned ngroups) {
+  const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= ngroups) return;
+  const unsigned per_row = (unsigned)g.nx / W, row = by_groups.div(t), zu = by_ny.div(row);
+  const int x0 = W * (int)(t - row * per_row), y = (int)(row - zu * (unsigned)g.ny), z = (int)zu;
+  const long long c0 = (long long)W * t;
   if (!((y > 0) & (y < g.ny - 1) & (z > 0) & (z < g.nz - 1))) {
 #pragma unroll 1
-    for (int k = 0; k < 4; ++k) update_node<ST, FORCE>(A, B, g, P, x0 + k, y, z, c0 + k);
+    for (int k = 0; k < W; ++k) update_node<ST, FORCE>(A, B, g, P, x0 + k, y, z, c0 + k);
     return;
   }
-  const bool lo_edge = x0 == 0, hi_edge = x0 == g.nx - 4, xper = g.periodic[0] != 0;
+  const bool lo_edge = x0 == 0, hi_edge = x0 == g.nx - W, xper = g.periodic[0] != 0;
   const unsigned short* Au = reinterpret_cast<const unsigned short*>(A);
   const long long nxy = (long long)g.nx * g.ny;
-  uint2 in[19];
+  // the element before x0 and the one after x0 + W - 1 (at a wall any element
+  // of the row: replaced below)
+  const int before_at = lo_edge ? (xper ? g.nx - 1 : 0) : -1, after_at = hi_edge ? (xper ? W - g.nx : 0) : W;
+  Words<W> in[19];
 #pragma unroll
   for (int i = 0; i < 19; ++i) {
     // aligned position of node x0 in the source row of direction i
-    const unsigned short* row = Au + i * g.plane + (c0 - ((long long)g.nx * cy(i) + nxy * cz(i)));
-    const uint2 w = __ldg(reinterpret_cast<const uint2*>(row));
-    if (cx(i) == 0) {
-      in[i] = w;
-    } else if (cx(i) == 1) {  // elements x0 - 1 .. x0 + 2
-      unsigned before;        // its high half: element x0 - 1
-      if (!lo_edge) before = __ldg(reinterpret_cast<const unsigned*>(row - 2));
-      else before = xper ? (unsigned)__ldg(row + g.nx - 1) << 16 : 0u;  // wall: replaced below
-      in[i] = make_uint2(__byte_perm(before, w.x, 0x5432), __byte_perm(w.x, w.y, 0x5432));
-    } else {                  // elements x0 + 1 .. x0 + 4
-      unsigned after;         // its low half: element x0 + 4
-      if (!hi_edge) after = __ldg(reinterpret_cast<const unsigned*>(row + 4));
-      else after = xper ? (unsigned)__ldg(row - x0) : 0u;  // wall: replaced below
-      in[i] = make_uint2(__byte_perm(w.x, w.y, 0x5432), __byte_perm(w.y, after, 0x5432));
+    const unsigned short* src = Au + i * g.plane + (c0 - ((long long)g.nx * cy(i) + nxy * cz(i)));
+    in[i].load(src);
+    if (cx(i) == 1) {  // elements x0 - 1 .. x0 + W - 2
+      const unsigned before = __ldg(src + before_at), first = in[i].w[0];
+      if (W == 4) in[i].w[W / 2 - 1] = __byte_perm(first, in[i].w[W / 2 - 1], 0x5432);
+      in[i].w[0] = before | (first << 16);
+    } else if (cx(i) == -1) {  // elements x0 + 1 .. x0 + W
+      const unsigned after = __ldg(src + after_at);
+      if (W == 4) in[i].w[0] = __byte_perm(in[i].w[0], in[i].w[W / 2 - 1], 0x5432);
+      in[i].w[W / 2 - 1] = (in[i].w[W / 2 - 1] >> 16) | (after << 16);
     }
   }
-  uint2 out[19];
 #pragma unroll
-  for (int half = 0; half < 2; ++half) {
-    float h0[19], h1[19];
+  for (int k = 0; k < W / 2; ++k) {
+    float2 v[19];
 #pragma unroll
-    for (int i = 0; i < 19; ++i) {
-      const float2 v = unpack2<ST>(half ? in[i].y : in[i].x);
-      h0[i] = v.x;
-      h1[i] = v.y;
-    }
+    for (int i = 0; i < 19; ++i) v[i] = unpack2<ST>(in[i].w[k]);
     if (!xper) {
       // halfway bounce-back at the x faces: f_in,i(x) = f+_opp(i)(x) + 6 w_i rho0 e_i.u_wall
-      if (half == 0 && lo_edge) {
+      if (k == 0 && lo_edge) {
 #pragma unroll
         for (int i = 0; i < 19; ++i)
-          if (cx(i) == 1) h0[i] = dev16<ST>(__ldg(Au + opp(i) * g.plane + c0)) + P.bb_wall[0][i];
+          if (cx(i) == 1) v[i].x = dev16<ST>(__ldg(Au + opp(i) * g.plane + c0)) + P.bb_wall[0][i];
       }
-      if (half == 1 && hi_edge) {
+      if (k == W / 2 - 1 && hi_edge) {
 #pragma unroll
         for (int i = 0; i < 19; ++i)
-          if (cx(i) == -1) h1[i] = dev16<ST>(__ldg(Au + opp(i) * g.plane + c0 + 3)) + P.bb_wall[1][i];
+          if (cx(i) == -1) v[i].y = dev16<ST>(__ldg(Au + opp(i) * g.plane + c0 + W - 1)) + P.bb_wall[1][i];
       }
     }
-    collide_inplace<FORCE>(h0, P);
-    collide_inplace<FORCE>(h1, P);
+    F32x2 h[19];
+#pragma unroll
+    for (int i = 0; i < 19; ++i) h[i] = pack(v[i].x, v[i].y);
+    collide_inplace<FORCE>(h, P);
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
-      const unsigned wv = pack2<ST>(h0[i], h1[i]);
-      if (half) out[i].y = wv; else out[i].x = wv;
+      const float2 r = unpack(h[i]);
+      in[i].w[k] = pack2<ST>(r.x, r.y);
     }
   }
   unsigned short* Bu = reinterpret_cast<unsigned short*>(B);
 #pragma unroll
-  for (int i = 0; i < 19; ++i) __stcs(reinterpret_cast<uint2*>(Bu + i * g.plane + c0), out[i]);
+  for (int i = 0; i < 19; ++i) in[i].store(Bu + i * g.plane + c0);
 }
 
-template <int ST, bool FORCE>
-static cudaError_t launch_bulk_pairs_t(const BulkLaunch& L, cudaStream_t s) {
+template <int ST, bool FORCE, int W>
+static cudaError_t launch_bulk16_t(const BulkLaunch& L, cudaStream_t s) {
   constexpr int S16 = ST == MI_STORE_F32 ? MI_STORE_F16_DEV : ST;
   using T16 = typename Store<S16>::T;
-  const int bx = L.block_x;
-  const int npair = L.g.nx / 2;
-  dim3 grid((npair + bx - 1) / bx, L.g.ny, L.g.nz);
-  if (L.pair_mode == 2)
-    k_bulk_pairs16<S16, FORCE, 6><<<grid, bx, 0, s>>>(reinterpret_cast<const T16*>(L.A), reinterpret_cast<T16*>(L.B),
-                                                      L.g, L.p);
-  else
-    k_bulk_pairs16<S16, FORCE, 8><<<grid, bx, 0, s>>>(reinterpret_cast<const T16*>(L.A), reinterpret_cast<T16*>(L.B),
-                                                      L.g, L.p);
-  return cudaGetLastError();
-}
-
-template <int ST, bool FORCE>
-static cudaError_t launch_bulk_quad_t(const BulkLaunch& L, cudaStream_t s) {
-  constexpr int S16 = ST == MI_STORE_F32 ? MI_STORE_F16_DEV : ST;
-  using T16 = typename Store<S16>::T;
-  const int bx = L.block_x;
-  const int nq = L.g.nx / 4;
-  dim3 grid((nq + bx - 1) / bx, L.g.ny, L.g.nz);
-  k_bulk_quad16<S16, FORCE><<<grid, bx, 0, s>>>(reinterpret_cast<const T16*>(L.A), reinterpret_cast<T16*>(L.B), L.g,
-                                                L.p);
+  const unsigned n = (unsigned)((long long)L.g.nx / W * L.g.ny * L.g.nz), bx = (unsigned)L.block_x;
+  k_bulk16<S16, FORCE, W><<<n / bx + (n % bx ? 1u : 0u), bx, 0, s>>>(
+      reinterpret_cast<const T16*>(L.A), reinterpret_cast<T16*>(L.B), L.g, L.p, fast_div((unsigned)L.g.nx / W),
+      fast_div((unsigned)L.g.ny), n);
   return cudaGetLastError();
 }
 
 template <int ST>
 static cudaError_t launch_bulk_st(const BulkLaunch& L, cudaStream_t s) {
-  if (ST != MI_STORE_F32 && L.pair_mode == 3 && L.g.nx % 4 == 0 && L.g.nx >= 4)
-    return L.forcing ? launch_bulk_quad_t<ST, true>(L, s) : launch_bulk_quad_t<ST, false>(L, s);
-  if (ST != MI_STORE_F32 && L.pairs && L.pair_mode != 3 && L.g.nx % 2 == 0 && L.g.nx >= 2)
-    return L.forcing ? launch_bulk_pairs_t<ST, true>(L, s) : launch_bulk_pairs_t<ST, false>(L, s);
+  if (ST != MI_STORE_F32 && L.nodes == 4 && L.g.nx % 4 == 0)
+    return L.forcing ? launch_bulk16_t<ST, true, 4>(L, s) : launch_bulk16_t<ST, false, 4>(L, s);
+  if (ST != MI_STORE_F32 && L.nodes == 2 && L.g.nx % 2 == 0)
+    return L.forcing ? launch_bulk16_t<ST, true, 2>(L, s) : launch_bulk16_t<ST, false, 2>(L, s);
   return L.forcing ? launch_bulk_t<ST, true>(L, s) : launch_bulk_t<ST, false>(L, s);
 }
 
 cudaError_t launch_bulk(const BulkLaunch& L, cudaStream_t s) {
   if (L.block_x <= 0 || L.block_x > 256 || (L.block_x % 32) != 0) return cudaErrorInvalidValue;
-  if (L.pairs && L.block_x > 128) return cudaErrorInvalidValue;
+  if (L.nodes > 1 && L.block_x > 128) return cudaErrorInvalidValue;
   switch (L.storage) {
     case MI_STORE_F32: return launch_bulk_st<MI_STORE_F32>(L, s);
     case MI_STORE_F16_DEV: return launch_bulk_st<MI_STORE_F16_DEV>(L, s);

@@ -129,8 +129,7 @@ struct BulkLaunch {
   int storage;
   bool forcing;
   int block_x;         // threads per block
-  bool pairs = false;  // 16-bit storages: two x-adjacent nodes per thread with paired accesses (nx even)
-  int pair_mode = 1;   // 16-bit paired kernel occupancy: 1 = up to 64 registers, 2 = up to 80
+  int nodes = 1;       // 16-bit storages: x-adjacent nodes per thread, 1, 2 (nx even) or 4 (nx a multiple of 4)
 };
 cudaError_t launch_bulk(const BulkLaunch& L, cudaStream_t s);
 

@@ -809,7 +809,7 @@ def shape_bench(B, scenes, n=300, h=0.25, seed=0):
                              "sample": "numpy oracle: the first particle at twice the spacing, time x 8"}}
 
 
-C4_KERNELS = ("k_prologue", "k_clear", "k_flag", "k_classify", "k_links_q", "k_refill", "k_bulk", "k_near",
+C4_KERNELS = ("k_prologue", "k_flag", "k_classify", "k_links_q", "k_refill", "k_bulk", "k_near",
               "k_links_ibb", "k_boundary", "k_dem_prologue", "k_broad_phase", "k_contacts", "k_integrate")
 # stated accuracy of each storage on the precision tank: the bounds that
 # tests/test_gpu_precision.py asserts on the 128^3 sub-run of that tank

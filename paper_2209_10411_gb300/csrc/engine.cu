@@ -181,7 +181,6 @@ mi_status mi_delbm::phase_flag(cudaStream_t st) {
   ParticleLaunch L = particle_launch();
   mi_status s;
   if ((s = launch_phase(this, st, MI_PHASE_FLAG, "k_prologue", [&] { return launch_prologue(L, st); })) != MI_OK) return s;
-  if ((s = launch_phase(this, st, MI_PHASE_FLAG, "k_clear", [&] { return launch_clear(L, st); })) != MI_OK) return s;
   if ((s = launch_phase(this, st, MI_PHASE_FLAG, "k_flag", [&] { return launch_flag(L, st); })) != MI_OK) return s;
   return launch_phase(this, st, MI_PHASE_FLAG, "k_classify", [&] { return launch_classify(L, st); });
 }
@@ -1710,19 +1709,24 @@ mi_status mi_delbm_add_particle(mi_delbm* h, int n, const double* centers, const
   if (sbc > 0x3FFFFFFFull) sbc = 0x3FFFFFFFull;
   st = h->ensure_list_capacity((unsigned)sbc, (unsigned)std::min<unsigned long long>(6ull * sbc, 0xFFFFFFF0ull), (unsigned)sbc);
   if (st != MI_OK) return st;
-  // box-kernel blocks per particle: about 8192 box nodes per flag block, and
-  // 8 warps of about 64 rows each per classification block (the classified
-  // region, old and new box widened by 2, has fewer than (ext + 8)^2 rows).
-  // Few long-lived blocks: these kernels run beside the bulk kernel, and the
-  // fewer SM slots they hold at a time, the less they slow it (eight times
-  // more blocks made the settling-tank step 2.4 % slower; sixteen times
-  // fewer made the particle chain outlast the 16-bit bulk kernel)
+  // box-kernel blocks per particle.  These kernels run beside the bulk kernel
+  // and are the head of the particle chain, so their grids follow the time the
+  // bulk kernel takes (its bytes at about 6400 GB/s): with a large lattice few
+  // long-lived blocks (32 box nodes per flag thread, 64 rows per
+  // classification warp; the classified region, old and new box widened by 2,
+  // has fewer than (ext + 8)^2 rows), which hold fewer SM slots at a time and
+  // slow the bulk kernel least; with a small one as many as there is work, since
+  // the step then waits for the chain (64^3: 28 rows in turn took a warp 55 us,
+  // the bulk kernel 11)
+  const double bulk_us = (double)h->ncell * 38.0 * (double)h->esize / 6.4e6;
+  const int spread = (int)std::min(32.0, std::max(1.0, bulk_us / 25.0));
+  const long long flag_nodes = 256ll * spread, cls_rows = 8ll * 2 * spread;
   const int npart = h->n_particles, stride = h->cfg.max_particles + 1;
   std::vector<int> boff(2 * (size_t)stride, 0);
   for (int q = 0; q < npart; ++q) {
     const int* e = h->hp[q].ext;
-    const long long fb = ((long long)e[0] * e[1] * e[2] + 8191) / 8192;
-    const long long cb = ((long long)(e[1] + 8) * (e[2] + 8) + 511) / 512;
+    const long long fb = ((long long)e[0] * e[1] * e[2] + flag_nodes - 1) / flag_nodes;
+    const long long cb = ((long long)(e[1] + 8) * (e[2] + 8) + cls_rows - 1) / cls_rows;
     boff[q + 1] = boff[q] + (int)std::min<long long>(std::max<long long>(fb, 1), 8192);
     boff[stride + q + 1] = boff[stride + q] + (int)std::min<long long>(std::max<long long>(cb, 1), 4096);
   }

@@ -426,7 +426,9 @@ cudaError_t launch_bulk(const BulkLaunch& L, cudaStream_t s) {
 //   f+_i(x_new) = f+_opp(i)(x_new + e_i) + 6 w_i rho0 (e_i . u_new)
 // when x_new + e_i is a fluid node that was also fluid at the previous step,
 // else f_eq,i(rho0, u_new); u_new is the rigid velocity at x_new of the
-// particle that covered it.  One thread per uncovered node.  With the
+// particle that covered it.  One warp per uncovered node, a lane per direction:
+// few nodes are uncovered in a step, and one thread per node waited for three
+// dependent loads in each of its 19 directions (19 us for one node).  With the
 // cover/uncover rule the same launch also moves node momenta: an uncovered
 // node's refilled momentum is taken from its particle, a covered node's
 // post-collision momentum is given to the particle that covers it.
@@ -434,18 +436,19 @@ cudaError_t launch_bulk(const BulkLaunch& L, cudaStream_t s) {
 namespace {
 __device__ __forceinline__ bool nbr_wrap(int x, int y, int z, int dx, int dy, int dz, const LatticeGeom& g,
                                          long long& out) {
+  // |dx|, |dy|, |dz| <= 1: one wrap at most
   int a = x + dx, b = y + dy, c = z + dz;
   if (a < 0 || a >= g.nx) {
     if (!g.periodic[0]) return false;
-    a = (a + g.nx) % g.nx;
+    a += a < 0 ? g.nx : -g.nx;
   }
   if (b < 0 || b >= g.ny) {
     if (!g.periodic[1]) return false;
-    b = (b + g.ny) % g.ny;
+    b += b < 0 ? g.ny : -g.ny;
   }
   if (c < 0 || c >= g.nz) {
     if (!g.periodic[2]) return false;
-    c = (c + g.nz) % g.nz;
+    c += c < 0 ? g.nz : -g.nz;
   }
   out = a + (long long)g.nx * (b + (long long)g.ny * c);
   return true;
@@ -487,18 +490,28 @@ __device__ __forceinline__ void moments_at(const typename Store<ST>::T* __restri
 }  // namespace
 
 namespace {
-// Cover/uncover rule: a node's population momentum J (FP32) and its torque
-// about the particle's position, sign * (J, (x - X_p) x J), added to the
-// particle's fixed-point hydrodynamic sums.
+// weight and opposite of a direction given at run time (lex, ley, lez: the
+// shared header's packed direction tables)
+__device__ __forceinline__ float lw(int j) { return j == 0 ? (1.0f / 3.0f) : (j <= 6 ? (1.0f / 18.0f) : (1.0f / 36.0f)); }
+__device__ __forceinline__ int lopp(int j) { return j == 0 ? 0 : ((j & 1) ? j + 1 : j - 1); }
+
+// Cover/uncover rule: a node's population momentum J = sum e_i h_i (FP32, lane i
+// holds h_i) and its torque about the particle's position, sign * (J, (x - X_p) x J),
+// added to the particle's fixed-point hydrodynamic sums.
 __device__ __forceinline__ void add_node_momentum(long long* facc, const DevParticle* Ps, uint32_t p, int x, int y,
-                                                  int z, const float J[3], float sign) {
+                                                  int z, float h, int ex, int ey, int ez, float sign, unsigned lane) {
+  float J[3] = {ex * h, ey * h, ez * h};
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    for (int a = 0; a < 3; ++a) J[a] += __shfl_xor_sync(0xffffffffu, J[a], o);
   const DevParticle& P = Ps[p];
   const float r0 = (float)(x - P.pos[0]), r1 = (float)(y - P.pos[1]), r2 = (float)(z - P.pos[2]);
   const float v[6] = {J[0], J[1], J[2], r1 * J[2] - r2 * J[1], r2 * J[0] - r0 * J[2], r0 * J[1] - r1 * J[0]};
-  for (int k = 0; k < 6; ++k) {
-    const long long iv = __float2ll_rn(sign * v[k] * 1099511627776.0f);
-    atomicAdd(reinterpret_cast<unsigned long long*>(facc + 6 * (size_t)p + k), (unsigned long long)iv);
-  }
+#pragma unroll
+  for (unsigned k = 0; k < 6; ++k)
+    if (lane == k)
+      atomicAdd(reinterpret_cast<unsigned long long*>(facc + 6 * (size_t)p + k),
+                (unsigned long long)__float2ll_rn(sign * v[k] * 1099511627776.0f));
 }
 }  // namespace
 
@@ -509,7 +522,12 @@ __global__ void __launch_bounds__(128) k_refill(BoundaryLaunch L) {
   const LatticeGeom& g = L.pl.g;
   const unsigned nn = min(L.pl.ctr->n_new, L.pl.cap_new);
   const float rho0 = L.p.rho0;
-  for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < nn; k += gridDim.x * blockDim.x) {
+  const unsigned lane = threadIdx.x & 31u, wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+                 nw = (gridDim.x * blockDim.x) >> 5;
+  const int i = lane < 19u ? (int)lane : 0;
+  const int ex = lex(i), ey = ley(i), ez = lez(i), oi = lopp(i);
+  const float wi = lw(i);
+  for (unsigned k = wid; k < nn; k += nw) {
     const long long c = L.pl.new_cell[k];
     int x, y, z;
     coords(c, g, x, y, z);
@@ -518,51 +536,37 @@ __global__ void __launch_bounds__(128) k_refill(BoundaryLaunch L) {
     float u[3];
     rigid_u(P, x, y, z, u);
     const float usq15 = 1.5f * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-    float J[3] = {0.f, 0.f, 0.f};  // momentum of the refilled populations (sum e_i (f_i - w_i))
-#pragma unroll
-    for (int i = 0; i < 19; ++i) {
-      const float eu = cx(i) * u[0] + cy(i) * u[1] + cz(i) * u[2];
-      long long nb;
-      float h;
-      if (i != 0 && nbr_wrap(x, y, z, cx(i), cy(i), cz(i), g, nb) && L.pl.owner_cur[nb] == OWNER_NONE &&
-          L.pl.owner_prev[nb] == OWNER_NONE) {
-        h = Store<ST>::dev(A + opp(i) * g.plane + nb, opp(i)) + 6.0f * wq(i) * rho0 * eu;
-      } else {
-        h = wq(i) * (rho0 - 1.0f) + wq(i) * rho0 * (3.0f * eu + 4.5f * eu * eu - usq15);
-      }
-      Store<ST>::put(A + i * g.plane + c, i, h);
-      J[0] += cx(i) * h;
-      J[1] += cy(i) * h;
-      J[2] += cz(i) * h;
-    }
-    // cover/uncover rule: the particle that uncovered the node gives up this momentum
-    if (L.pl.cover_uncover) add_node_momentum(L.pl.facc, L.pl.P, pid, x, y, z, J, -1.0f);
+    const float eu = ex * u[0] + ey * u[1] + ez * u[2];
+    long long nb = c;
+    const bool from = i != 0 && nbr_wrap(x, y, z, ex, ey, ez, g, nb);
+    const bool fluid = (L.pl.owner_cur[nb] == OWNER_NONE) & (L.pl.owner_prev[nb] == OWNER_NONE);
+    const float there = Store<ST>::dev_at(A + oi * g.plane + nb, wi);
+    const float h = from && fluid ? there + 6.0f * wi * rho0 * eu
+                                  : wi * (rho0 - 1.0f) + wi * rho0 * (3.0f * eu + 4.5f * eu * eu - usq15);
+    if (lane < 19u) Store<ST>::put_at(A + i * g.plane + c, wi, h);
+    // cover/uncover rule: the particle that uncovered the node gives up the
+    // momentum of the refilled populations, sum e_i (f_i - w_i)
+    if (L.pl.cover_uncover) add_node_momentum(L.pl.facc, L.pl.P, pid, x, y, z, lane < 19u ? h : 0.f, ex, ey, ez, -1.0f, lane);
   }
   if (!L.pl.cover_uncover) return;
   // covered nodes: the momentum of their post-collision populations f+(t)
   // (still in A: they were fluid) goes to the particle that covered them
   const unsigned nc = min(L.pl.ctr->n_cov, L.pl.cap_new);
-  for (unsigned k = blockIdx.x * blockDim.x + threadIdx.x; k < nc; k += gridDim.x * blockDim.x) {
+  for (unsigned k = wid; k < nc; k += nw) {
     const long long c = L.pl.cov_cell[k];
     int x, y, z;
     coords(c, g, x, y, z);
-    float J[3] = {0.f, 0.f, 0.f};
-#pragma unroll
-    for (int i = 1; i < 19; ++i) {
-      const float h = Store<ST>::dev(A + i * g.plane + c, i);
-      J[0] += cx(i) * h;
-      J[1] += cy(i) * h;
-      J[2] += cz(i) * h;
-    }
-    add_node_momentum(L.pl.facc, L.pl.P, L.pl.owner_cur[c], x, y, z, J, 1.0f);
+    const float h = Store<ST>::dev_at(A + i * g.plane + c, wi);
+    add_node_momentum(L.pl.facc, L.pl.P, L.pl.owner_cur[c], x, y, z, lane < 19u ? h : 0.f, ex, ey, ez, 1.0f, lane);
   }
 }
 
 // ---------------------------------------------------------------------------
-// Nodes next to an uncovered node: recomputed after the refill (the bulk
-// kernel may have read their neighbour's populations before it was refilled).
-// One thread per (uncovered node, direction); a node reached twice is written
-// twice with the same values.
+// An uncovered node and the nodes next to it: recomputed after the refill (the
+// bulk kernel may have read its populations before they were refilled), solid
+// ones too, whose values nothing uses but which would otherwise depend on
+// which kernel came first.  One thread per (uncovered node, direction); a node
+// reached twice is written twice with the same values.
 // ---------------------------------------------------------------------------
 template <int ST, bool FORCE>
 __global__ void __launch_bounds__(128) k_near(BoundaryLaunch L) {
@@ -571,14 +575,14 @@ __global__ void __launch_bounds__(128) k_near(BoundaryLaunch L) {
   T* __restrict__ B = static_cast<T*>(L.B);
   const LatticeGeom& g = L.pl.g;
   const unsigned nn = min(L.pl.ctr->n_new, L.pl.cap_new);
-  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < nn * 18u; t += gridDim.x * blockDim.x) {
-    const unsigned k = t / 18u;
-    const int d = 1 + (int)(t - 18u * k);
+  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < nn * 19u; t += gridDim.x * blockDim.x) {
+    const unsigned k = t / 19u;
+    const int d = (int)(t - 19u * k);
     int x, y, z;
     coords(L.pl.new_cell[k], g, x, y, z);
     long long nb;
-    if (!nbr_wrap(x, y, z, cx(d), cy(d), cz(d), g, nb)) continue;
-    if (L.pl.owner_cur[nb] != OWNER_NONE || (L.pl.cls[nb] & CLS_BOUNDARY)) continue;
+    if (!nbr_wrap(x, y, z, lex(d), ley(d), lez(d), g, nb)) continue;
+    if (L.pl.cls[nb] & CLS_BOUNDARY) continue;
     int a, b, c;
     coords(nb, g, a, b, c);
     update_node<ST, FORCE>(A, B, g, L.p, a, b, c, nb);
@@ -617,10 +621,6 @@ __global__ void __launch_bounds__(128) k_near(BoundaryLaunch L) {
 // ---------------------------------------------------------------------------
 namespace {
 constexpr unsigned FULLW = 0xffffffffu;
-// weight and opposite of a direction given at run time (lex, ley, lez: the
-// shared header's packed direction tables)
-__device__ __forceinline__ float lw(int j) { return j == 0 ? (1.0f / 3.0f) : (j <= 6 ? (1.0f / 18.0f) : (1.0f / 36.0f)); }
-__device__ __forceinline__ int lopp(int j) { return j == 0 ? 0 : ((j & 1) ? j + 1 : j - 1); }
 
 // Exact warp sum of 64-bit fixed-point values (|v| < 2^62): three 22-bit
 // pieces, each summed by one integer warp reduction (at most 32 x 2^22 < 2^27,
@@ -919,7 +919,8 @@ static inline int list_grid(int tuned, unsigned long long items, int threads) {
 
 template <int ST>
 static cudaError_t launch_refill_st(const BoundaryLaunch& L, cudaStream_t s) {
-  k_refill<ST><<<list_grid(L.grid, L.pl.cap_new, 128), 128, 0, s>>>(L);
+  // a warp per node; a step uncovers a small part of what the list can hold
+  k_refill<ST><<<list_grid(L.grid, (L.pl.cap_new + 15ull) / 16ull, 4), 128, 0, s>>>(L);
   return cudaGetLastError();
 }
 
@@ -959,7 +960,8 @@ cudaError_t launch_links_ibb(const BoundaryLaunch& L, cudaStream_t s) {
 
 template <int ST>
 static cudaError_t launch_near_st(const BoundaryLaunch& L, cudaStream_t s) {
-  const int grid = list_grid(L.grid, 18ull * L.pl.cap_new, 128);
+  // a step uncovers a small part of what the list can hold
+  const int grid = list_grid(L.grid, 19ull * ((L.pl.cap_new + 15ull) / 16ull), 128);
   if (L.forcing) k_near<ST, true><<<grid, 128, 0, s>>>(L);
   else k_near<ST, false><<<grid, 128, 0, s>>>(L);
   return cudaGetLastError();

@@ -25,21 +25,27 @@ namespace mi {
 namespace {
 constexpr float GUARD = FIELD_GUARD;
 
-__device__ __forceinline__ void quat_to_R_exact(const double q[4], double R[9]) {
-  // body -> world rotation of the normalised quaternion, unfused FP64
-  double n = __dsqrt_rn(__dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(q[0], q[0]), __dmul_rn(q[1], q[1])),
-                                            __dmul_rn(q[2], q[2])),
-                                  __dmul_rn(q[3], q[3])));
-  const double w = __ddiv_rn(q[0], n), x = __ddiv_rn(q[1], n), y = __ddiv_rn(q[2], n), z = __ddiv_rn(q[3], n);
-  R[0] = __dsub_rn(1.0, __dmul_rn(2.0, __dadd_rn(__dmul_rn(y, y), __dmul_rn(z, z))));
-  R[1] = __dmul_rn(2.0, __dsub_rn(__dmul_rn(x, y), __dmul_rn(w, z)));
-  R[2] = __dmul_rn(2.0, __dadd_rn(__dmul_rn(x, z), __dmul_rn(w, y)));
-  R[3] = __dmul_rn(2.0, __dadd_rn(__dmul_rn(x, y), __dmul_rn(w, z)));
-  R[4] = __dsub_rn(1.0, __dmul_rn(2.0, __dadd_rn(__dmul_rn(x, x), __dmul_rn(z, z))));
-  R[5] = __dmul_rn(2.0, __dsub_rn(__dmul_rn(y, z), __dmul_rn(w, x)));
-  R[6] = __dmul_rn(2.0, __dsub_rn(__dmul_rn(x, z), __dmul_rn(w, y)));
-  R[7] = __dmul_rn(2.0, __dadd_rn(__dmul_rn(y, z), __dmul_rn(w, x)));
-  R[8] = __dsub_rn(1.0, __dmul_rn(2.0, __dadd_rn(__dmul_rn(x, x), __dmul_rn(y, y))));
+// Entry k = lane of the body -> world rotation of the normalised quaternion q,
+// unfused FP64 (lanes 9 and up repeat entry 8).  An FP64 instruction costs the
+// same issue time for one lane as for 32 on this part, so the lanes share the
+// work: lane l divides component l & 3 by the norm, and one sequence of
+// products serves all nine entries, 1 - 2 (a^2 + c^2) or 2 (a b +- c d).
+__device__ __forceinline__ double rotation_entry(const double q[4], int lane) {
+  const double n = __dsqrt_rn(__dadd_rn(__dadd_rn(__dadd_rn(__dmul_rn(q[0], q[0]), __dmul_rn(q[1], q[1])),
+                                                  __dmul_rn(q[2], q[2])),
+                                        __dmul_rn(q[3], q[3])));
+  const int c4 = lane & 3;
+  const double v = __ddiv_rn(c4 == 0 ? q[0] : (c4 == 1 ? q[1] : (c4 == 2 ? q[2] : q[3])), n);
+  // components (w, x, y, z) = 0..3 of the factors a b and c d of entry k, a hexadecimal digit each
+  const int k = 4 * (lane < 8 ? lane : 8);
+  const double a = __shfl_sync(0xffffffffu, v, (int)((0x121211112ull >> k) & 15ull)),
+               b = __shfl_sync(0xffffffffu, v, (int)((0x133312322ull >> k) & 15ull)),
+               c = __shfl_sync(0xffffffffu, v, (int)((0x200030003ull >> k) & 15ull)),
+               d = __shfl_sync(0xffffffffu, v, (int)((0x212133233ull >> k) & 15ull));
+  const bool minus = (0x62 >> (k / 4)) & 1, diag = (0x111 >> (k / 4)) & 1;
+  const double p = __dmul_rn(c, d);
+  const double t = __dmul_rn(2.0, __dadd_rn(__dmul_rn(a, b), minus ? -p : p));
+  return diag ? __dsub_rn(1.0, t) : t;
 }
 
 // f(x) >= 1 in FP64, unfused, same operation order as the definition above,
@@ -117,81 +123,6 @@ __device__ __forceinline__ bool neighbour(int x, int y, int z, int dx, int dy, i
 }
 }  // namespace
 
-// ---------------------------------------------------------------------------
-// Prologue: bump the flag generation, zero counters and hydrodynamic force
-// sums, rotation matrices and node boxes at the current pose.
-// ---------------------------------------------------------------------------
-__global__ void k_prologue(ParticleLaunch L) {
-  // one warp per particle: every lane forms the rotation (the same FP64
-  // operations, so the same bits), then the lanes share out the float pairs
-  // of its entries and of the directions
-  const int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-  if (p == 0 && lane == 0) {
-    L.ctr->gen += 1u;
-    L.ctr->n_bc = 0;
-    L.ctr->n_links = 0;
-    L.ctr->n_new = 0;
-    L.ctr->n_cov = 0;
-  }
-  if (p >= L.np) return;
-  DevParticle& P = L.P[p];
-  double R[9];
-  quat_to_R_exact(P.quat, R);
-  if (lane < 9) {
-    double r = R[0];
-#pragma unroll
-    for (int k = 1; k < 9; ++k) r = lane == k ? R[k] : r;
-    const float rf = (float)r;
-    P.R[lane] = r;
-    P.Rf[lane] = rf;
-    P.Rs[0][lane] = rf;
-    P.Rs[1][lane] = (float)(r - (double)rf);
-  } else if (lane < 12) {
-    // R^T (X - floor X), entry k
-    const int k = lane - 9;
-    double fr[3], c[3];
-    for (int a = 0; a < 3; ++a) fr[a] = P.pos[a] - floor(P.pos[a]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) c[a] = k == 0 ? R[3 * a] : (k == 1 ? R[3 * a + 1] : R[3 * a + 2]);
-    const double t = c[0] * fr[0] + c[1] * fr[1] + c[2] * fr[2];
-    P.Ts[0][k] = (float)t;
-    P.Ts[1][k] = (float)(t - (double)P.Ts[0][k]);
-  }
-  if (lane < 19) {
-    // R^T e_d for direction d = lane
-    const int d = lane;
-    const double ex = lex(d), ey = ley(d), ez = lez(d);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const double e = R[k] * ex + R[3 + k] * ey + R[6 + k] * ez;
-      P.Es[d][k] = (float)e;
-      P.Es[d][3 + k] = (float)(e - (double)P.Es[d][k]);
-    }
-  }
-  if (lane == 0) {
-    for (int a = 0; a < 3; ++a) {
-      P.lo[a] = (int)floor(P.pos[a] - P.Rt) - 1;
-      P.posf[a] = (float)P.pos[a];
-      const double fl = floor(P.pos[a]);
-      P.pos_i[a] = (int)fl;
-      P.pos_fr[a] = (float)(P.pos[a] - fl);
-      P.velf[a] = (float)P.vel[a];
-      P.omegaf[a] = (float)P.omega[a];
-      const int prev = P.lo_hist[L.prev_buf][a];
-      if (prev != BOX_NONE && abs(P.lo[a] - prev) > 2) atomicOr(&L.ctr->status, STATUS_MOVED_TOO_FAR);
-    }
-    P.srad2[L.cur_buf] = -1;  // the solid radius of this step, grown by k_flag
-    for (int a = 0; a < 3; ++a) P.sctr[L.cur_buf][a] = (float)P.pos[a];
-  }
-  if (lane < 6) L.facc[6 * p + lane] = 0;
-}
-
-cudaError_t launch_prologue(const ParticleLaunch& L, cudaStream_t s) {
-  const int blocks = L.np > 0 ? (L.np + 3) / 4 : 1;  // four warps per block, a warp per particle
-  k_prologue<<<blocks, 128, 0, s>>>(L);
-  return cudaGetLastError();
-}
-
 // The particle owning block b of a box kernel's 1D grid (off[p] <= b <
 // off[p + 1], off[0] = 0) by binary search, its first block and block count.
 struct BoxBlock {
@@ -209,28 +140,99 @@ __device__ __forceinline__ BoxBlock box_block(const int* __restrict__ off, int n
 }
 
 // ---------------------------------------------------------------------------
-// Clear the owner buffer about to be rewritten, over the boxes it was last
-// written with.
+// Prologue, one launch of two independent parts.  The first blocks, a warp
+// per particle: bump the flag generation, zero counters and hydrodynamic
+// force sums, rotation matrices and node boxes at the current pose.  The other
+// blocks clear the owner buffer about to be rewritten over the boxes it was
+// last written with (nothing the first part touches).
 // ---------------------------------------------------------------------------
-__global__ void k_clear(ParticleLaunch L) {
-  const BoxBlock bb = box_block(L.flag_off, L.np, blockIdx.x);
-  const DevParticle& P = L.P[bb.p];
-  const int* lo = P.lo_hist[L.cur_buf];
-  if (lo[0] == BOX_NONE) return;
-  const Region r = clip_region(lo, P.ext, 0, L.g);
-  const unsigned n0 = (unsigned)r.n[0], n01 = n0 * (unsigned)r.n[1];
-  for (unsigned i = bb.b * blockDim.x + threadIdx.x; i < r.total; i += bb.nb * blockDim.x) {
-    const unsigned zi = i / n01, rem = i - zi * n01, yi = rem / n0;
-    const int x = r.lo[0] + (int)(rem - yi * n0);
-    const int y = r.lo[1] + (int)yi;
-    const int z = r.lo[2] + (int)zi;
-    L.owner_cur[lin(x, y, z, L.g)] = OWNER_NONE;
+constexpr int PROLOGUE_THREADS = 256;
+__global__ void __launch_bounds__(PROLOGUE_THREADS) k_prologue(ParticleLaunch L) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const int nprol = (L.np + PROLOGUE_THREADS / 32 - 1) / (PROLOGUE_THREADS / 32);
+  if ((int)blockIdx.x >= nprol) {
+    const BoxBlock bb = box_block(L.flag_off, L.np, (int)blockIdx.x - nprol);
+    const DevParticle& P = L.P[bb.p];
+    const int* lo = P.lo_hist[L.cur_buf];
+    if (lo[0] == BOX_NONE) return;
+    const Region r = clip_region(lo, P.ext, 0, L.g);
+    const unsigned n0 = (unsigned)r.n[0], n01 = n0 * (unsigned)r.n[1];
+    for (unsigned i = bb.b * blockDim.x + threadIdx.x; i < r.total; i += bb.nb * blockDim.x) {
+      const unsigned zi = i / n01, rem = i - zi * n01, yi = rem / n0;
+      const int x = r.lo[0] + (int)(rem - yi * n0);
+      const int y = r.lo[1] + (int)yi;
+      const int z = r.lo[2] + (int)zi;
+      L.owner_cur[lin(x, y, z, L.g)] = OWNER_NONE;
+    }
+    return;
   }
+  const int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (p == 0 && lane == 0) {
+    L.ctr->gen += 1u;
+    L.ctr->n_bc = 0;
+    L.ctr->n_links = 0;
+    L.ctr->n_new = 0;
+    L.ctr->n_cov = 0;
+  }
+  if (p >= L.np) return;
+  DevParticle& P = L.P[p];
+  const double r = rotation_entry(P.quat, lane);
+  double R[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) R[k] = __shfl_sync(FULL, r, k);
+  if (lane < 9) {
+    const float rf = (float)r;
+    P.R[lane] = r;
+    P.Rf[lane] = rf;
+    P.Rs[0][lane] = rf;
+    P.Rs[1][lane] = (float)(r - (double)rf);
+  }
+  // axis a = lane % 3 of the box and of the position's split; the stores by lanes 0-2
+  const int a = lane % 3;
+  const double pos = a == 0 ? P.pos[0] : (a == 1 ? P.pos[1] : P.pos[2]), fl = floor(pos), fr = pos - fl;
+  {
+    // R^T (X - floor X), entry a
+    double f[3], c[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      f[k] = __shfl_sync(FULL, fr, k);
+      c[k] = a == 0 ? R[3 * k] : (a == 1 ? R[3 * k + 1] : R[3 * k + 2]);
+    }
+    const double t = c[0] * f[0] + c[1] * f[1] + c[2] * f[2];
+    const int lo = (int)floor(pos - P.Rt) - 1;
+    if (lane < 3) {
+      const float tf = (float)t;
+      P.Ts[0][a] = tf;
+      P.Ts[1][a] = (float)(t - (double)tf);
+      P.lo[a] = lo;
+      P.posf[a] = (float)pos;
+      P.pos_i[a] = (int)fl;
+      P.pos_fr[a] = (float)fr;
+      P.velf[a] = (float)P.vel[a];
+      P.omegaf[a] = (float)P.omega[a];
+      P.sctr[L.cur_buf][a] = (float)pos;
+      const int prev = P.lo_hist[L.prev_buf][a];
+      if (prev != BOX_NONE && abs(lo - prev) > 2) atomicOr(&L.ctr->status, STATUS_MOVED_TOO_FAR);
+    }
+  }
+  if (lane < 19) {
+    // R^T e_d for direction d = lane
+    const int d = lane;
+    const double ex = lex(d), ey = ley(d), ez = lez(d);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double e = R[k] * ex + R[3 + k] * ey + R[6 + k] * ez;
+      P.Es[d][k] = (float)e;
+      P.Es[d][3 + k] = (float)(e - (double)P.Es[d][k]);
+    }
+  }
+  if (lane == 0) P.srad2[L.cur_buf] = -1;  // the solid radius of this step, grown by k_flag
+  if (lane < 6) L.facc[6 * p + lane] = 0;
 }
 
-cudaError_t launch_clear(const ParticleLaunch& L, cudaStream_t s) {
-  if (L.np == 0) return cudaSuccess;
-  k_clear<<<L.flag_blocks, 256, 0, s>>>(L);
+cudaError_t launch_prologue(const ParticleLaunch& L, cudaStream_t s) {
+  const int per = PROLOGUE_THREADS / 32, nprol = (L.np + per - 1) / per;
+  k_prologue<<<nprol + (L.np > 0 ? L.flag_blocks : 1), PROLOGUE_THREADS, 0, s>>>(L);
   return cudaGetLastError();
 }
 
@@ -347,9 +349,84 @@ cudaError_t launch_flag(const ParticleLaunch& L, cudaStream_t s) {
 // (solid now, fluid at the previous step).  Boxes may overlap: every block
 // writes the same class for a node, and a per-node generation stamp lets
 // exactly one block append it to the boundary / uncovered / covered lists.
+//
+// One warp per (y, z) row, 30 nodes at a time (lanes 1 to 30, lanes 0 and 31
+// their x neighbours): the owners of the row and of its eight neighbour rows
+// are one coalesced load each, a ballot turns each into a bit row, and a lane
+// takes the 18 solid bits around its node from the nine words (a load per
+// direction and node needs twice the loads, all waited for).  A warp keeps its
+// boundary nodes in shared memory and appends 32 at a time: all warps share
+// the two list counters, and one same-address atomic per counter and chunk
+// (about three boundary nodes) took most of the kernel's time on a lattice of
+// 300 particles.  The 32 nodes' links are written by the whole warp, a lane
+// per link.  Bound by L2 latency: 300 particles (0.82 M boundary nodes) 305 us
+// alone, 588 with an append per chunk, 640 with a load per direction and node
+// and links written node by node; the settling tank's three particles 108 us
+// (45 blocks beside the bulk kernel, before 219).
 // ---------------------------------------------------------------------------
+namespace {
+constexpr int CLS_WARPS = 8, CLS_KEEP = 64;  // a chunk adds at most 30 nodes to at most 31 kept
+struct BoundaryKeep {
+  uint32_t x[CLS_KEEP], yz[CLS_KEEP], mask[CLS_KEEP];  // y in the low 16 bits, z in the high (both <= 65535)
+};
+
+// Append the first n (<= 32) kept nodes and their links to the lists.
+__device__ __forceinline__ void append_boundary(const ParticleLaunch& L, const BoundaryKeep& K, int n, int lane) {
+  constexpr unsigned FULL = 0xffffffffu;
+  const uint32_t x = lane < n ? K.x[lane] : 0u, yz = lane < n ? K.yz[lane] : 0u, mask = lane < n ? K.mask[lane] : 0u;
+  const unsigned m = (unsigned)__popc(mask);
+  unsigned incl = m;
+#pragma unroll
+  for (int k = 1; k < 32; k <<= 1) {
+    const unsigned v = __shfl_up_sync(FULL, incl, k);
+    if (lane >= k) incl += v;
+  }
+  const unsigned total = __shfl_sync(FULL, incl, 31);
+  unsigned got = 0;
+  if (lane == 0) got = atomicAdd(&L.ctr->n_bc, (unsigned)n);
+  if (lane == 1) got = atomicAdd(&L.ctr->n_links, total);
+  const unsigned bi = __shfl_sync(FULL, got, 0) + (unsigned)lane, base_l = __shfl_sync(FULL, got, 1);
+  const unsigned lo_l = base_l + incl - m;
+  bool fits = false;  // this node's links are written
+  if (lane < n) {
+    if (bi >= L.cap_bc) {
+      atomicOr(&L.ctr->status, STATUS_BC_OVERFLOW);
+    } else {
+      L.bc_cell[bi] = (uint32_t)lin((int)x, (int)(yz & 0xffffu), (int)(yz >> 16), L.g);
+      L.bc_mask[bi] = mask;
+      L.bc_loff[bi] = lo_l;
+      fits = lo_l + m <= L.cap_links;
+      if (!fits) atomicOr(&L.ctr->status, STATUS_LINK_OVERFLOW);
+    }
+  }
+  // the links, a lane each: the node (lane s) by binary search in the prefix
+  // sums, the direction as the k-th set bit of its mask
+  for (unsigned t0 = 0; t0 < total; t0 += 32) {
+    const unsigned t = t0 + (unsigned)lane;
+    int s = 0;
+#pragma unroll
+    for (int k = 16; k > 0; k >>= 1)
+      if (__shfl_sync(FULL, incl, s + k - 1) <= t) s += k;
+    const unsigned e = __shfl_sync(FULL, incl - m, s);
+    unsigned ms = __shfl_sync(FULL, mask, s);
+    const unsigned sbi = __shfl_sync(FULL, bi, s), sx = __shfl_sync(FULL, x, s), syz = __shfl_sync(FULL, yz, s);
+    const bool ok = __shfl_sync(FULL, (int)fits, s) != 0;
+    if (t < total && ok) {
+      for (unsigned k = t - e; k > 0; --k) ms &= ms - 1u;
+      const int d = __ffs(ms) - 1;
+      long long nbr;
+      neighbour((int)sx, (int)(syz & 0xffffu), (int)(syz >> 16), lex(d), ley(d), lez(d), L.g, nbr);
+      L.link_bc[base_l + t] = sbi;
+      L.link_dir[base_l + t] = (uint8_t)d;
+      L.link_p[base_l + t] = L.owner_cur[nbr];
+    }
+  }
+}
+}  // namespace
+
 template <bool COV>
-__global__ void __launch_bounds__(256) k_classify(ParticleLaunch L) {
+__global__ void __launch_bounds__(32 * CLS_WARPS) k_classify(ParticleLaunch L) {
+  constexpr unsigned FULL = 0xffffffffu;
   const BoxBlock bb = box_block(L.cls_off, L.np, blockIdx.x);
   const DevParticle& P = L.P[bb.p];
   int lo[3], ext[3];
@@ -381,8 +458,12 @@ __global__ void __launch_bounds__(256) k_classify(ParticleLaunch L) {
   const unsigned gen = L.ctr->gen;
   // one warp per (y, z) row of the region: the row's x-interval inside
   // either sphere, computed once per row (rows that miss both are skipped by
-  // the whole warp), its nodes taken 32 at a time
+  // the whole warp)
   const int lane = threadIdx.x & 31;
+  __shared__ BoundaryKeep keep[CLS_WARPS];
+  BoundaryKeep& K = keep[threadIdx.x >> 5];
+  int kept = 0;
+  const LatticeGeom& g = L.g;
   const unsigned rows = (unsigned)r.n[1] * (unsigned)r.n[2];
   const unsigned wid = (bb.b * blockDim.x + threadIdx.x) >> 5, nw = (bb.nb * blockDim.x) >> 5;
   for (unsigned row = wid; row < rows; row += nw) {
@@ -409,103 +490,97 @@ __global__ void __launch_bounds__(256) k_classify(ParticleLaunch L) {
     // a row outside both spheres (xa > xb) is skipped before any index is
     // formed: xa = INT_MAX + lane would overflow
     if (xa > xb) continue;
-    for (int x = xa + lane; x <= xb; x += 32) {
-    const long long c = lin(x, y, z, L.g);
-    const bool solid = L.owner_cur[c] != OWNER_NONE;
-    const bool was = L.owner_prev[c] != OWNER_NONE;
-    uint32_t mask = 0;
-    if (!solid) {
-      const bool interior = (x > 0) & (x < L.g.nx - 1) & (y > 0) & (y < L.g.ny - 1) & (z > 0) & (z < L.g.nz - 1);
-      if (interior) {
-        const long long sy = L.g.nx, sz = (long long)L.g.nx * L.g.ny;
+    // the nine rows' first nodes, -1 outside the domain
+    long long base[9];
 #pragma unroll
-        for (int d = 1; d < 19; ++d)
-          if (__ldg(L.owner_cur + c + cx(d) + sy * cy(d) + sz * cz(d)) != OWNER_NONE) mask |= 1u << d;
-      } else {
-#pragma unroll 1
-        for (int d = 1; d < 19; ++d) {
-          long long nbr;
-          if (neighbour(x, y, z, cx(d), cy(d), cz(d), L.g, nbr) && L.owner_cur[nbr] != OWNER_NONE) mask |= 1u << d;
+    for (int k = 0; k < 9; ++k) {
+      int b = y + k % 3 - 1, c = z + k / 3 - 1;
+      bool in = true;
+      if (b < 0 || b >= g.ny) {
+        in = g.periodic[1] != 0;
+        b += b < 0 ? g.ny : -g.ny;
+      }
+      if (c < 0 || c >= g.nz) {
+        in = in && g.periodic[2] != 0;
+        c += c < 0 ? g.nz : -g.nz;
+      }
+      base[k] = in ? lin(0, b, c, g) : -1;
+    }
+    for (int xs = xa - 1; xs < xb; xs += 30) {
+      const int x = xs + lane;
+      const bool node = lane >= 1 && lane <= 30 && x <= xb;
+      int xw = x;
+      if (x < 0 || x >= g.nx) xw = g.periodic[0] ? (x < 0 ? x + g.nx : x - g.nx) : -1;
+      const bool load = x <= xb + 1 && xw >= 0;
+      uint32_t o[9];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) o[k] = load && base[k] >= 0 ? __ldg(L.owner_cur + base[k] + xw) : OWNER_NONE;
+      const long long c = base[4] + x;
+      const bool was = node && L.owner_prev[c] != OWNER_NONE;
+      unsigned bits[9], any = 0;
+#pragma unroll
+      for (int k = 0; k < 9; ++k) any |= bits[k] = __ballot_sync(FULL, o[k] != OWNER_NONE);
+      const bool solid = o[4] != OWNER_NONE;
+      uint32_t mask = 0;
+      if (any && node && !solid) {
+#pragma unroll
+        for (int d = 1; d < 19; ++d) mask |= ((bits[3 * (cz(d) + 1) + cy(d) + 1] >> (lane + cx(d))) & 1u) << d;
+      }
+      const bool isnew = node && !solid && was;
+      // covered: listed for the cover/uncover rule only, and not in the step
+      // that first flags the covering particle (it was not there before)
+      const bool iscov = COV && node && solid && !was && L.P[o[4]].lo_hist[L.prev_buf][0] != BOX_NONE;
+      if (node) L.cls[c] = (uint8_t)((solid ? CLS_SOLID : 0) | (mask ? CLS_BOUNDARY : 0) | (isnew ? CLS_NEW : 0));
+      bool list = mask || isnew || iscov;
+      if (!__any_sync(FULL, list)) continue;
+      if (list) list = atomicExch(L.stamp + c, gen) != gen;  // else another block listed it
+      const unsigned below = (1u << lane) - 1u;
+      const unsigned newm = __ballot_sync(FULL, list && isnew), bcm = __ballot_sync(FULL, list && mask != 0);
+      const unsigned covm = COV ? __ballot_sync(FULL, list && iscov) : 0u;
+      if (newm | covm) {
+        unsigned got = 0;
+        if (lane == 0 && newm) got = atomicAdd(&L.ctr->n_new, (unsigned)__popc(newm));
+        if (COV && lane == 1 && covm) got = atomicAdd(&L.ctr->n_cov, (unsigned)__popc(covm));
+        const unsigned base_new = __shfl_sync(FULL, got, 0), base_cov = __shfl_sync(FULL, got, 1);
+        if (list && isnew) {
+          const unsigned k = base_new + __popc(newm & below);
+          if (k < L.cap_new) L.new_cell[k] = (uint32_t)c;
+          else atomicOr(&L.ctr->status, STATUS_NEW_OVERFLOW);
+        }
+        if (COV && list && iscov) {
+          const unsigned k = base_cov + __popc(covm & below);
+          if (k < L.cap_new) L.cov_cell[k] = (uint32_t)c;
+          else atomicOr(&L.ctr->status, STATUS_NEW_OVERFLOW);
         }
       }
-    }
-    const bool isnew = !solid && was;
-    // covered: listed for the cover/uncover rule only, and not in the step
-    // that first flags the covering particle (it was not there before)
-    const bool iscov = COV && solid && !was && L.P[L.owner_cur[c]].lo_hist[L.prev_buf][0] != BOX_NONE;
-    L.cls[c] = (uint8_t)((solid ? CLS_SOLID : 0) | (mask ? CLS_BOUNDARY : 0) | (isnew ? CLS_NEW : 0));
-    if (!(mask || isnew || iscov)) continue;
-    if (atomicExch(L.stamp + c, gen) == gen) continue;  // another block listed it
-    // list appends aggregated over the lanes that got here: one atomic per
-    // counter and warp (all boundary nodes share the counters, and
-    // same-address atomics serialise in L2), offsets by ballot ranks and a scan
-    const cg::coalesced_group grp = cg::coalesced_threads();
-    const unsigned below = (1u << grp.thread_rank()) - 1u;
-    const unsigned newm = grp.ballot(isnew), bcm = grp.ballot(mask != 0);
-    const unsigned m = __popc(mask);
-    const unsigned m_excl = cg::exclusive_scan(grp, m);
-    unsigned base_new = 0, base_bc = 0, base_l = 0;
-    if (grp.thread_rank() == 0) {
-      if (newm) base_new = atomicAdd(&L.ctr->n_new, (unsigned)__popc(newm));
-      if (bcm) base_bc = atomicAdd(&L.ctr->n_bc, (unsigned)__popc(bcm));
-    }
-    if (grp.thread_rank() == grp.size() - 1) {
-      const unsigned total = m_excl + m;
-      if (total) base_l = atomicAdd(&L.ctr->n_links, total);
-    }
-    base_new = grp.shfl(base_new, 0);
-    base_bc = grp.shfl(base_bc, 0);
-    base_l = grp.shfl(base_l, grp.size() - 1);
-    if (isnew) {
-      const unsigned k = base_new + __popc(newm & below);
-      if (k < L.cap_new) L.new_cell[k] = (uint32_t)c;
-      else atomicOr(&L.ctr->status, STATUS_NEW_OVERFLOW);
-    }
-    if constexpr (COV) {
-      const unsigned covm = grp.ballot(iscov);
-      unsigned base_cov = 0;
-      if (grp.thread_rank() == 0 && covm) base_cov = atomicAdd(&L.ctr->n_cov, (unsigned)__popc(covm));
-      base_cov = grp.shfl(base_cov, 0);
-      if (iscov) {
-        const unsigned k = base_cov + __popc(covm & below);
-        if (k < L.cap_new) L.cov_cell[k] = (uint32_t)c;
-        else atomicOr(&L.ctr->status, STATUS_NEW_OVERFLOW);
+      if (list && mask) {
+        const int k = kept + __popc(bcm & below);
+        K.x[k] = (uint32_t)x;
+        K.yz[k] = (uint32_t)y | ((uint32_t)z << 16);
+        K.mask[k] = mask;
       }
-    }
-    if (mask) {
-      const unsigned bi = base_bc + __popc(bcm & below);
-      const unsigned lo_l = base_l + m_excl;
-      if (bi >= L.cap_bc) {
-        atomicOr(&L.ctr->status, STATUS_BC_OVERFLOW);
-        continue;
-      }
-      L.bc_cell[bi] = (uint32_t)c;
-      L.bc_mask[bi] = mask;
-      L.bc_loff[bi] = lo_l;
-      if (lo_l + m > L.cap_links) {
-        atomicOr(&L.ctr->status, STATUS_LINK_OVERFLOW);
-        continue;
-      }
-      unsigned k = 0;
-      for (int d = 1; d < 19; ++d) {
-        if (!((mask >> d) & 1u)) continue;
-        long long nbr;
-        neighbour(x, y, z, cx(d), cy(d), cz(d), L.g, nbr);
-        L.link_bc[lo_l + k] = bi;
-        L.link_dir[lo_l + k] = (uint8_t)d;
-        L.link_p[lo_l + k] = L.owner_cur[nbr];
-        ++k;
+      kept += __popc(bcm);
+      __syncwarp();
+      if (kept >= 32) {
+        append_boundary(L, K, 32, lane);
+        kept -= 32;  // the rest (fewer than 32) moves to the front
+        __syncwarp();
+        if (lane < kept) {
+          K.x[lane] = K.x[lane + 32];
+          K.yz[lane] = K.yz[lane + 32];
+          K.mask[lane] = K.mask[lane + 32];
+        }
+        __syncwarp();
       }
     }
   }
-  }
+  if (kept) append_boundary(L, K, kept, lane);
 }
 
 cudaError_t launch_classify(const ParticleLaunch& L, cudaStream_t s) {
   if (L.np == 0) return cudaSuccess;
-  // a warp per (y, z) row, about 64 rows per warp
-  if (L.cover_uncover) k_classify<true><<<L.classify_blocks, 256, 0, s>>>(L);
-  else k_classify<false><<<L.classify_blocks, 256, 0, s>>>(L);
+  if (L.cover_uncover) k_classify<true><<<L.classify_blocks, 32 * CLS_WARPS, 0, s>>>(L);
+  else k_classify<false><<<L.classify_blocks, 32 * CLS_WARPS, 0, s>>>(L);
   return cudaGetLastError();
 }
 

@@ -66,6 +66,9 @@ template <> struct Store<MI_STORE_F32> {
   using T = float;
   static __device__ __forceinline__ float dev(const float* p, int i) { return __ldg(p) - wq(i); }
   static __device__ __forceinline__ void put(float* p, int i, float h) { __stcs(p, h + wq(i)); }
+  // the same with the direction's weight, for a direction known at run time
+  static __device__ __forceinline__ float dev_at(const float* p, float w) { return *p - w; }
+  static __device__ __forceinline__ void put_at(float* p, float w, float h) { __stcs(p, h + w); }
 };
 template <> struct Store<MI_STORE_F16_DEV> {
   using T = __half;
@@ -75,6 +78,8 @@ template <> struct Store<MI_STORE_F16_DEV> {
   static __device__ __forceinline__ void put(__half* p, int, float h) {
     __stcs(reinterpret_cast<unsigned short*>(p), __half_as_ushort(__float2half_rn(h)));
   }
+  static __device__ __forceinline__ float dev_at(const __half* p, float) { return __half2float(*p); }
+  static __device__ __forceinline__ void put_at(__half* p, float, float h) { put(p, 0, h); }
 };
 template <> struct Store<MI_STORE_BF16_DEV> {
   using T = __nv_bfloat16;
@@ -84,6 +89,8 @@ template <> struct Store<MI_STORE_BF16_DEV> {
   static __device__ __forceinline__ void put(__nv_bfloat16* p, int, float h) {
     __stcs(reinterpret_cast<unsigned short*>(p), __bfloat16_as_ushort(__float2bfloat16_rn(h)));
   }
+  static __device__ __forceinline__ float dev_at(const __nv_bfloat16* p, float) { return __bfloat162float(*p); }
+  static __device__ __forceinline__ void put_at(__nv_bfloat16* p, float, float h) { put(p, 0, h); }
 };
 
 inline size_t store_bytes(int st) { return st == MI_STORE_F32 ? 4 : 2; }
@@ -224,7 +231,6 @@ struct ParticleLaunch {
   LatticeGeom g;
 };
 cudaError_t launch_prologue(const ParticleLaunch& L, cudaStream_t s);
-cudaError_t launch_clear(const ParticleLaunch& L, cudaStream_t s);
 cudaError_t launch_flag(const ParticleLaunch& L, cudaStream_t s);
 cudaError_t launch_classify(const ParticleLaunch& L, cudaStream_t s);
 cudaError_t launch_links_q(const ParticleLaunch& L, int grid, cudaStream_t s);

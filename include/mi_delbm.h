@@ -398,8 +398,7 @@ mi_status mi_delbm_set_graphs(mi_delbm *h, int enable);
 
 /* Choose the launch shapes of the bulk kernel (threads per block, from
  * 32/64/128/256) and of the list kernels (blocks per SM for the wall
- * fraction, refill and boundary-node kernels, from 2/4/8/16/32; the links'
- * bounce-back and the boundary nodes are timed together) by timing each candidate
+ * fraction, refill and boundary-node kernels, from 2/4/8/16/32) by timing each candidate
  * with CUDA events on the handle's stream, and use the fastest from then on.
  * With cache_path != NULL, a line {"key": ..., "bulk_block_x": .., "list_blocks_per_sm": ..}
  * for this device, lattice, storage and particle count is read from that file
@@ -423,11 +422,9 @@ enum {
    * start, one kernel runs all substeps of a step in one CTA (the same bits:
    * the same per-item and per-particle device code, no launch per substep) */
   MI_SCHEDULE_UNFUSED_DEM = 2,
-  /* the links' interpolated bounce-back and momentum exchange run on the
-   * particle side stream while the bulk kernel runs, instead of after it
-   * (the same bits; the boundary nodes' collision still follows the bulk
-   * kernel); steps that run the wall fractions, the refill and the boundary
-   * phase.  Implied by MI_SCHEDULE_OVERLAP_BOUNDARY */
+  /* the links' interpolated bounce-back and momentum exchange beside the bulk
+   * kernel instead of after it (the same bits).  One kernel computes them with
+   * the boundary nodes, so this is the schedule of MI_SCHEDULE_OVERLAP_BOUNDARY */
   MI_SCHEDULE_LINKS_BESIDE = 4
 };
 /* Set the step schedule (an OR of MI_SCHEDULE_* flags; 0 = default).
@@ -475,7 +472,7 @@ mi_status mi_delbm_phase_times(mi_delbm *h, double ms[8], long long launches[8],
  * the timed launches of `kernel` since the last reset of mi_delbm_phase_times
  * (not reset by this call).  Names: k_prologue, k_flag, k_classify,
  * k_links_q, k_refill, k_bulk (the bulk stream-collide, whichever variant the
- * tuning selects), k_near, k_links_ibb, k_boundary, k_scatter_boundary, k_dem_prologue,
+ * tuning selects), k_near, k_boundary, k_scatter_boundary, k_dem_prologue,
  * k_broad_phase, k_item_features, k_mlp_tc, k_contacts, k_integrate,
  * k_dem_substeps.  Synchronises.  Errors: MI_EINVAL (NULL argument). */
 mi_status mi_delbm_kernel_time(mi_delbm *h, const char *kernel, double *ms, long long *launches);

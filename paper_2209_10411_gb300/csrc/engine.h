@@ -15,11 +15,13 @@ struct TimedLaunch {
 };
 
 struct TuneChoice {
-  int bulk_block_x = 128;     // threads per block of the bulk kernel (along x)
-  int bulk_rows = 1;          // rows per thread of the bulk kernel
-  int bulk_pairs = 0;         // 0 one node per thread; 1, 2: two x-adjacent nodes per thread with paired
-                              // accesses (nx even; for 16-bit storages 1 and 2 select the register budget)
-  int list_blocks_per_sm = 8; // grid of the list kernels (links, refill, boundary, near) per SM
+  int bulk_block_x = 64;      // threads per block of the bulk kernel
+  int bulk_rows = 1;          // accepted and reported; the bulk kernel has one form
+  int bulk_pairs = 0;         // 16-bit storages: 0 one node per thread; 1, 2: two x-adjacent nodes (nx even);
+                              // 3: four (nx a multiple of 4)
+  int list_blocks_per_sm = 4; // grid of the list kernels (links, refill, boundary, near) per SM: the boundary nodes of
+                              // 300 particles took 569 us with 4, 603 with 8, 575 with 32 (fewer nodes at a time share
+                              // more of the caches)
   bool tuned = false;
 };
 
@@ -100,8 +102,6 @@ struct mi_delbm {
   uint32_t *link_bc = nullptr, *link_p = nullptr;
   uint8_t* link_dir = nullptr;
   float* link_q = nullptr;
-  float* link_g = nullptr;
-  long long* ibb_part = nullptr;     // per-block momentum-exchange sums of the link kernel
   uint32_t* new_cell = nullptr;
   uint32_t* cov_cell = nullptr;     // nodes covered this step (cover/uncover rule; capacity cap_new)
   unsigned cap_bc = 0, cap_links = 0, cap_new = 0;
@@ -109,7 +109,7 @@ struct mi_delbm {
   unsigned need_bc = 0, need_links = 0, need_new = 0;
   void* bc_tmp = nullptr;            // 19 stored values per boundary node (overlapped schedule)
   bool overlap_boundary = false;     // boundary nodes computed beside the bulk kernel, scattered after it
-  bool links_beside = false;         // the links' bounce-back beside the bulk kernel
+  bool links_beside = false;         // asked for the links alone: the same schedule
   bool unfused_dem = false;          // DEM substeps as separate launches even where the fused kernel applies
   bool cover_uncover = false;        // covered/uncovered-node momentum joins the hydrodynamic sums
   // blocks of the box kernels, sized per particle: device offsets (particle
@@ -146,8 +146,7 @@ struct mi_delbm {
   mi_status phase_refill(cudaStream_t st);
   mi_status phase_near();
   mi_status phase_bulk();
-  mi_status phase_links_ibb(cudaStream_t st);
-  mi_status phase_boundary();
+  mi_status phase_boundary(bool near);
   mi_status phase_boundary_beside(cudaStream_t st);
   mi_status phase_scatter_boundary();
   mi_status phase_swap();

@@ -166,9 +166,12 @@ __device__ __forceinline__ void collide_store(float (&h)[19], typename Store<ST>
 // own opposite population at a wall) before one load per direction, so all 19
 // loads are in flight together: with a branch per direction they were waited
 // for one after another, and every warp that holds a row's end paid for it.
+// Directions i with bit opp(i) of `own` set take the node's own opposite
+// population too (links into a solid).
 template <int ST>
 __device__ __forceinline__ void pull_node(const typename Store<ST>::T* __restrict__ A, const LatticeGeom& g,
-                                          const CollideParams& P, int x, int y, int z, long long c, float (&h)[19]) {
+                                          const CollideParams& P, int x, int y, int z, long long c, float (&h)[19],
+                                          uint32_t own = 0u) {
   const int nxy = g.nx * g.ny;
   // per axis: source offset and wall flag for e = +1 (source below) and e = -1
   const bool lo[3] = {x == 0, y == 0, z == 0}, hi[3] = {x == g.nx - 1, y == g.ny - 1, z == g.nz - 1};
@@ -192,7 +195,7 @@ __device__ __forceinline__ void pull_node(const typename Store<ST>::T* __restric
     int off = 0;
 #pragma unroll
     for (int a = 0; a < 3; ++a) off += e[a] == 1 ? om[a] : (e[a] == -1 ? op[a] : 0);
-    const long long at = wall ? opp(i) * g.plane + c : i * g.plane + (c + off);
+    const long long at = wall || ((own >> opp(i)) & 1u) ? opp(i) * g.plane + c : i * g.plane + (c + off);
     h[i] = Store<ST>::dev(A + at, i);  // w_opp = w_i
     // halfway bounce-back: f_in,i(x) = f+_opp(i)(x) + 6 w_i rho0 e_i.u_wall; a
     // corner crossing is attributed to x, then y, then z
@@ -569,7 +572,7 @@ __global__ void __launch_bounds__(128) k_refill(BoundaryLaunch L) {
 // reached twice is written twice with the same values.
 // ---------------------------------------------------------------------------
 template <int ST, bool FORCE>
-__global__ void __launch_bounds__(128) k_near(BoundaryLaunch L) {
+__device__ __forceinline__ void near_nodes(const BoundaryLaunch& L) {
   using T = typename Store<ST>::T;
   const T* __restrict__ A = static_cast<const T*>(L.A);
   T* __restrict__ B = static_cast<T*>(L.B);
@@ -589,31 +592,37 @@ __global__ void __launch_bounds__(128) k_near(BoundaryLaunch L) {
   }
 }
 
+template <int ST, bool FORCE>
+__global__ void __launch_bounds__(128) k_near(BoundaryLaunch L) {
+  near_nodes<ST, FORCE>(L);
+}
+
 // ---------------------------------------------------------------------------
-// Boundary nodes (Sec. 2.3.2) in two kernels.
+// Boundary nodes (Sec. 2.3.2), 128 to a block: a thread per node pulls its
+// populations and forms its moments, a thread per link of the block's nodes the
+// bounce-back population, a thread per node collides and stores into f+(t+1).
 //
-// k_links_ibb, one thread per link (x_f, d): x_f a fluid boundary node,
-// x_f + e_d a solid node of particle p at wall fraction q.  The population
-// that would have streamed from the solid neighbour into x_f along
-// j = opp(d) is the paper's interpolated bounce-back (Eqs. eqneq1, eqneq2,
-// neqd):
+// A link (x_f, d) joins the node x_f to a solid node x_f + e_d of particle p at
+// wall fraction q.  The population that would have streamed from the solid
+// neighbour into x_f along j = opp(d) is the paper's interpolated bounce-back
+// (Eqs. eqneq1, eqneq2, neqd):
 //   G_j = f_eq,d(rho_f, u_d) + [f+_d(x_f) - f_eq,d(rho_f, u_f)] + 6 w_d rho0 (e_j . u_w)
 //   u_d = u*/3 + 2 u**/3 (piecewise in q), u_w = v_p + omega_p x (x_w - X_p)
-// (or the halfway rule f+_d + 6 w_d rho0 e_j.u_w in Ladd mode), kept per
-// link.  The Galilean-invariant momentum exchange of the link,
+// (or the halfway rule f+_d + 6 w_d rho0 e_j.u_w in Ladd mode).  The Galilean-
+// invariant momentum exchange of the link,
 //   dP = (e_d - u_w) f+_d - (e_j - u_w) G_j = e_d (2 w_d + h_d + h_G) - u_w (h_d - h_G),
 // and its torque about X_p are rounded to 2^-40 fixed point per link and
-// summed in integers (over the warp, then per block, then over the blocks):
-// the sums do not depend on the order in which links are visited.  It reads
-// f+(t) only (A, after the refill), so it may run beside the bulk kernel
-// (a schedule option); by default it runs after it.
+// summed in integers (over the warp, then by 64-bit atomics of whole warps): the
+// sums do not depend on the order in which links are visited.
 //
-// k_boundary, one thread per boundary node, for each direction j: pull
-// streaming where the source is fluid, halfway bounce-back where it is
-// outside the domain, the link's G_j where it is solid; then BGK collision,
-// written into f+(t+1).  Up to IBB_SHARED_PARTICLES particles the link kernel
-// leaves its momentum exchange as per-block sums, which this kernel adds into
-// the particles' sums first (no launch of its own).
+// Bound by the gathers: a link reads the 19 populations of the node behind its
+// own, a 32-byte sector each.  One kernel per link (38 gathers: its own node's
+// too) that kept G for a second kernel per node took 497 + 320 us for 0.82 M
+// nodes and 3.35 M links in FP32 (300 particles, 512^3) and 27 + 22 us for
+// three cobbles' 32 k nodes; together they take 569 us (474 in 16 bits) and 24
+// us.  (A thread per node that goes through its links in turn, with atomics of
+// its own where the particle changes, took 1200 us.)  The nodes around
+// uncovered ones (k_near) are recomputed by the same launch.
 //
 // A link is used only when every link of its node fitted into the link list
 // (an overflow, reported by the classification, leaves the node on halfway
@@ -649,116 +658,126 @@ __device__ __forceinline__ long long fixed_2m40(float v) {
   return ((long long)__float2int_rn(h) << 20) + (long long)ir;
 }
 
-}  // namespace
-
 // The link entries of node bi fit into the list (its links were written by
 // the classification of this step).
 __device__ __forceinline__ bool links_fit(uint32_t loff, uint32_t mask, unsigned cap_links) {
   return (unsigned long long)loff + (unsigned)__popc(mask) <= (unsigned long long)cap_links;
 }
 
-template <int ST, bool LADD, bool SHARED>
-__global__ void __launch_bounds__(256) k_links_ibb(BoundaryLaunch L) {
-  // the block's sums per particle (SHARED) as 64-bit integers in two 32-bit
-  // words (native 32-bit shared atomics, the carry of the low word added to
-  // the high word), else the global sums directly
-  __shared__ unsigned s_lo[SHARED ? 6 * IBB_SHARED_PARTICLES : 1], s_hi[SHARED ? 6 * IBB_SHARED_PARTICLES : 1];
+__device__ __forceinline__ void add_force(long long* facc, int p, int k, long long v) {
+  atomicAdd(reinterpret_cast<unsigned long long*>(facc + 6 * (size_t)p + k), (unsigned long long)v);
+}
+constexpr int BOUNDARY_THREADS = 128;
+}  // namespace
+
+template <int ST, bool FORCE, bool LADD>
+__global__ void __launch_bounds__(BOUNDARY_THREADS) k_boundary(BoundaryLaunch L) {
+  constexpr int N = BOUNDARY_THREADS;  // nodes of a block at a time
+  __shared__ float s_g[18][N];         // the links' G by direction and node
+  __shared__ float4 s_mom[N];          // rho_f, u_f
+  __shared__ int3 s_xyz[N];
+  __shared__ uint32_t s_mask[N], s_loff[N], s_cell[N];
+  __shared__ int s_incl[N];            // links of the nodes up to this one
+  __shared__ int s_warp[N / 32];
   using T = typename Store<ST>::T;
   const T* __restrict__ A = static_cast<const T*>(L.A);
+  T* __restrict__ B = static_cast<T*>(L.B);
+  const LatticeGeom& g = L.pl.g;
   const ParticleLaunch& pl = L.pl;
-  const LatticeGeom& g = pl.g;
-  const unsigned nl = min(pl.ctr->n_links, pl.cap_links);
   const unsigned nbc = min(pl.ctr->n_bc, pl.cap_bc);
+  const int t = (int)threadIdx.x, lane = t & 31, w = t >> 5;
   const float rho0 = L.p.rho0;
-  const unsigned lane = threadIdx.x & 31u;
-  const unsigned stride = gridDim.x * blockDim.x;
-  const int n6 = 6 * pl.np;
-  if constexpr (SHARED) {
-    for (int k = threadIdx.x; k < n6; k += blockDim.x) s_lo[k] = s_hi[k] = 0u;
-    __syncthreads();
-  }
-  const auto flush = [&](int q, const long long* w) {
-    for (int k = 0; k < 6; ++k) {
-      if constexpr (SHARED) {
-        // (hi, lo) += w modulo 2^64: every wrap of the low word is seen by
-        // exactly the addition that made it, which carries it into the high word
-        const unsigned long long u = (unsigned long long)w[k];
-        const unsigned lo = (unsigned)u, old = atomicAdd(&s_lo[6 * q + k], lo);
-        const unsigned hi = (unsigned)(u >> 32) + (old + lo < old ? 1u : 0u);
-        if (hi) atomicAdd(&s_hi[6 * q + k], hi);
-      } else {
-        atomicAdd(reinterpret_cast<unsigned long long*>(pl.facc + 6 * q + k), (unsigned long long)w[k]);
-      }
-    }
-  };
-  int pacc = -1;  // lane 0: particle of the running fixed-point sums
-  long long iacc[6] = {0, 0, 0, 0, 0, 0};
-  // whole warps step together (the sums below are warp collectives)
-  for (unsigned base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < nl; base += stride) {
-    const unsigned l = base + lane;
-    int p = -1;
-    float v[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-    const unsigned bi = l < nl ? pl.link_bc[l] : 0xffffffffu;
-    uint32_t loff = 0, mask = 0;
-    if (bi < nbc) {
-      loff = pl.bc_loff[bi];
+  if (L.near) near_nodes<ST, FORCE>(L);
+  int pacc = -1;  // the particle of the warp's running fixed-point sums, component k in lane k
+  long long acc = 0;
+  for (unsigned first = blockIdx.x * N; first < nbc; first += gridDim.x * N) {
+    // ---- a thread per node: its pull and its moments ----
+    const unsigned bi = first + (unsigned)t;
+    const bool node = bi < nbc;
+    long long c = 0;
+    uint32_t mask = 0;
+    int m = 0;
+    float h[19];
+    if (node) {
+      c = pl.bc_cell[bi];
       mask = pl.bc_mask[bi];
-    }
-    // an entry of this step: inside the range of the node it names, which fitted
-    if (bi < nbc && l >= loff && l - loff < (unsigned)__popc(mask) && links_fit(loff, mask, pl.cap_links)) {
-      const long long c = pl.bc_cell[bi];
+      const uint32_t loff = pl.bc_loff[bi];
+      m = links_fit(loff, mask, pl.cap_links) ? __popc(mask) : 0;
       int x, y, z;
       coords(c, g, x, y, z);
-      const int d = pl.link_dir[l];
-      const int j = lopp(d);
-      const int ed[3] = {lex(d), ley(d), lez(d)};
-      const bool inside = (g.periodic[0] || (unsigned)(x + ed[0]) < (unsigned)g.nx) &&
-                          (g.periodic[1] || (unsigned)(y + ed[1]) < (unsigned)g.ny) &&
-                          (g.periodic[2] || (unsigned)(z + ed[2]) < (unsigned)g.nz);
-      if (inside) {
-        // own post-collision populations and moments (rho_f, u_f)
-        float h[19];
+      pull_node<ST>(A, g, L.p, x, y, z, c, h, mask);
+      if (!LADD) {
+        float rho, u[3];
+        moments_at<ST>(A, g.plane, c, rho, u);
+        s_mom[t] = make_float4(rho, u[0], u[1], u[2]);
+      }
+      s_xyz[t] = make_int3(x, y, z);
+      s_mask[t] = mask;
+      s_loff[t] = loff;
+      s_cell[t] = (uint32_t)c;
+    }
+    int incl = m;
 #pragma unroll
-        for (int i = 0; i < 19; ++i) h[i] = Store<ST>::dev(A + i * g.plane + c, i);
-        float dr = 0.f, j0 = 0.f, j1 = 0.f, j2 = 0.f;
+    for (int k = 1; k < 32; k <<= 1) {
+      const int v = __shfl_up_sync(FULLW, incl, k);
+      if (lane >= k) incl += v;
+    }
+    if (lane == 31) s_warp[w] = incl;
+    __syncthreads();
+    int total = 0;
 #pragma unroll
-        for (int i = 0; i < 19; ++i) {
-          dr += h[i];
-          j0 += cx(i) * h[i];
-          j1 += cy(i) * h[i];
-          j2 += cz(i) * h[i];
-        }
-        float hopp = h[0];  // f+_d(x_f) - w_d
+    for (int k = 0; k < N / 32; ++k) {
+      if (k < w) incl += s_warp[k];
+      total += s_warp[k];
+    }
+    s_incl[t] = incl;
+    __syncthreads();
+    // ---- a thread per link of the block's nodes ----
+    for (int base = 32 * w; base < total; base += N) {
+      const int i = base + lane;
+      int p = -1;
+      float v[6];
+      if (i < total) {
+        int s = 0;  // its node: the first with more than i links up to it
 #pragma unroll
-        for (int i = 1; i < 19; ++i) hopp = i == d ? h[i] : hopp;
-        const float rho_f = 1.0f + dr;
-        const float irho_f = 1.0f / rho_f;
-        const float uf[3] = {j0 * irho_f, j1 * irho_f, j2 * irho_f};
+        for (int k = N / 2; k > 0; k >>= 1)
+          if (s_incl[s + k - 1] <= i) s += k;
+        const uint32_t ms = s_mask[s];
+        const unsigned l = s_loff[s] + (unsigned)(i - (s_incl[s] - __popc(ms)));
+        const long long cs = s_cell[s];
+        const int3 at = s_xyz[s];
+        const int d = pl.link_dir[l];
         p = (int)pl.link_p[l];
-        const DevParticle& P = pl.P[p];
         const float q = LADD ? 0.5f : pl.link_q[l];
-        const float wj = lw(j);
+        const int ed[3] = {lex(d), ley(d), lez(d)};
+        const float wd = lw(d);
+        const float hopp = Store<ST>::dev_at(A + d * g.plane + cs, wd);  // f+_d(x_f) - w_d
+        // u at the second fluid node x_f - e_d when it is fluid, else u_f
+        float rho_f = 1.0f, uf[3] = {0.f, 0.f, 0.f}, uff[3] = {0.f, 0.f, 0.f};
+        if (!LADD) {
+          const float4 mom = s_mom[s];
+          rho_f = mom.x;
+          uff[0] = uf[0] = mom.y;
+          uff[1] = uf[1] = mom.z;
+          uff[2] = uf[2] = mom.w;
+          long long ff;
+          if (!((ms >> lopp(d)) & 1u) && nbr_wrap(at.x, at.y, at.z, -ed[0], -ed[1], -ed[2], g, ff)) {
+            float rr;
+            moments_at<ST>(A, g.plane, ff, rr, uff);
+          }
+        }
         // wall point relative to the particle position: x - X = (x - floor X) - frac X,
         // the integer part exact and the fraction rounded once to FP32
-        const float r0 = ((float)(x - P.pos_i[0]) - P.pos_fr[0]) + q * ed[0];
-        const float r1 = ((float)(y - P.pos_i[1]) - P.pos_fr[1]) + q * ed[1];
-        const float r2 = ((float)(z - P.pos_i[2]) - P.pos_fr[2]) + q * ed[2];
+        const DevParticle& P = pl.P[p];
+        const float r0 = ((float)(at.x - P.pos_i[0]) - P.pos_fr[0]) + q * ed[0];
+        const float r1 = ((float)(at.y - P.pos_i[1]) - P.pos_fr[1]) + q * ed[1];
+        const float r2 = ((float)(at.z - P.pos_i[2]) - P.pos_fr[2]) + q * ed[2];
         float uw[3];
         uw[0] = P.velf[0] + (P.omegaf[1] * r2 - P.omegaf[2] * r1);
         uw[1] = P.velf[1] + (P.omegaf[2] * r0 - P.omegaf[0] * r2);
         uw[2] = P.velf[2] + (P.omegaf[0] * r1 - P.omegaf[1] * r0);
-        const float wall = 6.0f * wj * rho0 * (-ed[0] * uw[0] - ed[1] * uw[1] - ed[2] * uw[2]);
-        float G;
-        if (LADD) {
-          G = hopp + wall;
-        } else {
-          // u at the second fluid node x_f - e_d when it is fluid, else u_f
-          float uff[3] = {uf[0], uf[1], uf[2]};
-          long long ff;
-          if (nbr_wrap(x, y, z, -ed[0], -ed[1], -ed[2], g, ff) && pl.owner_cur[ff] == OWNER_NONE) {
-            float rr;
-            moments_at<ST>(A, g.plane, ff, rr, uff);
-          }
+        float G = hopp + 6.0f * wd * rho0 * (-ed[0] * uw[0] - ed[1] * uw[1] - ed[2] * uw[2]);
+        if (!LADD) {
           float ud[3];
           const float i1q = 1.0f / (1.0f + q), iq = 1.0f / q;
           const float a1 = (1.0f - q) * i1q, a2 = 2.0f * q * i1q;
@@ -772,10 +791,13 @@ __global__ void __launch_bounds__(256) k_links_ibb(BoundaryLaunch L) {
           const float euf = ed[0] * uf[0] + ed[1] * uf[1] + ed[2] * uf[2];
           const float ud2 = ud[0] * ud[0] + ud[1] * ud[1] + ud[2] * ud[2];
           const float uf2 = uf[0] * uf[0] + uf[1] * uf[1] + uf[2] * uf[2];
-          G = hopp + wj * rho_f * (3.0f * (eud - euf) + 4.5f * (eud * eud - euf * euf) - 1.5f * (ud2 - uf2)) + wall;
+          G += wd * rho_f * (3.0f * (eud - euf) + 4.5f * (eud * eud - euf * euf) - 1.5f * (ud2 - uf2));
         }
-        pl.link_g[l] = G;
-        const float s2 = 2.0f * wj + hopp + G, dl = hopp - G;
+        s_g[d - 1][s] = G;
+        // momentum exchange, rounded per link (v * 2^40 is exact in FP32 and the
+        // rounding is to nearest even: odd-symmetric, so opposite links of a
+        // closed body cancel exactly)
+        const float s2 = 2.0f * wd + hopp + G, dl = hopp - G;
         v[0] = ed[0] * s2 - uw[0] * dl;
         v[1] = ed[1] * s2 - uw[1] * dl;
         v[2] = ed[2] * s2 - uw[2] * dl;
@@ -783,130 +805,40 @@ __global__ void __launch_bounds__(256) k_links_ibb(BoundaryLaunch L) {
         v[4] = r2 * v[0] - r0 * v[2];
         v[5] = r0 * v[1] - r1 * v[0];
       }
-    }
-    // momentum exchange: each link's contribution rounded to 2^-40 fixed point
-    // in its own lane (v * 2^40 is exact in FP32 and the rounding is to nearest
-    // even: odd-symmetric, so opposite links of a closed body cancel exactly),
-    // summed over the warp in integers and kept by lane 0 while the particle
-    // does not change
-    if (__any_sync(FULLW, p >= 0)) {
-      const int pmin = __reduce_min_sync(FULLW, p >= 0 ? p : 0x7fffffff);
-      const bool single = __all_sync(FULLW, p < 0 || p == pmin);
-      long long iv[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) iv[k] = p >= 0 ? fixed_2m40(v[k]) : 0LL;
-      if (single) {
-#pragma unroll
-        for (int k = 0; k < 6; ++k) iv[k] = warp_sum_fixed(iv[k]);
-        if (lane == 0) {
-          if (pacc != pmin) {
-            if (pacc >= 0) flush(pacc, iacc);
-            pacc = pmin;
-            for (int k = 0; k < 6; ++k) iacc[k] = 0;
-          }
-          for (int k = 0; k < 6; ++k) iacc[k] += iv[k];
+      // the links' sums over the warp, particle by particle (nearly always one)
+      for (unsigned left = __ballot_sync(FULLW, p >= 0); left;) {
+        const int ps = __shfl_sync(FULLW, p, __ffs(left) - 1);
+        const bool mine = p == ps;
+        left &= ~__ballot_sync(FULLW, mine);
+        if (ps != pacc) {
+          if (lane < 6 && pacc >= 0) add_force(pl.facc, pacc, lane, acc);
+          pacc = ps;
+          acc = 0;
         }
-      } else if (p >= 0) {  // links to several particles: per-link atomics
-        flush(p, iv);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+          const long long sum = warp_sum_fixed(mine ? fixed_2m40(v[k]) : 0);
+          if (lane == k) acc += sum;
+        }
       }
     }
-  }
-  if (lane == 0 && pacc >= 0) flush(pacc, iacc);
-  if constexpr (SHARED) {
     __syncthreads();
-    long long* out = L.part + (size_t)blockIdx.x * n6;
-    for (int k = threadIdx.x; k < n6; k += blockDim.x)
-      out[k] = (long long)(((unsigned long long)s_hi[k] << 32) | (unsigned long long)s_lo[k]);
-  }
-}
-
-template <int ST, bool FORCE>
-__global__ void __launch_bounds__(256) k_boundary(BoundaryLaunch L) {
-  using T = typename Store<ST>::T;
-  const T* __restrict__ A = static_cast<const T*>(L.A);
-  T* __restrict__ B = static_cast<T*>(L.B);
-  const LatticeGeom& g = L.pl.g;
-  const ParticleLaunch& pl = L.pl;
-  const unsigned nbc = min(pl.ctr->n_bc, pl.cap_bc);
-  const float om = L.p.omega;
-  if (L.part && pl.np <= IBB_SHARED_PARTICLES) {
-    // the link kernel's per-block momentum-exchange sums into the particles'
-    // fixed-point sums (it ran before this kernel), a warp per component
-    const int n6 = 6 * pl.np;
-    const unsigned lane = threadIdx.x & 31u;
-    for (unsigned k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; k < (unsigned)n6;
-         k += (gridDim.x * blockDim.x) >> 5) {
-      long long v = 0;
-      for (int b = (int)lane; b < L.part_blocks; b += 32) v += L.part[(size_t)b * n6 + k];
-      v = warp_sum_fixed(v);
-      if (lane == 0 && v) atomicAdd(reinterpret_cast<unsigned long long*>(pl.facc + k), (unsigned long long)v);
-    }
-  }
-  for (unsigned bi = blockIdx.x * blockDim.x + threadIdx.x; bi < nbc; bi += gridDim.x * blockDim.x) {
-    const long long c = pl.bc_cell[bi];
-    const uint32_t mask = pl.bc_mask[bi];
-    const uint32_t loff = pl.bc_loff[bi];
-    const bool fit = links_fit(loff, mask, pl.cap_links);
-    int x, y, z;
-    coords(c, g, x, y, z);
-    float h[19];
+    // ---- a thread per node: collision and store ----
+    if (node) {
+      if (m)
 #pragma unroll
-    for (int j = 0; j < 19; ++j) {
-      const int d = opp(j);  // link direction of j (towards the source node)
-      int sx = x - cx(j), sy = y - cy(j), sz = z - cz(j);
-      int face = -1;  // a corner crossing is attributed to x, then y, then z
-      if (sz < 0) { if (g.periodic[2]) sz += g.nz; else face = 4; }
-      else if (sz >= g.nz) { if (g.periodic[2]) sz -= g.nz; else face = 5; }
-      if (sy < 0) { if (g.periodic[1]) sy += g.ny; else face = 2; }
-      else if (sy >= g.ny) { if (g.periodic[1]) sy -= g.ny; else face = 3; }
-      if (sx < 0) { if (g.periodic[0]) sx += g.nx; else face = 0; }
-      else if (sx >= g.nx) { if (g.periodic[0]) sx -= g.nx; else face = 1; }
-      if (face >= 0) {
-        h[j] = Store<ST>::dev(A + d * g.plane + c, d) + L.p.bb_wall[face][j];
-      } else if (j == 0 || !((mask >> d) & 1u)) {
-        h[j] = Store<ST>::dev(A + j * g.plane + (sx + (long long)g.nx * (sy + (long long)g.ny * sz)), j);
-      } else if (fit) {
-        h[j] = pl.link_g[loff + __popc(mask & ((1u << d) - 1u))];
-      } else {
-        h[j] = Store<ST>::dev(A + d * g.plane + c, d);
+        for (int j = 1; j < 19; ++j)
+          if ((mask >> opp(j)) & 1u) h[j] = s_g[opp(j) - 1][t];
+      collide_inplace<FORCE>(h, L.p);
+#pragma unroll
+      for (int j = 0; j < 19; ++j) {
+        if (L.tmp) Store<ST>::put(static_cast<T*>(L.tmp) + 19 * (size_t)bi + j, j, h[j]);
+        else Store<ST>::put(B + j * g.plane + c, j, h[j]);
       }
     }
-    // BGK collision of the node
-    float drho = 0.f, j0 = 0.f, j1 = 0.f, j2 = 0.f;
-#pragma unroll
-    for (int i = 0; i < 19; ++i) {
-      drho += h[i];
-      j0 += cx(i) * h[i];
-      j1 += cy(i) * h[i];
-      j2 += cz(i) * h[i];
-    }
-    const float rho = 1.0f + drho;
-    const float irho = 1.0f / rho;
-    float u0, u1, u2;
-    if (FORCE) {
-      u0 = (j0 + 0.5f * L.p.force[0]) * irho;
-      u1 = (j1 + 0.5f * L.p.force[1]) * irho;
-      u2 = (j2 + 0.5f * L.p.force[2]) * irho;
-    } else {
-      u0 = j0 * irho;
-      u1 = j1 * irho;
-      u2 = j2 * irho;
-    }
-    const float usq15 = 1.5f * (u0 * u0 + u1 * u1 + u2 * u2);
-#pragma unroll
-    for (int j = 0; j < 19; ++j) {
-      const float eu = cx(j) * u0 + cy(j) * u1 + cz(j) * u2;
-      const float feq_dev = wq(j) * (drho + rho * (3.0f * eu + 4.5f * eu * eu - usq15));
-      float hp = h[j] + om * (feq_dev - h[j]);
-      if (FORCE) {
-        const float eF = cx(j) * L.p.force[0] + cy(j) * L.p.force[1] + cz(j) * L.p.force[2];
-        const float uF = u0 * L.p.force[0] + u1 * L.p.force[1] + u2 * L.p.force[2];
-        hp += (1.0f - 0.5f * om) * wq(j) * (3.0f * (eF - uF) + 9.0f * eu * eF);
-      }
-      if (L.tmp) Store<ST>::put(static_cast<T*>(L.tmp) + 19 * (size_t)bi + j, j, hp);
-      else Store<ST>::put(B + j * g.plane + c, j, hp);
-    }
+    __syncthreads();  // the shared arrays are free for the next nodes
   }
+  if (lane < 6 && pacc >= 0) add_force(pl.facc, pacc, lane, acc);
 }
 
 // A list kernel's grid: the tuned block count, but no more blocks than the
@@ -935,30 +867,6 @@ cudaError_t launch_refill(const BoundaryLaunch& L, cudaStream_t s) {
 }
 
 template <int ST>
-static cudaError_t launch_links_ibb_st(const BoundaryLaunch& L, cudaStream_t s) {
-  const bool ladd = L.bb_mode == MI_BB_LADD;
-  if (L.part && L.pl.np <= IBB_SHARED_PARTICLES) {
-    if (ladd) k_links_ibb<ST, true, true><<<L.part_blocks, 256, 0, s>>>(L);
-    else k_links_ibb<ST, false, true><<<L.part_blocks, 256, 0, s>>>(L);
-  } else {
-    const int grid = list_grid(L.grid, L.pl.cap_links, 256);
-    if (ladd) k_links_ibb<ST, true, false><<<grid, 256, 0, s>>>(L);
-    else k_links_ibb<ST, false, false><<<grid, 256, 0, s>>>(L);
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_links_ibb(const BoundaryLaunch& L, cudaStream_t s) {
-  if (L.pl.np == 0) return cudaSuccess;
-  switch (L.storage) {
-    case MI_STORE_F32: return launch_links_ibb_st<MI_STORE_F32>(L, s);
-    case MI_STORE_F16_DEV: return launch_links_ibb_st<MI_STORE_F16_DEV>(L, s);
-    case MI_STORE_BF16_DEV: return launch_links_ibb_st<MI_STORE_BF16_DEV>(L, s);
-  }
-  return cudaErrorInvalidValue;
-}
-
-template <int ST>
 static cudaError_t launch_near_st(const BoundaryLaunch& L, cudaStream_t s) {
   // a step uncovers a small part of what the list can hold
   const int grid = list_grid(L.grid, 19ull * ((L.pl.cap_new + 15ull) / 16ull), 128);
@@ -977,11 +885,11 @@ cudaError_t launch_near(const BoundaryLaunch& L, cudaStream_t s) {
   return cudaErrorInvalidValue;
 }
 
-template <int ST>
+template <int ST, bool FORCE>
 static cudaError_t launch_boundary_st(const BoundaryLaunch& L, cudaStream_t s) {
-  const int grid = list_grid(L.grid, L.pl.cap_bc, 256);
-  if (L.forcing) k_boundary<ST, true><<<grid, 256, 0, s>>>(L);
-  else k_boundary<ST, false><<<grid, 256, 0, s>>>(L);
+  const int grid = list_grid(L.grid, L.pl.cap_bc, BOUNDARY_THREADS);
+  if (L.bb_mode == MI_BB_LADD) k_boundary<ST, FORCE, true><<<grid, BOUNDARY_THREADS, 0, s>>>(L);
+  else k_boundary<ST, FORCE, false><<<grid, BOUNDARY_THREADS, 0, s>>>(L);
   return cudaGetLastError();
 }
 
@@ -1007,9 +915,9 @@ cudaError_t launch_scatter_boundary(const BoundaryLaunch& L, cudaStream_t s) {
 cudaError_t launch_boundary(const BoundaryLaunch& L, cudaStream_t s) {
   if (L.pl.np == 0) return cudaSuccess;
   switch (L.storage) {
-    case MI_STORE_F32: return launch_boundary_st<MI_STORE_F32>(L, s);
-    case MI_STORE_F16_DEV: return launch_boundary_st<MI_STORE_F16_DEV>(L, s);
-    case MI_STORE_BF16_DEV: return launch_boundary_st<MI_STORE_BF16_DEV>(L, s);
+    case MI_STORE_F32: return L.forcing ? launch_boundary_st<MI_STORE_F32, true>(L, s) : launch_boundary_st<MI_STORE_F32, false>(L, s);
+    case MI_STORE_F16_DEV: return L.forcing ? launch_boundary_st<MI_STORE_F16_DEV, true>(L, s) : launch_boundary_st<MI_STORE_F16_DEV, false>(L, s);
+    case MI_STORE_BF16_DEV: return L.forcing ? launch_boundary_st<MI_STORE_BF16_DEV, true>(L, s) : launch_boundary_st<MI_STORE_BF16_DEV, false>(L, s);
   }
   return cudaErrorInvalidValue;
 }

@@ -464,12 +464,21 @@ __global__ void __launch_bounds__(32 * CLS_WARPS) k_classify(ParticleLaunch L) {
   BoundaryKeep& K = keep[threadIdx.x >> 5];
   int kept = 0;
   const LatticeGeom& g = L.g;
-  const unsigned rows = (unsigned)r.n[1] * (unsigned)r.n[2];
+  // the rows in tiles of 4 x 4 (y, z), which the warps take in turn (parts of
+  // one when there are more warps): a warp's nodes then lie together on the
+  // surface, and the gathers of the kernels that walk the lists find each
+  // other's sectors in the caches
+  const unsigned ty = ((unsigned)r.n[1] + 3u) / 4u, slots = 16u * ty * (((unsigned)r.n[2] + 3u) / 4u);
   const unsigned wid = (bb.b * blockDim.x + threadIdx.x) >> 5, nw = (bb.nb * blockDim.x) >> 5;
-  for (unsigned row = wid; row < rows; row += nw) {
-    const unsigned zi = row / (unsigned)r.n[1];
-    const int y = r.lo[1] + (int)(row - zi * (unsigned)r.n[1]);
-    const int z = r.lo[2] + (int)zi;
+  const unsigned each = min(16u, (slots + nw - 1u) / nw);
+  for (unsigned n = 0, slot = wid * each; slot < slots;) {
+    const unsigned at = slot;
+    if (++n % each) ++slot;
+    else slot += (nw - 1u) * each + 1u;
+    const unsigned tile = at >> 4, tz = tile / ty;
+    const int yi = (int)(4u * (tile - tz * ty) + (at & 3u)), zi = (int)(4u * tz + ((at >> 2) & 3u));
+    if (yi >= r.n[1] || zi >= r.n[2]) continue;
+    const int y = r.lo[1] + yi, z = r.lo[2] + zi;
     int xa = INT_MAX, xb = INT_MIN;
     {
       const float hc = rc2 - ((y - cc1) * (y - cc1) + (z - cc2) * (z - cc2));

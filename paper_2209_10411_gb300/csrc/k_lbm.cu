@@ -572,13 +572,13 @@ __global__ void __launch_bounds__(128) k_refill(BoundaryLaunch L) {
 // reached twice is written twice with the same values.
 // ---------------------------------------------------------------------------
 template <int ST, bool FORCE>
-__device__ __forceinline__ void near_nodes(const BoundaryLaunch& L) {
+__device__ __forceinline__ void near_nodes(const BoundaryLaunch& L, unsigned block, unsigned blocks) {
   using T = typename Store<ST>::T;
   const T* __restrict__ A = static_cast<const T*>(L.A);
   T* __restrict__ B = static_cast<T*>(L.B);
   const LatticeGeom& g = L.pl.g;
   const unsigned nn = min(L.pl.ctr->n_new, L.pl.cap_new);
-  for (unsigned t = blockIdx.x * blockDim.x + threadIdx.x; t < nn * 19u; t += gridDim.x * blockDim.x) {
+  for (unsigned t = block * blockDim.x + threadIdx.x; t < nn * 19u; t += blocks * blockDim.x) {
     const unsigned k = t / 19u;
     const int d = (int)(t - 19u * k);
     int x, y, z;
@@ -594,7 +594,7 @@ __device__ __forceinline__ void near_nodes(const BoundaryLaunch& L) {
 
 template <int ST, bool FORCE>
 __global__ void __launch_bounds__(128) k_near(BoundaryLaunch L) {
-  near_nodes<ST, FORCE>(L);
+  near_nodes<ST, FORCE>(L, blockIdx.x, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -687,10 +687,15 @@ __global__ void __launch_bounds__(BOUNDARY_THREADS) k_boundary(BoundaryLaunch L)
   const unsigned nbc = min(pl.ctr->n_bc, pl.cap_bc);
   const int t = (int)threadIdx.x, lane = t & 31, w = t >> 5;
   const float rho0 = L.p.rho0;
-  if (L.near) near_nodes<ST, FORCE>(L);
+  // the last near_blocks blocks take the nodes around uncovered ones
+  const unsigned blocks = gridDim.x - (unsigned)L.near_blocks;
+  if (blockIdx.x >= blocks) {
+    near_nodes<ST, FORCE>(L, blockIdx.x - blocks, (unsigned)L.near_blocks);
+    return;
+  }
   int pacc = -1;  // the particle of the warp's running fixed-point sums, component k in lane k
   long long acc = 0;
-  for (unsigned first = blockIdx.x * N; first < nbc; first += gridDim.x * N) {
+  for (unsigned first = blockIdx.x * N; first < nbc; first += blocks * N) {
     // ---- a thread per node: its pull and its moments ----
     const unsigned bi = first + (unsigned)t;
     const bool node = bi < nbc;
@@ -866,10 +871,15 @@ cudaError_t launch_refill(const BoundaryLaunch& L, cudaStream_t s) {
   return cudaErrorInvalidValue;
 }
 
+// blocks of the nodes around uncovered ones: a step uncovers a small part of
+// what the list can hold
+static int near_grid(const BoundaryLaunch& L) {
+  return list_grid(L.grid, 19ull * ((L.pl.cap_new + 15ull) / 16ull), BOUNDARY_THREADS);
+}
+
 template <int ST>
 static cudaError_t launch_near_st(const BoundaryLaunch& L, cudaStream_t s) {
-  // a step uncovers a small part of what the list can hold
-  const int grid = list_grid(L.grid, 19ull * ((L.pl.cap_new + 15ull) / 16ull), 128);
+  const int grid = near_grid(L);
   if (L.forcing) k_near<ST, true><<<grid, 128, 0, s>>>(L);
   else k_near<ST, false><<<grid, 128, 0, s>>>(L);
   return cudaGetLastError();
@@ -887,9 +897,11 @@ cudaError_t launch_near(const BoundaryLaunch& L, cudaStream_t s) {
 
 template <int ST, bool FORCE>
 static cudaError_t launch_boundary_st(const BoundaryLaunch& L, cudaStream_t s) {
-  const int grid = list_grid(L.grid, L.pl.cap_bc, BOUNDARY_THREADS);
-  if (L.bb_mode == MI_BB_LADD) k_boundary<ST, FORCE, true><<<grid, BOUNDARY_THREADS, 0, s>>>(L);
-  else k_boundary<ST, FORCE, false><<<grid, BOUNDARY_THREADS, 0, s>>>(L);
+  BoundaryLaunch M = L;
+  M.near_blocks = L.near ? near_grid(L) : 0;
+  const int grid = list_grid(L.grid, L.pl.cap_bc, BOUNDARY_THREADS) + M.near_blocks;
+  if (L.bb_mode == MI_BB_LADD) k_boundary<ST, FORCE, true><<<grid, BOUNDARY_THREADS, 0, s>>>(M);
+  else k_boundary<ST, FORCE, false><<<grid, BOUNDARY_THREADS, 0, s>>>(M);
   return cudaGetLastError();
 }
 

@@ -843,16 +843,17 @@ cudaError_t launch_links_q(const ParticleLaunch& L, int grid, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------
-// Rigid-body update, four lanes of a warp per particle (rigid_dev.cuh).
+// Rigid-body update, eight lanes of a warp per particle (rigid_dev.cuh).
 // ---------------------------------------------------------------------------
-__global__ void k_integrate(IntegrateLaunch L) {
-  const int p = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-  if (p < L.np) integrate_particle_lanes(L, p, threadIdx.x & 31);
+__global__ void __launch_bounds__(128) k_integrate(IntegrateLaunch L) {
+  const int first = (int)blockIdx.x * (128 / RIGID_LANES);
+  integrate_particles(L, first, min(L.np, first + 128 / RIGID_LANES));
 }
 
 cudaError_t launch_integrate(const IntegrateLaunch& L, cudaStream_t s) {
   if (L.np == 0) return cudaSuccess;
-  k_integrate<<<(L.np + 3) / 4, 128, 0, s>>>(L);
+  const int per = 128 / RIGID_LANES;
+  k_integrate<<<(L.np + per - 1) / per, 128, 0, s>>>(L);
   return cudaGetLastError();
 }
 

@@ -244,7 +244,8 @@ struct BoundaryLaunch {
   int bb_mode;
   int grid;
   void* tmp;  // when set, k_boundary writes node k's 19 values to tmp[19 k ..] instead of B
-  bool near;  // k_boundary also recomputes the nodes around uncovered ones (k_near)
+  bool near;  // k_boundary also recomputes the nodes around uncovered ones (k_near),
+  int near_blocks = 0;  // in this many further blocks (set by the launch)
 };
 cudaError_t launch_refill(const BoundaryLaunch& L, cudaStream_t s);
 // The boundary nodes: bounce-back of their links, momentum exchange, stream and collide.

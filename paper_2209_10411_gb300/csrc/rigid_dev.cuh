@@ -8,98 +8,181 @@ namespace mi {
 
 // FP64: semi-implicit Euler for the velocity, Euler's equations in the body
 // frame, exponential map for the orientation; buoyancy-corrected gravity
-// (m - rho0 V) g.  FP64 instructions issue at a small fraction of the FP32
-// rate on this part and the update of one particle is one long dependent
-// chain, so four lanes of a warp share it: lane a < 3 owns component a of
-// every 3-vector (its column of R for R^T v, its row for R v), lane c < 4
-// component c of the quaternion product, and the few values a lane needs
-// from the others come by shuffles; scalars (norms, the half-angle series)
-// are computed alike in the four lanes.  Rotations use
-// R = (w^2 - v.v) I + 2 v v^T + 2 w [v]x of the unit quaternion (w, v);
-// sin(a)/a and cos(a) of the half rotation angle a come from their Taylor
-// series when a <= 1/64 (terms to a^8: the first omitted term is below 2^-53
-// relative there), from the library functions otherwise.
-// ---------------------------------------------------------------------------
+// (m - rho0 V) g.
+//
+// Bound by FP64 issue: a warp's FP64 instruction takes the pipe for about 64
+// cycles on this part, for one lane as for 32, and the update is one dependent
+// chain, so its time is its number of FP64 instructions.  Eight lanes of a warp
+// share a particle (four particles to a warp) and every instruction does as
+// many of its values as have the same form; values pass by shuffles, which
+// cost next to nothing beside.  Lane c < 3 of either four owns component c of
+// every 3-vector and of the quaternion's vector part, lane 3 its scalar; the
+// first four rotate the angular velocity and sum the cosine's series while the
+// second rotate the torque and sum the sine's.  The products of the
+// quaternion's components serve the new rotation's rows (angular velocity to
+// the world frame) and the next substep's columns.  47 FP64 instructions a
+// substep: two particles' 100 substeps in one CTA take 227 us
+// (367 with four lanes a particle, 100 instructions, no shared products).
+//
+// Rotations use R = 2 (v v^T + w [v]x + (w^2 - 1/2) I) of the unit quaternion
+// (w, v); sin(a)/a and cos(a) of the half rotation angle a come from their
+// Taylor series when a <= 1/64 (terms to a^8: the first omitted term is below
+// 2^-53 relative there), from the library functions otherwise.  1/|q| of a
+// quaternion whose squared norm n is within 2^-26 of 1 (every product made
+// here) is 1.5 - n / 2, off by 3/8 (n - 1)^2 < 2^-53; one that is handed in is
+// normalised when n is more than 64 ulps from 1.
+//
+// Every operation is written out as a single rounding, so the substep kernel
+// and the fused loop give the same bits whatever the compiler hoists.
 __device__ __forceinline__ double pick3(int a, double x, double y, double z) { return a == 0 ? x : (a == 1 ? y : z); }
 
-// Lanes 0-3 of a warp update particle p (the other lanes return at once).
-__device__ __forceinline__ void integrate_particle_lanes(const IntegrateLaunch& L, int p, int lane) {
-  if (lane >= 4) return;
-  constexpr unsigned M4 = 0xfu;
-  DevParticle& P = L.P[p];
-  const int a = lane < 3 ? lane : 2;  // lane 3 repeats component z and stores no 3-vector
-  const int a1 = a == 2 ? 0 : a + 1, a2 = a == 0 ? 2 : a - 1;
-  // force and torque: fixed-point sums that other threads built with atomics, read past the L1
-  double F = (double)__ldcg(L.facc + 6 * p + a) * FIX_INV;
-  double T = (double)__ldcg(L.facc + 6 * p + 3 + a) * FIX_INV;
+// One lane's part of a particle.
+struct RigidLane {
+  int c, a, a1, a2;          // lane of the four; its component and the two after it (cyclic; lane 3 repeats 2)
+  bool second;               // of the second four
+  double dt, hdt, acc, dtm;  // dt, dt / 2, (F + (m - rho0 V) g)_a, dt / m
+  double T;                  // torque (world), component a
+  double I[3], Ii[3];        // rows a of the inertia tensor and its inverse
+  double pos, vel, om;       // component a
+  double q;                  // component a of the quaternion's vector part, or its scalar (lane 3)
+  double ca, cb, cc;         // half of R[a][a], R[a1][a], R[a2][a]
+};
+
+constexpr unsigned RIGID_FULL = 0xffffffffu;
+constexpr int RIGID_LANES = 8;
+__device__ __forceinline__ double quad(double v, int k) { return __shfl_sync(RIGID_FULL, v, k, 4); }
+__device__ __forceinline__ double dot3(double a0, double b0, double a1, double b1, double a2, double b2) {
+  return __fma_rn(a2, b2, __fma_rn(a1, b1, __dmul_rn(a0, b0)));
+}
+// the sum of the four lanes' squares, the same in each
+__device__ __forceinline__ double quad_norm2(double v) {
+  double s = __dmul_rn(v, v);
+  s = __dadd_rn(s, __shfl_xor_sync(RIGID_FULL, s, 1));
+  return __dadd_rn(s, __shfl_xor_sync(RIGID_FULL, s, 2));
+}
+// whether n lies within about `ulps` units in the last place of 1 (an integer comparison)
+__device__ __forceinline__ bool near_one(double n, long long ulps) {
+  const long long d = __double_as_longlong(n) - 0x3FF0000000000000LL;
+  return d < ulps && d > -2 * ulps;
+}
+
+// The half entries of row a (ra, rb, rc along a, a1, a2) and of column a (in S) of the rotation of S.q.
+__device__ __forceinline__ void rigid_rotation(RigidLane& S, double& rb, double& rc) {
+  const double x = quad(S.q, 0), y = quad(S.q, 1), z = quad(S.q, 2), w = quad(S.q, 3);
+  const double va = pick3(S.a, x, y, z), va1 = pick3(S.a1, x, y, z), va2 = pick3(S.a2, x, y, z);
+  S.ca = __fma_rn(va, va, __fma_rn(w, w, -0.5));
+  const double p1 = __dmul_rn(va, va1), p2 = __dmul_rn(w, va2), p3 = __dmul_rn(va, va2), p4 = __dmul_rn(w, va1);
+  S.cb = __dadd_rn(p1, p2);
+  S.cc = __dsub_rn(p3, p4);
+  rb = __dsub_rn(p1, p2);
+  rc = __dadd_rn(p3, p4);
+}
+
+// Particle p's lane (0..7).  The force sums were built with atomics by other
+// threads: read past the L1.
+__device__ __forceinline__ RigidLane rigid_load(const IntegrateLaunch& L, int p, int lane) {
+  RigidLane S;
+  const DevParticle& P = L.P[p];
+  S.c = lane & 3;
+  S.second = lane >= 4;
+  S.a = S.c < 3 ? S.c : 2;
+  S.a1 = S.a == 2 ? 0 : S.a + 1;
+  S.a2 = S.a == 0 ? 2 : S.a - 1;
+  double F = (double)__ldcg(L.facc + 6 * p + S.a) * FIX_INV;
+  S.T = (double)__ldcg(L.facc + 6 * p + 3 + S.a) * FIX_INV;
   if (L.fc) {
-    F += (double)__ldcg(L.fc + 6 * p + a) * FIX_INV;
-    T += (double)__ldcg(L.fc + 6 * p + 3 + a) * FIX_INV;
+    F = __dadd_rn(F, (double)__ldcg(L.fc + 6 * p + S.a) * FIX_INV);
+    S.T = __dadd_rn(S.T, (double)__ldcg(L.fc + 6 * p + 3 + S.a) * FIX_INV);
   }
-  const double m = P.mass, dt = L.dt;
-  const double wg = m - L.rho0 * P.volume;
-  const double vel = P.vel[a] + dt / m * (F + wg * L.gravity[a]);
-  // unit quaternion of the current pose (w, v) and column a of its rotation
-  const double q0 = P.quat[0], q1 = P.quat[1], q2 = P.quat[2], q3 = P.quat[3];
-  const double iqn = 1.0 / sqrt(q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3);
-  const double w = q0 * iqn, vx = q1 * iqn, vy = q2 * iqn, vz = q3 * iqn;
-  const double s = w * w - (vx * vx + vy * vy + vz * vz);
-  const double va = pick3(a, vx, vy, vz), va1 = pick3(a1, vx, vy, vz), va2 = pick3(a2, vx, vy, vz);
-  const double C_a = s + 2.0 * va * va;               // R[a][a]
-  const double C_a1 = 2.0 * (va1 * va + w * va2);     // R[a1][a]
-  const double C_a2 = 2.0 * (va2 * va - w * va1);     // R[a2][a]
+  const double m = P.mass;
+  S.dt = L.dt;
+  S.hdt = __dmul_rn(0.5, L.dt);
+  S.dtm = __ddiv_rn(L.dt, m);
+  S.acc = __fma_rn(__fma_rn(-L.rho0, P.volume, m), L.gravity[S.a], F);
+  for (int k = 0; k < 3; ++k) {
+    S.I[k] = P.inertia[3 * S.a + k];
+    S.Ii[k] = P.inv_inertia[3 * S.a + k];
+  }
+  S.pos = P.pos[S.a];
+  S.vel = P.vel[S.a];
+  S.om = P.omega[S.a];
+  S.q = P.quat[S.c < 3 ? S.c + 1 : 0];
+  const double n = quad_norm2(S.q);
+  if (!near_one(n, 64)) S.q = __dmul_rn(S.q, __ddiv_rn(1.0, __dsqrt_rn(n)));
+  double rb, rc;
+  rigid_rotation(S, rb, rc);
+  return S;
+}
+
+__device__ __forceinline__ void rigid_store(const IntegrateLaunch& L, int p, const RigidLane& S) {
+  if (S.second) return;
+  DevParticle& P = L.P[p];
+  P.quat[S.c < 3 ? S.c + 1 : 0] = S.q;
+  if (S.c < 3) {
+    P.pos[S.c] = S.pos;
+    P.vel[S.c] = S.vel;
+    P.omega[S.c] = S.om;
+  }
+}
+
+// One substep; all 32 lanes of the warp take part (the shuffles).
+__device__ __forceinline__ void rigid_substep(RigidLane& S) {
+  const int a = S.a, a1 = S.a1, a2 = S.a2;
+  S.vel = __fma_rn(S.dtm, S.acc, S.vel);
+  S.pos = __fma_rn(S.dt, S.vel, S.pos);
   // body-frame angular velocity and torque: (R^T x)_a = R[a][a] x_a + R[a1][a] x_a1 + R[a2][a] x_a2
-  const double om_a = P.omega[a], om_a1 = P.omega[a1], om_a2 = P.omega[a2];
-  const double T_a1 = __shfl_sync(M4, T, a1), T_a2 = __shfl_sync(M4, T, a2);
-  double wb = C_a * om_a + C_a1 * om_a1 + C_a2 * om_a2;
-  const double Tb = C_a * T + C_a1 * T_a1 + C_a2 * T_a2;
-  const double wb0 = __shfl_sync(M4, wb, 0), wb1 = __shfl_sync(M4, wb, 1), wb2 = __shfl_sync(M4, wb, 2);
-  const double* I = P.inertia;
-  const double* Ii = P.inv_inertia;
-  const double Iw = I[3 * a] * wb0 + I[3 * a + 1] * wb1 + I[3 * a + 2] * wb2;
-  const double Iw_a1 = __shfl_sync(M4, Iw, a1), Iw_a2 = __shfl_sync(M4, Iw, a2);
-  const double wb_a1 = pick3(a1, wb0, wb1, wb2), wb_a2 = pick3(a2, wb0, wb1, wb2);
-  const double rhs = Tb - (wb_a1 * Iw_a2 - wb_a2 * Iw_a1);
-  const double r0 = __shfl_sync(M4, rhs, 0), r1 = __shfl_sync(M4, rhs, 1), r2 = __shfl_sync(M4, rhs, 2);
-  wb += dt * (Ii[3 * a] * r0 + Ii[3 * a + 1] * r1 + Ii[3 * a + 2] * r2);
-  // q <- normalize(q (x) exp(wb dt / 2)): dq = (cos h, (sin h / h) wb dt / 2), h = |wb| dt / 2
-  const double th = wb * dt;
-  const double t0 = __shfl_sync(M4, th, 0), t1 = __shfl_sync(M4, th, 1), t2 = __shfl_sync(M4, th, 2);
-  const double h2 = 0.25 * (t0 * t0 + t1 * t1 + t2 * t2);
-  double c, sa;  // cos h, sin(h) / h
+  const double v = S.second ? S.T : S.om;
+  double b = dot3(S.ca, v, S.cb, quad(v, a1), S.cc, quad(v, a2));
+  b = __dadd_rn(b, b);
+  const double other = __shfl_xor_sync(RIGID_FULL, b, 4);
+  const double wb = S.second ? other : b, Tb = S.second ? b : other;
+  const double wb0 = quad(wb, 0), wb1 = quad(wb, 1), wb2 = quad(wb, 2);
+  const double Iw = dot3(S.I[0], wb0, S.I[1], wb1, S.I[2], wb2);
+  const double rhs = __fma_rn(pick3(a2, wb0, wb1, wb2), quad(Iw, a1), __fma_rn(-pick3(a1, wb0, wb1, wb2), quad(Iw, a2), Tb));
+  const double wn = __fma_rn(S.dt, dot3(S.Ii[0], quad(rhs, 0), S.Ii[1], quad(rhs, 1), S.Ii[2], quad(rhs, 2)), wb);
+  // q <- normalize(q (x) exp(u)): dq = (cos h, (sin h / h) u), u = wn dt / 2, h = |u|
+  const double u = __dmul_rn(wn, S.hdt), u0 = quad(u, 0), u1 = quad(u, 1), u2 = quad(u, 2);
+  const double h2 = dot3(u0, u0, u1, u1, u2, u2);
+  double series;  // cos h (first four), sin(h) / h (second)
   if (h2 <= 1.0 / 4096.0) {
-    c = 1.0 + h2 * (-1.0 / 2 + h2 * (1.0 / 24 + h2 * (-1.0 / 720 + h2 * (1.0 / 40320))));
-    sa = 1.0 + h2 * (-1.0 / 6 + h2 * (1.0 / 120 + h2 * (-1.0 / 5040 + h2 * (1.0 / 362880))));
+    series = __fma_rn(h2, S.second ? 1.0 / 362880 : 1.0 / 40320, S.second ? -1.0 / 5040 : -1.0 / 720);
+    series = __fma_rn(h2, series, S.second ? 1.0 / 120 : 1.0 / 24);
+    series = __fma_rn(h2, series, S.second ? -1.0 / 6 : -1.0 / 2);
+    series = __fma_rn(h2, series, 1.0);
   } else {
-    const double hn = sqrt(h2);
-    c = cos(hn);
-    sa = sin(hn) / hn;
+    const double hn = __dsqrt_rn(h2);
+    series = S.second ? __ddiv_rn(sin(hn), hn) : cos(hn);
   }
-  const double sn = 0.5 * sa;
-  const double d0 = c, d1 = sn * t0, d2 = sn * t1, d3 = sn * t2;
-  // component `lane` of q (x) dq: sum over k of sign * q_k * dq_perm(k)
-  const int cq = lane;
-  const double e0 = cq == 0 ? d0 : (cq == 1 ? d1 : (cq == 2 ? d2 : d3));   // with q0, sign +
-  const double e1 = cq == 0 ? -d1 : (cq == 1 ? d0 : (cq == 2 ? -d3 : d2));  // with q1
-  const double e2 = cq == 0 ? -d2 : (cq == 1 ? d3 : (cq == 2 ? d0 : -d1));  // with q2
-  const double e3 = cq == 0 ? -d3 : (cq == 1 ? -d2 : (cq == 2 ? d1 : d0));  // with q3
-  double r = w * e0 + vx * e1 + vy * e2 + vz * e3;
-  const double n0 = __shfl_sync(M4, r, 0), n1 = __shfl_sync(M4, r, 1), n2 = __shfl_sync(M4, r, 2),
-               n3 = __shfl_sync(M4, r, 3);
-  const double irn = 1.0 / sqrt(n0 * n0 + n1 * n1 + n2 * n2 + n3 * n3);
-  r *= irn;
-  P.quat[cq] = r;
-  // new angular velocity in the world frame: row a of the new rotation times wb
-  const double W = n0 * irn, X = n1 * irn, Y = n2 * irn, Z = n3 * irn;
-  const double s2 = W * W - (X * X + Y * Y + Z * Z);
-  const double ua = pick3(a, X, Y, Z), ua1 = pick3(a1, X, Y, Z), ua2 = pick3(a2, X, Y, Z);
-  const double wn0 = __shfl_sync(M4, wb, 0), wn1 = __shfl_sync(M4, wb, 1), wn2 = __shfl_sync(M4, wb, 2);
-  const double wn_a = pick3(a, wn0, wn1, wn2), wn_a1 = pick3(a1, wn0, wn1, wn2), wn_a2 = pick3(a2, wn0, wn1, wn2);
-  const double omega = (s2 + 2.0 * ua * ua) * wn_a + 2.0 * (ua * ua1 - W * ua2) * wn_a1 + 2.0 * (ua * ua2 + W * ua1) * wn_a2;
-  if (lane < 3) {
-    P.vel[a] = vel;
-    P.omega[a] = omega;
-    P.pos[a] += dt * vel;
+  __syncwarp();
+  const double swap = __shfl_xor_sync(RIGID_FULL, series, 4);
+  const double d0 = S.second ? swap : series, dv = __dmul_rn(S.second ? series : swap, u);
+  const double d1 = quad(dv, 0), d2 = quad(dv, 1), d3 = quad(dv, 2);
+  const double x = quad(S.q, 0), y = quad(S.q, 1), z = quad(S.q, 2), w = quad(S.q, 3);
+  // this lane's component of q (x) dq
+  const double e0 = S.c == 3 ? d0 : (S.c == 0 ? d1 : (S.c == 1 ? d2 : d3));    // with w
+  const double e1 = S.c == 3 ? -d1 : (S.c == 0 ? d0 : (S.c == 1 ? -d3 : d2));  // with x
+  const double e2 = S.c == 3 ? -d2 : (S.c == 0 ? d3 : (S.c == 1 ? d0 : -d1));  // with y
+  const double e3 = S.c == 3 ? -d3 : (S.c == 0 ? -d2 : (S.c == 1 ? d1 : d0));  // with z
+  const double r = __fma_rn(z, e3, dot3(w, e0, x, e1, y, e2));
+  const double n = quad_norm2(r);
+  S.q = __dmul_rn(r, near_one(n, 1LL << 26) ? __fma_rn(-0.5, n, 1.5) : __ddiv_rn(1.0, __dsqrt_rn(n)));
+  // new angular velocity in the world frame: row a of the new rotation times wn
+  double rb, rc;
+  rigid_rotation(S, rb, rc);
+  const double o = dot3(S.ca, wn, rb, quad(wn, a1), rc, quad(wn, a2));
+  S.om = __dadd_rn(o, o);
+}
+
+// One substep of the particles [first, last) by the block's threads, four to a warp.
+__device__ __forceinline__ void integrate_particles(const IntegrateLaunch& L, int first, int last) {
+  const int lane = threadIdx.x & (RIGID_LANES - 1);
+  for (int base = first + (int)(threadIdx.x >> 5) * 4; base < last; base += (int)blockDim.x / RIGID_LANES) {
+    const int p = base + (int)((threadIdx.x & 31) / RIGID_LANES);
+    const bool mine = p < last;
+    RigidLane S = rigid_load(L, mine ? p : last - 1, lane);
+    rigid_substep(S);
+    __syncwarp();
+    if (mine) rigid_store(L, p, S);
   }
 }
 

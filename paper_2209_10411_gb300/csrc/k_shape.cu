@@ -15,7 +15,9 @@ namespace mi {
 namespace {
 
 constexpr int SH_THREADS = 256;
-constexpr int SH_MAX_BALLS = 4096;  // balls of one particle staged in shared memory (64 KB)
+constexpr int SH_MAX_BALLS = 4096;  // balls of one particle
+constexpr int SH_STAGED = 512;      // staged in shared memory up to this many (8 KB), else read from global memory
+constexpr int SH_POOL = 64;          // band cells of a warp waiting for their gradients (at most 31 + 32)
 constexpr unsigned SH_FULL = 0xffffffffu;
 
 struct ShapeLaunch {
@@ -35,6 +37,20 @@ struct ShapeLaunch {
   float* axes;
 };
 
+// a particle's balls: staged in shared memory, or where the caller has them
+// (there also two by two, x0 x1 y0 y1 and z0 z1 k0 k1, for the probes; an odd
+// last one with itself at k = 0)
+struct Staged {
+  const float4 *b, *pairs;
+  __device__ __forceinline__ float4 operator[](int j) const { return b[j]; }
+};
+struct InPlace {
+  const float* b;
+  __device__ __forceinline__ float4 operator[](int j) const {
+    return make_float4(__ldg(b + 4 * j), __ldg(b + 4 * j + 1), __ldg(b + 4 * j + 2), __ldg(b + 4 * j + 3));
+  }
+};
+
 // cell centre -lo + (i + 1/2) h with single FP32 roundings
 __device__ __forceinline__ float sh_coord(float lo, int i, float h) {
   return __fadd_rn(lo, __fmul_rn(__fadd_rn((float)i, 0.5f), h));
@@ -42,7 +58,8 @@ __device__ __forceinline__ float sh_coord(float lo, int i, float h) {
 
 // f at (x, y, z): differences, squares, (d0^2 + d1^2) + d2^2 and one IEEE
 // division per ball, each a single FP32 rounding, balls in order
-__device__ __forceinline__ float sh_field(const float4* B, int nb, float x, float y, float z) {
+template <class BallTable>
+__device__ __forceinline__ float sh_field(const BallTable& B, int nb, float x, float y, float z) {
   float f = 0.f;
   for (int j = 0; j < nb; ++j) {
     const float4 b = B[j];
@@ -61,26 +78,32 @@ __device__ __forceinline__ float sh_field(const float4* B, int nb, float x, floa
 struct ShapeProbe {
   float f, rm;
 };
-__device__ __forceinline__ ShapeProbe sh_probe(const float4* B, int nb, float x, float y, float z) {
-  float f0 = 0.f, f1 = 0.f, m0 = INFINITY, m1 = INFINITY;
-  int j = 0;
-  for (; j + 2 <= nb; j += 2) {
-    const float4 a = B[j], b = B[j + 1];
-    const float a0 = x - a.x, a1 = y - a.y, a2 = z - a.z, b0 = x - b.x, b1 = y - b.y, b2 = z - b.z;
-    const float ra = a0 * a0 + a1 * a1 + a2 * a2, rb = b0 * b0 + b1 * b1 + b2 * b2;
-    f0 += __fdividef(a.w, ra);
-    f1 += __fdividef(b.w, rb);
-    m0 = fminf(m0, ra);
-    m1 = fminf(m1, rb);
+__device__ __forceinline__ ShapeProbe sh_probe(const Staged& B, int nb, float x, float y, float z) {
+  // two balls at a time in packed pairs and with one reciprocal,
+  // k0 / r0 + k1 / r1 = (k0 r1 + k1 r0) / (r0 r1): the special-function pipe
+  // would otherwise set the time
+  const F32x2 xx = pack(x, x), yy = pack(y, y), zz = pack(z, z);
+  float f = 0.f, m = INFINITY;
+#pragma unroll 2
+  for (int j = 0; j < nb; j += 2) {
+    const float4 a = B.pairs[j], b = B.pairs[j + 1];
+    const F32x2 dx = vsub(xx, pack(a.x, a.y)), dy = vsub(yy, pack(a.z, a.w)), dz = vsub(zz, pack(b.x, b.y));
+    const float2 r = unpack(vfma(dz, dz, vfma(dy, dy, vmul(dx, dx))));
+    f += __fdividef(b.z * r.y + b.w * r.x, r.x * r.y);
+    m = fminf(m, fminf(r.x, r.y));
   }
-  if (j < nb) {
+  return {f, sqrtf(m)};
+}
+__device__ __forceinline__ ShapeProbe sh_probe(const InPlace& B, int nb, float x, float y, float z) {
+  float f = 0.f, m = INFINITY;
+  for (int j = 0; j < nb; ++j) {
     const float4 a = B[j];
-    const float a0 = x - a.x, a1 = y - a.y, a2 = z - a.z;
-    const float ra = a0 * a0 + a1 * a1 + a2 * a2;
-    f0 += __fdividef(a.w, ra);
-    m0 = fminf(m0, ra);
+    const float d0 = x - a.x, d1 = y - a.y, d2 = z - a.z;
+    const float r = d0 * d0 + d1 * d1 + d2 * d2;
+    f += __fdividef(a.w, r);
+    m = fminf(m, r);
   }
-  return {f0 + f1, sqrtf(fminf(m0, m1))};
+  return {f, sqrtf(m)};
 }
 
 // Cells beyond this one that certainly stay below `low` (f below it) or above
@@ -97,7 +120,8 @@ __device__ __forceinline__ int sh_stretch(const ShapeProbe& q, float low, float 
   return k >= 1.0f ? (int)fminf(k, 1e6f) : 0;
 }
 
-__device__ __forceinline__ float sh_gradnorm(const float4* B, int nb, float x, float y, float z) {
+template <class BallTable>
+__device__ __forceinline__ float sh_gradnorm(const BallTable& B, int nb, float x, float y, float z) {
   float gx = 0.f, gy = 0.f, gz = 0.f;
   for (int j = 0; j < nb; ++j) {
     const float4 b = B[j];
@@ -144,14 +168,27 @@ __device__ __forceinline__ void sh_add(float v, double* dst, float* red) {
   }
 }
 
-// The particle's balls into shared memory; whether every k is a number >= 0 (the
-// probes' bounds hold), the same in every thread.
-__device__ __forceinline__ bool sh_stage(const ShapeLaunch& S, int b0, int nb, float4* sb) {
+// The particle's balls into shared memory where they fit; whether every k is a
+// number >= 0 (the probes' bounds hold), the same in every thread.
+__device__ __forceinline__ bool sh_stage(const ShapeLaunch& S, int b0, int nb, float4* sb, float4* pairs) {
   bool plain = true;
   for (int j = threadIdx.x; j < nb; j += SH_THREADS) {
     const float4 v = make_float4(S.balls[4 * (b0 + j)], S.balls[4 * (b0 + j) + 1], S.balls[4 * (b0 + j) + 2],
                                  S.balls[4 * (b0 + j) + 3]);
-    sb[j] = v;
+    if (nb <= SH_STAGED) {
+      sb[j] = v;
+      float *p = reinterpret_cast<float*>(pairs + (j & ~1)), *q = p + (j & 1);
+      q[0] = v.x;
+      q[2] = v.y;
+      q[4] = v.z;
+      q[6] = v.w;
+      if (j == nb - 1 && !(j & 1)) {
+        p[1] = v.x;
+        p[3] = v.y;
+        p[5] = v.z;
+        p[7] = 0.f;
+      }
+    }
     plain = plain && v.w >= 0.f && isfinite(v.w) && isfinite(v.x) && isfinite(v.y) && isfinite(v.z);
   }
   return __syncthreads_and(plain) != 0;
@@ -163,66 +200,115 @@ __device__ __forceinline__ bool sh_stage(const ShapeLaunch& S, int b0, int nb, f
 // the probe settles (fluid: nothing to do; solid beyond the band: the moments
 // alone), cell by cell only inside the band; sh_field with its IEEE divisions
 // decides a cell only where the probe lies within its rounding error of 1,
-// 1 - eps or 1 + eps.  The same cells, in the same order, as an evaluation in
-// every cell gives: the sums are the same bits.  Bound by FP32 issue: the 300
-// particles of 8-64 balls at h = 1/4 take SHAPE1 ms, an evaluation in every cell
-// 33.7 ms (a sixth of the cells are solid, a twentieth lie in the band).
+// 1 - eps or 1 + eps.  The warp pools its cells of the band and takes 32
+// gradients at a time, a lane each (the threads meet the band in different turns
+// and some have many more of its cells); each thread adds its own, in its order.
+// The same cells, in the same order, as an evaluation in every cell gives: the
+// sums are the same bits.  Bound by FP32 issue: the 300 particles of 8-64 balls at
+// h = 1/4 take 6.7 ms; an evaluation in every cell 33.7 ms (a sixth of the cells
+// are solid, a twentieth lie in the band), the gradients in the turn that meets
+// them 11.8 ms, a queue per thread 9.1 ms.
+struct ShapeSums {
+  unsigned cnt;
+  float m[9], band;
+};
+template <class BallTable>
+__device__ __forceinline__ void sh_columns1(const ShapeLaunch& S, const BallTable& B, int nb, bool plain, int n, float lo,
+                                            float* zs, int* whose, ShapeSums& o) {
+  const float h = S.h, eps = S.eps;
+  const float slack = 1e-5f + 2.4e-7f * (float)nb, ih = 1.0f / h, blur = 2e-6f * -lo;
+  const int lane = threadIdx.x & 31;
+  // whole warps step together (the gradients are taken together)
+  for (long long col0 = (long long)blockIdx.x * SH_THREADS + (threadIdx.x & ~31u); col0 < (long long)n * n;
+       col0 += (long long)gridDim.x * SH_THREADS) {
+    const long long col = col0 + (threadIdx.x & 31u);
+    const int ix = (int)(col % n), iy = (int)(col / n);
+    const float x = sh_coord(lo, ix, h), y = sh_coord(lo, iy, h);
+    int iz = col < (long long)n * n ? 0 : n, kept = 0;  // kept: the warp's pooled cells
+    for (bool any = true; any;) {
+      const bool on = iz < n;
+      bool in_band = false;
+      float z = 0.f;
+      if (on) {
+        z = sh_coord(lo, iz, h);
+        int more = 0;  // cells after this one of the same kind
+        bool solid;
+        const ShapeProbe q = sh_probe(B, nb, x, y, z);
+        const float near = slack * fmaxf(q.f, 1.0f);
+        if (plain && fabsf(q.f - 1.0f) > near && fabsf(q.f - (1.0f - eps)) > near && fabsf(q.f - (1.0f + eps)) > near) {
+          solid = q.f > 1.0f;
+          in_band = fabsf(q.f - 1.0f) < eps;
+          if (!in_band) more = min(sh_stretch(q, 1.0f - eps, 1.0f + eps, slack, ih, blur), n - 1 - iz);
+        } else {
+          const float f = sh_field(B, nb, x, y, z);
+          solid = f >= 1.0f;
+          in_band = fabsf(__fsub_rn(f, 1.0f)) < eps;
+        }
+        if (solid) {
+          for (int k = 0; k <= more; ++k) {
+            const float zk = sh_coord(lo, iz + k, h);
+            ++o.cnt;
+            o.m[0] += x;
+            o.m[1] += y;
+            o.m[2] += zk;
+            o.m[3] += x * x;
+            o.m[4] += x * y;
+            o.m[5] += x * zk;
+            o.m[6] += y * y;
+            o.m[7] += y * zk;
+            o.m[8] += zk * zk;
+          }
+        }
+        iz += 1 + more;
+      }
+      const unsigned band = __ballot_sync(SH_FULL, in_band);
+      if (in_band) {
+        const int at = kept + __popc(band & ((1u << lane) - 1u));
+        zs[at] = z;
+        whose[at] = lane;
+      }
+      kept += __popc(band);
+      any = __any_sync(SH_FULL, iz < n);
+      __syncwarp();
+      while (kept >= 32 || (kept > 0 && !any)) {
+        const int take = min(kept, 32), owner = lane < take ? whose[lane] : -1;
+        const float zo = lane < take ? zs[lane] : 0.f;
+        const float xo = __shfl_sync(SH_FULL, x, owner & 31), yo = __shfl_sync(SH_FULL, y, owner & 31);
+        const float g = lane < take ? sh_gradnorm(B, nb, xo, yo, zo) : 0.f;
+        for (int k = 0; k < take; ++k) {
+          const float gk = __shfl_sync(SH_FULL, g, k);
+          if (__shfl_sync(SH_FULL, owner, k) == lane) o.band += gk;
+        }
+        kept -= take;
+        if (lane < kept) {  // the rest (fewer than 32) to the front
+          zs[lane] = zs[lane + 32];
+          whose[lane] = whose[lane + 32];
+        }
+        __syncwarp();
+      }
+    }
+  }
+}
+
 __global__ void __launch_bounds__(SH_THREADS) k_shape_pass1(ShapeLaunch S) {
-  extern __shared__ float4 sb[];
+  __shared__ float4 sb[SH_STAGED], pairs[SH_STAGED];
+  __shared__ float zs[SH_THREADS / 32][SH_POOL];
+  __shared__ int whose[SH_THREADS / 32][SH_POOL];
+  const int w = threadIdx.x >> 5;
   __shared__ float red[SH_THREADS / 32];
   const int p = blockIdx.y;
   const int b0 = S.ball_off[p], nb = S.ball_off[p + 1] - b0;
   if (nb < 1 || nb > SH_MAX_BALLS) return;  // no solid cell counted: NaN descriptors
-  const bool plain = sh_stage(S, b0, nb, sb);
-  const int n = S.grid_n[p];
-  const float lo = -S.grid_r[p], h = S.h, eps = S.eps;
-  const float slack = 1e-5f + 2.4e-7f * (float)nb, ih = 1.0f / h, blur = 2e-6f * S.grid_r[p];
-  unsigned cnt = 0;
-  float m[9] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, band = 0.f;
-  for (long long col = (long long)blockIdx.x * SH_THREADS + threadIdx.x; col < (long long)n * n;
-       col += (long long)gridDim.x * SH_THREADS) {
-    const int ix = (int)(col % n), iy = (int)(col / n);
-    const float x = sh_coord(lo, ix, h), y = sh_coord(lo, iy, h);
-    for (int iz = 0; iz < n;) {
-      const float z = sh_coord(lo, iz, h);
-      int more = 0;  // cells after this one of the same kind
-      bool solid, in_band;
-      const ShapeProbe q = sh_probe(sb, nb, x, y, z);
-      const float near = slack * fmaxf(q.f, 1.0f);
-      if (plain && fabsf(q.f - 1.0f) > near && fabsf(q.f - (1.0f - eps)) > near && fabsf(q.f - (1.0f + eps)) > near) {
-        solid = q.f > 1.0f;
-        in_band = fabsf(q.f - 1.0f) < eps;
-        if (!in_band) more = min(sh_stretch(q, 1.0f - eps, 1.0f + eps, slack, ih, blur), n - 1 - iz);
-      } else {
-        const float f = sh_field(sb, nb, x, y, z);
-        solid = f >= 1.0f;
-        in_band = fabsf(__fsub_rn(f, 1.0f)) < eps;
-      }
-      if (solid) {
-        for (int k = 0; k <= more; ++k) {
-          const float zk = sh_coord(lo, iz + k, h);
-          ++cnt;
-          m[0] += x;
-          m[1] += y;
-          m[2] += zk;
-          m[3] += x * x;
-          m[4] += x * y;
-          m[5] += x * zk;
-          m[6] += y * y;
-          m[7] += y * zk;
-          m[8] += zk * zk;
-        }
-      }
-      if (in_band) band += sh_gradnorm(sb, nb, x, y, z);
-      iz += 1 + more;
-    }
-  }
-  unsigned c = cnt;
+  const bool plain = sh_stage(S, b0, nb, sb, pairs);
+  ShapeSums o = {0u, {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, 0.f};
+  if (nb <= SH_STAGED) sh_columns1(S, Staged{sb, pairs}, nb, plain, S.grid_n[p], -S.grid_r[p], zs[w], whose[w], o);
+  else sh_columns1(S, InPlace{S.balls + 4 * (size_t)b0}, nb, plain, S.grid_n[p], -S.grid_r[p], zs[w], whose[w], o);
+  unsigned c = o.cnt;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(SH_FULL, c, o);
+  for (int k = 16; k > 0; k >>= 1) c += __shfl_xor_sync(SH_FULL, c, k);
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(S.cnt + p, (unsigned long long)c);
-  sh_add(band, S.acc + 10 * p, red);
-  for (int a = 0; a < 9; ++a) sh_add(m[a], S.acc + 10 * p + 1 + a, red);
+  sh_add(o.band, S.acc + 10 * p, red);
+  for (int a = 0; a < 9; ++a) sh_add(o.m[a], S.acc + 10 * p + 1 + a, red);
 }
 
 // principal axes by cyclic Jacobi rotations of the centred second moments
@@ -285,20 +371,16 @@ __global__ void k_shape_axes(ShapeLaunch S) {
 }
 
 // grid 2 along the axes: extents and the columns along the shortest axis, the
-// columns walked as in grid 1 (27.6 ms with an evaluation in every cell, SHAPE2 so)
-__global__ void __launch_bounds__(SH_THREADS) k_shape_pass2(ShapeLaunch S) {
-  extern __shared__ float4 sb[];
-  const int p = blockIdx.y;
-  const int b0 = S.ball_off[p], nb = S.ball_off[p + 1] - b0;
-  if (S.cnt[p] == 0 || nb > SH_MAX_BALLS) return;
-  const bool plain = sh_stage(S, b0, nb, sb);
+// columns walked as in grid 1 (27.6 ms with an evaluation in every cell, 2.95 so)
+template <class BallTable>
+__device__ __forceinline__ void sh_columns2(const ShapeLaunch& S, const BallTable& B, int nb, bool plain, int p,
+                                            float (&mn)[3], float (&mx)[3]) {
   const float* fr = S.frame + 12 * p;
   const float cx = fr[0], cy = fr[1], cz = fr[2];
   const float* E = fr + 3;  // rows: long, intermediate, short axes
   const int n2 = S.grid_n[p] + 4;
   const float h = S.h, lo = -(S.grid_r[p] + 2.0f * h);
   const float slack = 1e-5f + 2.4e-7f * (float)nb, ih = 1.0f / h, blur = 1e-5f * S.grid_r[p];
-  float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
   for (long long col = (long long)blockIdx.x * SH_THREADS + threadIdx.x; col < (long long)n2 * n2;
        col += (long long)gridDim.x * SH_THREADS) {
     const int i1 = (int)(col % n2), i2 = (int)(col / n2);
@@ -310,12 +392,12 @@ __global__ void __launch_bounds__(SH_THREADS) k_shape_pass2(ShapeLaunch S) {
       const float x = px + u3 * E[6], y = py + u3 * E[7], z = pz + u3 * E[8];
       int more = 0;
       bool solid;
-      const ShapeProbe q = sh_probe(sb, nb, x, y, z);
+      const ShapeProbe q = sh_probe(B, nb, x, y, z);
       if (plain && fabsf(q.f - 1.0f) > slack * fmaxf(q.f, 1.0f)) {
         solid = q.f > 1.0f;
         more = min(sh_stretch(q, 1.0f, 1.0f, slack, ih, blur), n2 - 1 - i3);
       } else {
-        solid = sh_field(sb, nb, x, y, z) >= 1.0f;
+        solid = sh_field(B, nb, x, y, z) >= 1.0f;
       }
       if (solid) {
         any = true;
@@ -333,6 +415,17 @@ __global__ void __launch_bounds__(SH_THREADS) k_shape_pass2(ShapeLaunch S) {
       atomicOr(S.bits + (size_t)p * S.words + (bit >> 5), 1u << (bit & 31));
     }
   }
+}
+
+__global__ void __launch_bounds__(SH_THREADS) k_shape_pass2(ShapeLaunch S) {
+  __shared__ float4 sb[SH_STAGED], pairs[SH_STAGED];
+  const int p = blockIdx.y;
+  const int b0 = S.ball_off[p], nb = S.ball_off[p + 1] - b0;
+  if (S.cnt[p] == 0 || nb > SH_MAX_BALLS) return;
+  const bool plain = sh_stage(S, b0, nb, sb, pairs);
+  float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
+  if (nb <= SH_STAGED) sh_columns2(S, Staged{sb, pairs}, nb, plain, p, mn, mx);
+  else sh_columns2(S, InPlace{S.balls + 4 * (size_t)b0}, nb, plain, p, mn, mx);
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
 #pragma unroll
@@ -437,10 +530,6 @@ extern "C" mi_status mi_shape_descriptors(int n_particles, const int* ball_off, 
   S.bits = reinterpret_cast<unsigned*>(sp);
   S.out = out;
   S.axes = axes;
-  const size_t smem = sizeof(float4) * (size_t)SH_MAX_BALLS;
-  if (cudaFuncSetAttribute(k_shape_pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-      cudaFuncSetAttribute(k_shape_pass2, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return MI_ECUDA;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return MI_ECUDA;
@@ -450,9 +539,9 @@ extern "C" mi_status mi_shape_descriptors(int n_particles, const int* ball_off, 
   if (bx1 > cap) bx1 = cap;
   if (bx2 > cap) bx2 = cap;
   k_shape_clear<<<dim3((unsigned)((words + 255) / 256 + 1), n_particles), 256, 0, s>>>(S);
-  k_shape_pass1<<<dim3((unsigned)bx1, n_particles), SH_THREADS, smem, s>>>(S);
+  k_shape_pass1<<<dim3((unsigned)bx1, n_particles), SH_THREADS, 0, s>>>(S);
   k_shape_axes<<<(n_particles + 127) / 128, 128, 0, s>>>(S);
-  k_shape_pass2<<<dim3((unsigned)bx2, n_particles), SH_THREADS, smem, s>>>(S);
+  k_shape_pass2<<<dim3((unsigned)bx2, n_particles), SH_THREADS, 0, s>>>(S);
   k_shape_final<<<n_particles, SH_THREADS, 0, s>>>(S);
   return cudaGetLastError() == cudaSuccess ? MI_OK : MI_ECUDA;
 }

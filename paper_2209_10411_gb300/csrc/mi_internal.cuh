@@ -112,6 +112,50 @@ template <> __device__ __forceinline__ unsigned short pack16<MI_STORE_BF16_DEV>(
 }
 
 // ---------------------------------------------------------------------------
+// Packed FP32 pairs: one instruction for both values, each a single rounding
+// (the scalar forms beside them give the same bits one value at a time).
+// ---------------------------------------------------------------------------
+struct F32x2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ float vfma(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ float vadd(float a, float b) { return __fadd_rn(a, b); }
+__device__ __forceinline__ float vsub(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ float vset(float s, float) { return s; }
+__device__ __forceinline__ F32x2 pack(float lo, float hi) {
+  F32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 unpack(F32x2 a) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(a.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vfma(F32x2 a, F32x2 b, F32x2 c) {
+  F32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vadd(F32x2 a, F32x2 b) {
+  F32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vsub(F32x2 a, F32x2 b) {
+  F32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vmul(F32x2 a, F32x2 b) {
+  F32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 vset(float s, F32x2) { return pack(s, s); }
+
+// ---------------------------------------------------------------------------
 // Launch parameters of the lattice kernels.
 // ---------------------------------------------------------------------------
 struct LatticeGeom {

@@ -38,17 +38,6 @@ static FastDiv fast_div(unsigned d) {
 // Every operation is a single rounding in both, so a node's result does not
 // depend on which of the two computed it.
 
-// 1 / rho: the hardware approximation and one Newton step by FMA (no slow path)
-__device__ __forceinline__ float rcp_start(float a) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
-  return r;
-}
-__device__ __forceinline__ F32x2 rcp_start(F32x2 a) {
-  const float2 v = unpack(a);
-  return pack(rcp_start(v.x), rcp_start(v.y));
-}
-
 // BGK collision on deviations h_i = f_i - w_i.
 //   rho = 1 + sum h_i, j = sum e_i h_i (sum w_i = 1, sum w_i e_i = 0)
 //   f_eq,i - w_i = w_i (rho - 1) + w_i rho (3 e.u + 4.5 (e.u)^2 - 1.5 u.u)
@@ -73,7 +62,7 @@ __device__ __forceinline__ void collide_inplace(V (&h)[19], const CollideParams&
   u[2] = vadd(vadd(d[3], vsub(d[6], d[7])), vsub(d[8], d[9]));
   const V one = vset(1.0f, drho);
   const V rho = vadd(one, drho);
-  V r = rcp_start(rho);
+  V r = rcp_start(rho);  // and one Newton step: no slow path
   r = vfma(r, vfma(vsub(vset(0.0f, r), rho), r, one), r);
   if (FORCE)
     for (int a = 0; a < 3; ++a) u[a] = vadd(u[a], vset(0.5f * P.force[a], r));

@@ -155,6 +155,17 @@ __device__ __forceinline__ F32x2 vmul(F32x2 a, F32x2 b) {
 }
 __device__ __forceinline__ F32x2 vset(float s, F32x2) { return pack(s, s); }
 
+// 1 / a, the hardware's approximation (a relative error of about 2^-23, subnormals flushed)
+__device__ __forceinline__ float rcp_start(float a) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
+  return r;
+}
+__device__ __forceinline__ F32x2 rcp_start(F32x2 a) {
+  const float2 v = unpack(a);
+  return pack(rcp_start(v.x), rcp_start(v.y));
+}
+
 // ---------------------------------------------------------------------------
 // Launch parameters of the lattice kernels.
 // ---------------------------------------------------------------------------

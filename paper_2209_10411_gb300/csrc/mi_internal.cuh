@@ -296,6 +296,7 @@ struct ParticleLaunch {
   const int* flag_off;
   const int* cls_off;
   int flag_blocks, classify_blocks;
+  int cls_unit;               // rows a classification warp takes together (1 or 4)
   LatticeGeom g;
 };
 cudaError_t launch_prologue(const ParticleLaunch& L, cudaStream_t s);

@@ -177,9 +177,6 @@ __global__ void __launch_bounds__(PROLOGUE_THREADS) k_prologue(ParticleLaunch L)
   if (p >= L.np) return;
   DevParticle& P = L.P[p];
   const double r = rotation_entry(P.quat, lane);
-  double R[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) R[k] = __shfl_sync(FULL, r, k);
   if (lane < 9) {
     const float rf = (float)r;
     P.R[lane] = r;

@@ -248,15 +248,17 @@ __device__ __forceinline__ void sh_columns1(const ShapeLaunch& S, const BallTabl
           for (int k = 0; k <= more; ++k) {
             const float zk = sh_coord(lo, iz + k, h);
             ++o.cnt;
-            o.m[0] += x;
-            o.m[1] += y;
-            o.m[2] += zk;
-            o.m[3] += x * x;
-            o.m[4] += x * y;
-            o.m[5] += x * zk;
-            o.m[6] += y * y;
-            o.m[7] += y * zk;
-            o.m[8] += zk * zk;
+            // each rounding stated, so that the sums (and through the axes the
+            // projection's columns) do not turn on how a loop is contracted
+            o.m[0] = __fadd_rn(o.m[0], x);
+            o.m[1] = __fadd_rn(o.m[1], y);
+            o.m[2] = __fadd_rn(o.m[2], zk);
+            o.m[3] = __fmaf_rn(x, x, o.m[3]);
+            o.m[4] = __fmaf_rn(x, y, o.m[4]);
+            o.m[5] = __fmaf_rn(x, zk, o.m[5]);
+            o.m[6] = __fadd_rn(o.m[6], __fmul_rn(y, y));
+            o.m[7] = __fmaf_rn(y, zk, o.m[7]);
+            o.m[8] = __fmaf_rn(zk, zk, o.m[8]);
           }
         }
         iz += 1 + more;

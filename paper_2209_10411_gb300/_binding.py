@@ -536,8 +536,8 @@ class Simulation:
         """overlap_boundary: compute the boundary nodes beside the bulk kernel
         (True) or after it; unfused_dem: run DEM substeps as one launch
         sequence per substep instead of the fused substep kernel;
-        links_beside: the links' bounce-back and momentum exchange beside the
-        bulk kernel instead of after it."""
+        links_beside: the same as overlap_boundary (one kernel computes the
+        links with the boundary nodes)."""
         flags = (SCHEDULE_OVERLAP_BOUNDARY if overlap_boundary else 0) | (SCHEDULE_UNFUSED_DEM if unfused_dem else 0) | \
             (SCHEDULE_LINKS_BESIDE if links_beside else 0)
         self._check(lib.mi_delbm_set_schedule(self.h, flags))

@@ -151,6 +151,7 @@ ParticleLaunch mi_delbm::particle_launch() const {
   L.balls = dballs;
   L.balls_d = dballs_d;
   L.balls_w = dballs_w;
+  L.balls_s = dballs_s;
   L.max_balls_per_particle = max_balls_pp < 2048 ? max_balls_pp : 2048;
   L.cur_buf = owner_cur;
   L.prev_buf = owner_cur ^ 1;
@@ -717,10 +718,11 @@ mi_status mi_delbm::ensure_particle_buffers() {
   dP = (DevParticle*)dalloc(sizeof(DevParticle) * np);
   dballs = (float4*)dalloc(sizeof(float4) * nb);
   dballs_d = (double*)dalloc(sizeof(double) * 4 * nb);
-  dballs_w = (float4*)dalloc(sizeof(float4) * 3 * nb);
+  float4*& links_balls = cfg.storage == MI_STORE_F32 ? dballs_w : dballs_s;
+  links_balls = (float4*)dalloc(sizeof(float4) * (cfg.storage == MI_STORE_F32 ? 3 : 2) * nb);
   dblk_off = (int*)dalloc(sizeof(int) * 2 * ((size_t)np + 1));
   if (!dblk_off) return fail(MI_ENOMEM, "particle buffers: device allocation failed");
-  if (!owner[0] || !owner[1] || !stamp || !dctr || !facc || !fc || !dP || !dballs || !dballs_d || !dballs_w)
+  if (!owner[0] || !owner[1] || !stamp || !dctr || !facc || !fc || !dP || !dballs || !dballs_d || !links_balls)
     return fail(MI_ENOMEM, "particle buffers: device allocation failed");
   cudaError_t e = cudaMemsetAsync(owner[0], 0xFF, ncell * 4, stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(owner[1], 0xFF, ncell * 4, stream);
@@ -901,9 +903,9 @@ mi_status mi_delbm_create(const mi_delbm_config* cfg, mi_delbm** out) {
   if (cfg->storage != MI_STORE_F32) {
     // 16-bit storages: four nodes per thread (64-bit accesses) when nx allows
     // and the lattice has enough nodes to fill the chip with a quarter of the
-    // threads (64^3: 13.8 us against 8.6 with two nodes, 128^3: 34.5 against
-    // 33.1, 160^3: equal, 192^3: 94.7 against 98.4, 192 x 192 x 768: 346
-    // against 370), else two
+    // threads (64^3: 12.6 us against 8.2 with two nodes, 128^3: 35.0 against
+    // 34.1, 160^3: 63 against 60, 192^3: equal, 192 x 192 x 768: 366 against
+    // 370), else two
     if (cfg->nx % 4 == 0 && ncell >= (1 << 22)) h->tune.bulk_pairs = 3;
     else if (cfg->nx % 2 == 0) h->tune.bulk_pairs = 1;
   }
@@ -1537,10 +1539,23 @@ mi_status mi_delbm_add_particle(mi_delbm* h, int n, const double* centers, const
   std::vector<double> c(centers, centers + 3 * (size_t)n);
   const int off = h->n_balls_total;
   auto upload_balls = [&]() -> cudaError_t {
-    std::vector<float4> bf(n);
+    std::vector<float4> bf(n), bs(2 * (size_t)n);
     std::vector<double> bd(4 * (size_t)n);
     for (int i = 0; i < n; ++i) {
       bf[i] = make_float4((float)c[3 * i], (float)c[3 * i + 1], (float)c[3 * i + 2], (float)k[i]);
+      // hi + lo split for k_links_q16's float-float residual: a centre coordinate
+      // below 1024 in magnitude as its nearest multiple of 2^-12 (exact in FP32)
+      // plus the FP32 remainder, so that its difference with a link origin split
+      // the same way is exact; k as its FP32 rounding plus the remainder
+      double hi[4];
+      for (int a = 0; a < 3; ++a) {
+        const double v = c[3 * i + a];
+        hi[a] = std::fabs(v) < 1024.0 ? std::rint(v * 4096.0) / 4096.0 : (double)(float)v;
+      }
+      hi[3] = (double)(float)k[i];
+      bs[2 * i] = make_float4((float)hi[0], (float)hi[1], (float)hi[2], (float)hi[3]);
+      bs[2 * i + 1] = make_float4((float)(c[3 * i] - hi[0]), (float)(c[3 * i + 1] - hi[1]),
+                                  (float)(c[3 * i + 2] - hi[2]), (float)(k[i] - hi[3]));
       bd[4 * i] = c[3 * i];
       bd[4 * i + 1] = c[3 * i + 1];
       bd[4 * i + 2] = c[3 * i + 2];
@@ -1549,6 +1564,8 @@ mi_status mi_delbm_add_particle(mi_delbm* h, int n, const double* centers, const
     cudaError_t e = cudaMemcpyAsync(h->dballs + off, bf.data(), sizeof(float4) * n, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess)
       e = cudaMemcpyAsync(h->dballs_d + 4 * (size_t)off, bd.data(), sizeof(double) * 4 * n, cudaMemcpyHostToDevice, h->stream);
+    if (e == cudaSuccess && h->dballs_s)
+      e = cudaMemcpyAsync(h->dballs_s + 2 * (size_t)off, bs.data(), sizeof(float4) * 2 * n, cudaMemcpyHostToDevice, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     return e;
   };

@@ -67,7 +67,8 @@ struct mi_delbm {
   mi::DevParticle* dP = nullptr;
   float4* dballs = nullptr;
   double* dballs_d = nullptr;
-  float4* dballs_w = nullptr;   // per ball: three float4 in the lattice frame, written by k_flag each step
+  float4* dballs_w = nullptr;   // FP32 storage, per ball: three float4 in the lattice frame, written by k_flag each step
+  float4* dballs_s = nullptr;   // 16-bit storages, per ball: FP32 (c, k), then the FP32 remainders of the FP64 (c, k)
   int n_balls_total = 0;
   int max_balls_pp = 0;              // largest ball count of one particle
   uint32_t* stamp = nullptr;

@@ -33,61 +33,63 @@ static FastDiv fast_div(unsigned d) {
   return {(unsigned)((((1ull << l) - d) << 32) / d + 1), l > 1 ? 1u : l, l > 1 ? l - 1 : 0u};
 }
 
-// One or two nodes per value: the collision is written once over V = float (one
-// node) or V = F32x2 (two nodes, packed FP32 pairs: one instruction for both).
-// Every operation is a single rounding in both, so a node's result does not
-// depend on which of the two computed it.
-
 // BGK collision on deviations h_i = f_i - w_i.
 //   rho = 1 + sum h_i, j = sum e_i h_i (sum w_i = 1, sum w_i e_i = 0)
 //   f_eq,i - w_i = w_i (rho - 1) + w_i rho (3 e.u + 4.5 (e.u)^2 - 1.5 u.u)
 //   h+_i = (1 - omega) h_i + omega (f_eq,i - w_i)   [+ Guo source]
-// A direction and its opposite (2k - 1, 2k) share the even part of f_eq and
-// take its odd part with either sign, and the moments come from their sums
-// and differences: about 130 operations a node, where forming each direction
-// by itself took 260.
+// in two forms, by storage.  Every operation of either is written out as a single
+// rounding, and a direction and its opposite (2k - 1, 2k) share what is the same
+// or exactly the negative.
+
+// 1 / rho, rounded to nearest (a start within an ulp and one Newton step in fused
+// operations: Markstein 1990), without the range checks of the general division.
+template <class V>
+__device__ __forceinline__ V inverse(V rho) {
+  const V r = rcp_start(rho);
+  return vfma(r, vfma(vsub(vset(0.0f, r), rho), r, vset(1.0f, r)), r);
+}
+
+// FP32 storage: the moments from the sums and differences of opposite directions,
+// the odd part of the equilibrium from the momentum, the even part from the odd
+// one; about 150 operations a node.
 //
 // omega / 36 and omega / 12 are float pairs, and the weights 1, 2 and 12 times
 // them: a rounded omega w_i is the same relative error at every node and step,
 // a source of mass and momentum.  The states of the particles after 20 steps of
 // a 64^3 box, against 64 bits: 1.2e-10 off with pairs, 5e-10 with rounded products.
-template <bool FORCE, class V>
-__device__ __forceinline__ void collide_inplace(V (&h)[19], const CollideParams& P) {
-  V s[10], d[10];  // pair k: h[2k - 1] + h[2k], h[2k - 1] - h[2k]
+template <bool FORCE>
+__device__ __forceinline__ void collide_pairs(float (&h)[19], const CollideParams& P) {
+  float s[10], d[10];  // pair k: h[2k - 1] + h[2k], h[2k - 1] - h[2k]
 #pragma unroll
   for (int k = 1; k < 10; ++k) {
     s[k] = vadd(h[2 * k - 1], h[2 * k]);
     d[k] = vsub(h[2 * k - 1], h[2 * k]);
   }
-  const V drho = vadd(vadd(vadd(h[0], vadd(s[1], s[2])), vadd(s[3], vadd(s[4], s[5]))),
-                      vadd(vadd(s[6], s[7]), vadd(s[8], s[9])));
-  V j[3], u[3];  // the momentum, 1.5 times the velocity
+  const float drho = vadd(vadd(vadd(h[0], vadd(s[1], s[2])), vadd(s[3], vadd(s[4], s[5]))),
+                          vadd(vadd(s[6], s[7]), vadd(s[8], s[9])));
+  float j[3], u[3];  // the momentum, 1.5 times the velocity
   j[0] = vadd(vadd(d[1], vadd(d[4], d[5])), vadd(d[6], d[7]));
   j[1] = vadd(vadd(d[2], vsub(d[4], d[5])), vadd(d[8], d[9]));
   j[2] = vadd(vadd(d[3], vsub(d[6], d[7])), vsub(d[8], d[9]));
-  const V one = vset(1.0f, drho);
-  const V rho = vadd(one, drho);
-  V r = rcp_start(rho);  // and one Newton step: no slow path
-  r = vfma(r, vfma(vsub(vset(0.0f, r), rho), r, one), r);
+  const float r15 = vmul(1.5f, inverse(vadd(1.0f, drho)));
   if (FORCE)
-    for (int a = 0; a < 3; ++a) j[a] = vadd(j[a], vset(0.5f * P.force[a], r));
-  V v[3];  // omega / 12 times the momentum: odd part 3 omega w_i rho e.u, even part that times 1.5 e.u
-  const V r15 = vmul(vset(1.5f, r), r);
+    for (int a = 0; a < 3; ++a) j[a] = vadd(j[a], 0.5f * P.force[a]);
+  float v[3];  // omega / 12 times the momentum: odd part 3 omega w_i rho e.u, even part that times 1.5 e.u
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     u[a] = vmul(j[a], r15);
-    v[a] = vfma(vset(P.c12[0], r), j[a], vmul(vset(P.c12[1], r), j[a]));
+    v[a] = vfma(P.c12[0], j[a], vmul(P.c12[1], j[a]));
   }
-  const V base = vsub(drho, vfma(j[0], u[0], vfma(j[1], u[1], vmul(j[2], u[2]))));  // drho - 1.5 rho u.u
-  const V based = vfma(vset(P.c36[0], r), base, vmul(vset(P.c36[1], r), base)), basea = vadd(based, based);
+  const float base = vsub(drho, vfma(j[0], u[0], vfma(j[1], u[1], vmul(j[2], u[2]))));  // drho - 1.5 rho u.u
+  const float based = vfma(P.c36[0], base, vmul(P.c36[1], base)), basea = vadd(based, based);
   const float om = P.omega;
-  const V keep = vset(P.keep, r);
-  V uF;
-  if (FORCE) uF = vfma(vset(P.force[0], r), u[0], vfma(vset(P.force[1], r), u[1], vmul(vset(P.force[2], r), u[2])));
+  float uF = 0.f;
+  if (FORCE) uF = vfma(P.force[0], u[0], vfma(P.force[1], u[1], vmul(P.force[2], u[2])));
+  const auto relax = [&](int i, float e) { h[i] = vfma(P.keep, h[i], e); };
   {
-    V e0 = vmul(vset(12.0f, r), based);
-    if (FORCE) e0 = vfma(vset(-2.0f * (1.0f - 0.5f * om) * wq(0), r), uF, e0);
-    h[0] = vfma(keep, h[0], e0);
+    float e0 = vmul(12.0f, based);
+    if (FORCE) e0 = vfma(-2.0f * (1.0f - 0.5f * om) * wq(0), uF, e0);
+    relax(0, e0);
   }
 #pragma unroll
   for (int k = 1; k < 10; ++k) {
@@ -95,24 +97,104 @@ __device__ __forceinline__ void collide_inplace(V (&h)[19], const CollideParams&
     // 1.5 e_i . u: the first non-zero component of every odd direction is +1
     const int a = cx(i) ? 0 : (cy(i) ? 1 : 2), b = cz(i) ? 2 : 1;
     const bool plus = (b == 1 ? cy(i) : cz(i)) > 0;
-    const V eu = k <= 3 ? u[a] : (plus ? vadd(u[a], u[b]) : vsub(u[a], u[b]));
-    V odd = k <= 3 ? vadd(v[a], v[a]) : (plus ? vadd(v[a], v[b]) : vsub(v[a], v[b]));
-    V even = vfma(odd, eu, k <= 3 ? basea : based);
+    const float eu = k <= 3 ? u[a] : (plus ? vadd(u[a], u[b]) : vsub(u[a], u[b]));
+    float odd = k <= 3 ? vadd(v[a], v[a]) : (plus ? vadd(v[a], v[b]) : vsub(v[a], v[b]));
+    float even = vfma(odd, eu, k <= 3 ? basea : based);
     if (FORCE) {
       const float g = (1.0f - 0.5f * om) * wq(i);
       const float eF = cx(i) * P.force[0] + cy(i) * P.force[1] + cz(i) * P.force[2];
-      even = vadd(even, vfma(vset(6.0f * g * eF, r), eu, vmul(vset(-2.0f * g, r), uF)));
-      odd = vadd(odd, vset(3.0f * g * eF, r));
+      even = vadd(even, vfma(6.0f * g * eF, eu, vmul(-2.0f * g, uF)));
+      odd = vadd(odd, 3.0f * g * eF);
     }
-    h[i] = vfma(keep, h[i], vadd(even, odd));
-    h[i + 1] = vfma(keep, h[i + 1], vsub(even, odd));
+    relax(i, vadd(even, odd));
+    relax(i + 1, vsub(even, odd));
   }
+}
+
+// The momentum of 16-bit storages: by the differences of opposite directions, or
+// added direction by direction (SEQ: boundary nodes, links, covered nodes).
+template <bool SEQ, class V>
+__device__ __forceinline__ void momentum(const V (&h)[19], V (&j)[3]) {
+  if (SEQ) {
+    j[0] = vsub(h[1], h[2]);
+    j[1] = vsub(h[3], h[4]);
+    j[2] = vsub(h[5], h[6]);
+#pragma unroll
+    for (int i = 7; i < 19; ++i) {
+      if (cx(i)) j[0] = cx(i) > 0 ? vadd(j[0], h[i]) : vsub(j[0], h[i]);
+      if (cy(i)) j[1] = cy(i) > 0 ? vadd(j[1], h[i]) : vsub(j[1], h[i]);
+      if (cz(i)) j[2] = cz(i) > 0 ? vadd(j[2], h[i]) : vsub(j[2], h[i]);
+    }
+  } else {
+    V d[10];
+#pragma unroll
+    for (int k = 1; k < 10; ++k) d[k] = vsub(h[2 * k - 1], h[2 * k]);
+    j[0] = vadd(vadd(vadd(vadd(d[1], d[4]), d[5]), d[6]), d[7]);
+    j[1] = vadd(vadd(vsub(vadd(d[2], d[4]), d[5]), d[8]), d[9]);
+    j[2] = vsub(vadd(vsub(vadd(d[3], d[6]), d[7]), d[8]), d[9]);
+  }
+}
+
+// 16-bit storages, one node (V = float) or two (V = F32x2, packed FP32 pairs: one
+// instruction for both; a node's result does not depend on which).  Here the order of
+// the operations is part of the result: a value near the middle of two
+// representable ones moves by a whole unit (2^-11 or 2^-8 of it) when its FP32 value
+// moves by one ulp, the bounce-back hands such a unit on to the particles, and a
+// light one's velocity then differs by 1e-7 after 20 steps.  So it is
+// fixed, direction by direction,
+//   fma(omega, fma(w_i, fma(rho, fma(-1.5, u.u, fma(3, e.u, 4.5 e.u e.u)), drho), -h_i), h_i)
+// with omega = 1 / tau rounded once.  About 170 operations a node: 256 x 256 x 512 in
+// FP16 takes 402 us with it, 397 with the form above.
+template <bool FORCE, bool SEQ = false, class V>
+__device__ __forceinline__ void collide_ordered(V (&h)[19], const CollideParams& P) {
+  V drho = h[0];
+#pragma unroll
+  for (int i = 1; i < 19; ++i) drho = vadd(drho, h[i]);
+  V u[3];
+  momentum<SEQ>(h, u);
+  const V rho = vadd(vset(1.0f, drho), drho), irho = inverse(rho);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) u[a] = vmul(FORCE ? vadd(u[a], vset(0.5f * P.force[a], irho)) : u[a], irho);
+  const V usq = vfma(u[2], u[2], vfma(u[0], u[0], vmul(u[1], u[1])));
+  const V m15 = vset(-1.5f, rho), m_om = vset(-P.omega, rho), three = vset(3.0f, rho), m_three = vset(-3.0f, rho);
+  V uF;
+  if (FORCE) uF = vfma(u[2], vset(P.force[2], rho), vfma(u[0], vset(P.force[0], rho), vmul(u[1], vset(P.force[1], rho))));
+  // h_i relaxed towards w_i (drho + rho n), n the bracket above; f: the source's bracket
+  const auto relax = [&](int i, V n, V f) {
+    const V x = vfma(vset(-wq(i), rho), vfma(rho, n, drho), h[i]);  // exactly the negative of f_eq - w - h
+    h[i] = vfma(m_om, x, h[i]);
+    if (FORCE) h[i] = vfma(vset((1.0f - 0.5f * P.omega) * wq(i), rho), f, h[i]);
+  };
+  relax(0, vmul(m15, usq), FORCE ? vmul(m_three, uF) : rho);
+#pragma unroll
+  for (int k = 1; k < 10; ++k) {
+    const int i = 2 * k - 1;
+    // e_i . u: the first non-zero component of every odd direction is +1
+    const int a = cx(i) ? 0 : (cy(i) ? 1 : 2), b = cz(i) ? 2 : 1;
+    const V eu = k <= 3 ? u[a] : ((b == 1 ? cy(i) : cz(i)) > 0 ? vadd(u[a], u[b]) : vsub(u[a], u[b]));
+    const V sq = vmul(vmul(vset(4.5f, rho), eu), eu);
+    const V np = vfma(m15, usq, vfma(three, eu, sq)), nm = vfma(m15, usq, vfma(m_three, eu, sq));
+    V fp = rho, fm = rho;
+    if (FORCE) {
+      const V eF = vset(cx(i) * P.force[0] + cy(i) * P.force[1] + cz(i) * P.force[2], rho), n9 = vmul(vset(9.0f, rho), eu);
+      fp = vfma(n9, eF, vmul(three, vsub(eF, uF)));
+      fm = vfma(n9, eF, vmul(m_three, vadd(eF, uF)));
+    }
+    relax(i, np, fp);
+    relax(i + 1, nm, fm);
+  }
+}
+
+template <int ST, bool FORCE, bool SEQ = false>
+__device__ __forceinline__ void collide(float (&h)[19], const CollideParams& P) {
+  if constexpr (ST == MI_STORE_F32) collide_pairs<FORCE>(h, P);
+  else collide_ordered<FORCE, SEQ>(h, P);
 }
 
 template <int ST, bool FORCE>
 __device__ __forceinline__ void collide_store(float (&h)[19], typename Store<ST>::T* __restrict__ B,
                                               long long plane, long long c, const CollideParams& P) {
-  collide_inplace<FORCE>(h, P);
+  collide<ST, FORCE>(h, P);
 #pragma unroll
   for (int i = 0; i < 19; ++i) Store<ST>::put(B + i * plane + c, i, h[i]);
 }
@@ -194,13 +276,15 @@ __device__ __forceinline__ void update_node(const typename Store<ST>::T* __restr
 // recomputed by k_near.  Nodes anywhere else have no solid or uncovered
 // neighbour, so their update here is final.
 //
-// Bound by HBM: FP32 alone, 256 x 256 x 512 in 0.798 ms = 6.39 TB/s (0.94 of a
-// copy), 512^3 in 3.06 ms = 6.67 TB/s (0.98), 141 x 83 x 119 in 38 us.  With
+// Bound by HBM: FP32 alone, 256 x 256 x 512 in 0.786 ms = 6.49 TB/s (0.955 of a
+// copy), 512^3 in 3.05 ms = 6.68 TB/s (0.98), 141 x 83 x 119 in 37 us.  With
 // rows as blocks, a branch per direction at the faces and the collision formed
 // direction by direction these took 0.955 ms, 3.53 ms and 74 us.  Blocks of 64
-// threads measured best from 64^3 to 512^3 (32: up to 3 % more, 256: 4 %).
+// threads measured best from 64^3 to 512^3 (32: up to 3 % more, 128: 1 %).  The
+// registers decide whether the 19 loads are issued together: 48 (40 with a body
+// force, 0.790 ms), where the compiler's own choices of 42 and 48 took 0.799 and 0.801.
 template <int ST, bool FORCE>
-__global__ void __launch_bounds__(256) k_bulk(const typename Store<ST>::T* __restrict__ A,
+__global__ void __launch_bounds__(256, FORCE ? 6 : 5) k_bulk(const typename Store<ST>::T* __restrict__ A,
                                               typename Store<ST>::T* __restrict__ B, LatticeGeom g,
                                               CollideParams P, FastDiv by_nx, FastDiv by_ny, unsigned ncell) {
   const unsigned c = blockIdx.x * blockDim.x + threadIdx.x;
@@ -236,14 +320,14 @@ static cudaError_t launch_bulk_t(const BulkLaunch& L, cudaStream_t s) {
 // on the y and z faces take the general per-node path.  The same concurrency
 // contract as k_bulk.  Requires nx % W == 0.
 //
-// Bound by HBM: 256 x 256 x 512 FP16 in 0.394 ms = 6.48 TB/s (0.95 of a copy),
-// 512^3 in 1.59 ms, four nodes per thread.  With unpacked FP32 arithmetic, rows
+// Bound by HBM: 256 x 256 x 512 FP16 in 0.402 ms = 6.34 TB/s (0.93 of a copy),
+// 512^3 in 1.60 ms, four nodes per thread.  With unpacked FP32 arithmetic, rows
 // as blocks and branches per direction at the faces these took 0.522 and 1.99
-// ms: that kernel waited for instruction issue.  Two nodes per thread reach 0.449
+// ms: that kernel waited for instruction issue.  Two nodes per thread reach 0.430
 // ms (more instructions a byte) but, with twice the threads, win on small
-// lattices: 64^3 in 8 against 12 us; the one-node kernel takes 0.598 ms.  Five
-// blocks of 128 threads per SM (96 registers, a few spilled) measured 7 % faster
-// than four (128 registers).
+// lattices: 64^3 in 8 against 13 us; the one-node kernel takes 0.611 ms.  Five
+// blocks of 128 threads per SM (96 registers, a few spilled) measured 4 % faster
+// than four (128 registers), 5 % with a body force (0.425 ms).
 template <int ST> __device__ __forceinline__ float2 unpack2(unsigned w);
 template <> __device__ __forceinline__ float2 unpack2<MI_STORE_F16_DEV>(unsigned w) {
   return __half22float2(*reinterpret_cast<const __half2*>(&w));
@@ -281,7 +365,7 @@ template <> struct Words<4> {
 };
 
 template <int ST, bool FORCE, int W>
-__global__ void __launch_bounds__(128, W == 4 ? (FORCE ? 4 : 5) : (FORCE ? 6 : 7))
+__global__ void __launch_bounds__(128, W == 4 ? 5 : (FORCE ? 7 : 8))
     k_bulk16(const typename Store<ST>::T* __restrict__ A, typename Store<ST>::T* __restrict__ B, LatticeGeom g,
              CollideParams P, FastDiv by_groups, FastDiv by_ny, unsigned ngroups) {
   const unsigned t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -337,7 +421,7 @@ __global__ void __launch_bounds__(128, W == 4 ? (FORCE ? 4 : 5) : (FORCE ? 6 : 7
     F32x2 h[19];
 #pragma unroll
     for (int i = 0; i < 19; ++i) h[i] = pack(v[i].x, v[i].y);
-    collide_inplace<FORCE>(h, P);
+    collide_ordered<FORCE>(h, P);
 #pragma unroll
     for (int i = 0; i < 19; ++i) {
       const float2 r = unpack(h[i]);
@@ -456,14 +540,15 @@ __device__ __forceinline__ float lw(int j) { return j == 0 ? (1.0f / 3.0f) : (j 
 __device__ __forceinline__ int lopp(int j) { return j == 0 ? 0 : ((j & 1) ? j + 1 : j - 1); }
 
 // Cover/uncover rule: a node's population momentum J = sum e_i h_i (FP32, lane i
-// holds h_i) and its torque about the particle's position, sign * (J, (x - X_p) x J),
-// added to the particle's fixed-point hydrodynamic sums.
+// holds h_i, added direction by direction) and its torque about the particle's
+// position, sign * (J, (x - X_p) x J), added to the particle's fixed-point
+// hydrodynamic sums.
 __device__ __forceinline__ void add_node_momentum(long long* facc, const DevParticle* Ps, uint32_t p, int x, int y,
-                                                  int z, float h, int ex, int ey, int ez, float sign, unsigned lane) {
-  float J[3] = {ex * h, ey * h, ez * h};
+                                                  int z, float h, float sign, unsigned lane) {
+  float all[19], J[3];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    for (int a = 0; a < 3; ++a) J[a] += __shfl_xor_sync(0xffffffffu, J[a], o);
+  for (int i = 1; i < 19; ++i) all[i] = __shfl_sync(0xffffffffu, h, i);
+  momentum<true>(all, J);
   const DevParticle& P = Ps[p];
   const float r0 = (float)(x - P.pos[0]), r1 = (float)(y - P.pos[1]), r2 = (float)(z - P.pos[2]);
   const float v[6] = {J[0], J[1], J[2], r1 * J[2] - r2 * J[1], r2 * J[0] - r0 * J[2], r0 * J[1] - r1 * J[0]};
@@ -506,7 +591,7 @@ __global__ void __launch_bounds__(128) k_refill(BoundaryLaunch L) {
     if (lane < 19u) Store<ST>::put_at(A + i * g.plane + c, wi, h);
     // cover/uncover rule: the particle that uncovered the node gives up the
     // momentum of the refilled populations, sum e_i (f_i - w_i)
-    if (L.pl.cover_uncover) add_node_momentum(L.pl.facc, L.pl.P, pid, x, y, z, lane < 19u ? h : 0.f, ex, ey, ez, -1.0f, lane);
+    if (L.pl.cover_uncover) add_node_momentum(L.pl.facc, L.pl.P, pid, x, y, z, h, -1.0f, lane);
   }
   if (!L.pl.cover_uncover) return;
   // covered nodes: the momentum of their post-collision populations f+(t)
@@ -517,7 +602,7 @@ __global__ void __launch_bounds__(128) k_refill(BoundaryLaunch L) {
     int x, y, z;
     coords(c, g, x, y, z);
     const float h = Store<ST>::dev_at(A + i * g.plane + c, wi);
-    add_node_momentum(L.pl.facc, L.pl.P, L.pl.owner_cur[c], x, y, z, lane < 19u ? h : 0.f, ex, ey, ez, 1.0f, lane);
+    add_node_momentum(L.pl.facc, L.pl.P, L.pl.owner_cur[c], x, y, z, h, 1.0f, lane);
   }
 }
 
@@ -669,9 +754,15 @@ __global__ void __launch_bounds__(BOUNDARY_THREADS) k_boundary(BoundaryLaunch L)
       coords(c, g, x, y, z);
       pull_node<ST>(A, g, L.p, x, y, z, c, h, mask);
       if (!LADD) {
-        float rho, u[3];
-        moments_at<ST>(A, g.plane, c, rho, u);
-        s_mom[t] = make_float4(rho, u[0], u[1], u[2]);
+        float own[19], j[3];
+#pragma unroll
+        for (int i = 0; i < 19; ++i) own[i] = Store<ST>::dev(A + i * g.plane + c, i);
+        float dr = 0.f;
+#pragma unroll
+        for (int i = 0; i < 19; ++i) dr += own[i];
+        momentum<true>(own, j);
+        const float rho = 1.0f + dr, irho = inverse(rho);
+        s_mom[t] = make_float4(rho, j[0] * irho, j[1] * irho, j[2] * irho);
       }
       s_xyz[t] = make_int3(x, y, z);
       s_mask[t] = mask;
@@ -738,8 +829,11 @@ __global__ void __launch_bounds__(BOUNDARY_THREADS) k_boundary(BoundaryLaunch L)
         uw[0] = P.velf[0] + (P.omegaf[1] * r2 - P.omegaf[2] * r1);
         uw[1] = P.velf[1] + (P.omegaf[2] * r0 - P.omegaf[0] * r2);
         uw[2] = P.velf[2] + (P.omegaf[0] * r1 - P.omegaf[1] * r0);
-        float G = hopp + 6.0f * wd * rho0 * (-ed[0] * uw[0] - ed[1] * uw[1] - ed[2] * uw[2]);
-        if (!LADD) {
+        const float wall = 6.0f * wd * rho0 * (-ed[0] * uw[0] - ed[1] * uw[1] - ed[2] * uw[2]);
+        float G;
+        if (LADD) {
+          G = hopp + wall;
+        } else {
           float ud[3];
           const float i1q = 1.0f / (1.0f + q), iq = 1.0f / q;
           const float a1 = (1.0f - q) * i1q, a2 = 2.0f * q * i1q;
@@ -753,7 +847,7 @@ __global__ void __launch_bounds__(BOUNDARY_THREADS) k_boundary(BoundaryLaunch L)
           const float euf = ed[0] * uf[0] + ed[1] * uf[1] + ed[2] * uf[2];
           const float ud2 = ud[0] * ud[0] + ud[1] * ud[1] + ud[2] * ud[2];
           const float uf2 = uf[0] * uf[0] + uf[1] * uf[1] + uf[2] * uf[2];
-          G += wd * rho_f * (3.0f * (eud - euf) + 4.5f * (eud * eud - euf * euf) - 1.5f * (ud2 - uf2));
+          G = hopp + wd * rho_f * (3.0f * (eud - euf) + 4.5f * (eud * eud - euf * euf) - 1.5f * (ud2 - uf2)) + wall;
         }
         s_g[d - 1][s] = G;
         // momentum exchange, rounded per link (v * 2^40 is exact in FP32 and the
@@ -791,7 +885,7 @@ __global__ void __launch_bounds__(BOUNDARY_THREADS) k_boundary(BoundaryLaunch L)
 #pragma unroll
         for (int j = 1; j < 19; ++j)
           if ((mask >> opp(j)) & 1u) h[j] = s_g[opp(j) - 1][t];
-      collide_inplace<FORCE>(h, L.p);
+      collide<ST, FORCE, true>(h, L.p);
 #pragma unroll
       for (int j = 0; j < 19; ++j) {
         if (L.tmp) Store<ST>::put(static_cast<T*>(L.tmp) + 19 * (size_t)bi + j, j, h[j]);

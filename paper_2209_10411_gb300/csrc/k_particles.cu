@@ -182,6 +182,31 @@ __global__ void __launch_bounds__(PROLOGUE_THREADS) k_prologue(ParticleLaunch L)
     P.R[lane] = r;
     P.Rf[lane] = rf;
   }
+  if (L.balls_s) {
+    // the body frame as float pairs (k_links_q16): R, R^T (X - floor X) by lanes
+    // 0 to 2, R^T e_d by lane d
+    double R[9], f[3];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) R[k] = __shfl_sync(FULL, r, k);
+    for (int k = 0; k < 3; ++k) f[k] = P.pos[k] - floor(P.pos[k]);
+    if (lane < 9) {
+      P.Rs[0][lane] = (float)r;
+      P.Rs[1][lane] = (float)(r - (double)(float)r);
+    }
+    if (lane < 3) {
+      const double t = pick3(lane, R[0], R[1], R[2]) * f[0] + pick3(lane, R[3], R[4], R[5]) * f[1] +
+                       pick3(lane, R[6], R[7], R[8]) * f[2];
+      P.Ts[0][lane] = (float)t;
+      P.Ts[1][lane] = (float)(t - (double)(float)t);
+    }
+    if (lane < 19)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const double e = R[k] * lex(lane) + R[3 + k] * ley(lane) + R[6 + k] * lez(lane);
+        P.Es[lane][k] = (float)e;
+        P.Es[lane][3 + k] = (float)(e - (double)(float)e);
+      }
+  }
   // axis a = lane of the box and of the position's split
   if (lane < 3) {
     const int a = lane;
@@ -262,8 +287,8 @@ __global__ void __launch_bounds__(32 * FLAG_WARPS, 3) k_flag(ParticleLaunch L) {
   if (threadIdx.x == 0) rr_s = -1;
   if (staged)
     for (int i = threadIdx.x; i < nb; i += blockDim.x) sb[i] = L.balls[P.ball_off + i];
-  // the ball table of the wall fractions (below), by the particle's first block
-  if (bb.b == 0)
+  // the ball table of FP32 storage's wall fractions (below), by the particle's first block
+  if (bb.b == 0 && L.balls_w)
     for (int i = threadIdx.x; i < nb; i += blockDim.x)
       lattice_ball(P, L.balls_d + 4 * (size_t)(P.ball_off + i), L.balls_w + 3 * (size_t)(P.ball_off + i));
   __syncthreads();
@@ -721,8 +746,9 @@ cudaError_t launch_classify(const ParticleLaunch& L, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------------------
-// Wall fraction of each link: root q in (0, 1] of g(q) = f_p(x_f + q e_d) - 1
-// (Sec. 2.3.2; reading A7: along the link that points into the solid, c0 = 1).
+// Wall fraction of each link, FP32 storage (16 bits: k_links16.cu): root q in (0, 1]
+// of g(q) = f_p(x_f + q e_d) - 1 (Sec. 2.3.2; reading A7: along the link that points
+// into the solid, c0 = 1).
 //
 // In the lattice frame, with the balls' centres turned once per step (k_flag,
 // FP64): a link point relative to floor X is n + q e with whole numbers n and e.
@@ -908,6 +934,7 @@ cudaError_t launch_links_q(const ParticleLaunch& L, int grid, cudaStream_t s) {
   // no more blocks than the link list's capacity can use
   const unsigned long long need = ((unsigned long long)L.cap_links + 255ull) / 256ull;
   if (need < (unsigned long long)grid) grid = need < 1 ? 1 : (int)need;
+  if (L.balls_s) return launch_links_q16(L, grid, s);
   k_links_q<<<grid, 256, 0, s>>>(L);
   return cudaGetLastError();
 }

@@ -224,6 +224,11 @@ struct DevParticle {
   int pos_i[3];                              // floor(pos), and pos - floor(pos) in FP32: node offsets
   float pos_fr[3];                           //   x - X = (x - pos_i) - pos_fr without FP64 arithmetic
   float Rf[9];                               // R rounded to FP32 (set with pos_i, pos_fr each step)
+  // 16-bit storages: float pairs (hi, lo) of the body frame at the current pose,
+  // for the wall fraction's float-float arithmetic (set by the prologue each step):
+  float Rs[2][9];                            //   R
+  float Ts[2][3];                            //   R^T (X - floor X)
+  float Es[19][6];                           //   R^T e_d: hi xyz, lo xyz per direction d
   float core_s;                              // core scale s = ((r_e - R_s) / r_e)^2 (constant)
   float Rb_f, re_f, skin_f;                  // FP32 copies of R_b, r_e, R_s (constant)
   float link_grid;                           // spacing the wall fraction splits coordinates on (constant, see link_grid_of)
@@ -236,7 +241,7 @@ struct DevParticle {
   float sctr[2][3];                          // the position (FP32) the solid nodes of buffer b were flagged at
 };
 
-// The wall fraction (k_links_q) splits every coordinate difference u of a link
+// The wall fraction of FP32 storage (k_links_q) splits every coordinate difference u of a link
 // point and a ball into a multiple of link_grid and a remainder.  A link point
 // and a centre are both within R_b + 1.5 of the particle's origin cell, so
 // |u| < 2 R_b + 4 <= 2^12 link_grid makes |u|^2 a whole number below 2^24 of
@@ -272,7 +277,11 @@ struct ParticleLaunch {
   int np;
   const float4* balls;        // (c_x, c_y, c_z, k) FP32
   const double* balls_d;      // (c_x, c_y, c_z, k) FP64, 4 per ball
-  float4* balls_w;            // per ball three float4 in the lattice frame at the current pose (lattice_ball)
+  // the wall fraction's ball table, by storage (the other one NULL): FP32 three float4
+  // a ball in the lattice frame at the current pose (lattice_ball), 16 bits two float4 a
+  // ball, FP32 (c, k) and the FP32 remainders of the FP64 values
+  float4* balls_w;
+  const float4* balls_s;
   int max_balls_per_particle;
   uint32_t* owner_cur;        // buffer being written this step
   const uint32_t* owner_prev; // flags of the previous step
@@ -303,6 +312,7 @@ cudaError_t launch_prologue(const ParticleLaunch& L, cudaStream_t s);
 cudaError_t launch_flag(const ParticleLaunch& L, cudaStream_t s);
 cudaError_t launch_classify(const ParticleLaunch& L, cudaStream_t s);
 cudaError_t launch_links_q(const ParticleLaunch& L, int grid, cudaStream_t s);
+cudaError_t launch_links_q16(const ParticleLaunch& L, int grid, cudaStream_t s);  // its form for 16-bit storages
 
 struct BoundaryLaunch {
   ParticleLaunch pl;

@@ -119,13 +119,12 @@ CollideParams mi_delbm::collide_params() const {
   CollideParams p;
   std::memset(&p, 0, sizeof(p));
   p.omega = (float)(1.0 / cfg.tau);
-  p.keep = 1.0f - p.omega;
   const auto split = [](double v, float (&out)[2]) {
     out[0] = (float)v;
     out[1] = (float)(v - (double)out[0]);
   };
-  split((1.0 - (double)p.keep) / 36.0, p.c36);
-  split((1.0 - (double)p.keep) / 12.0, p.c12);
+  split((double)p.omega / 36.0, p.c36);
+  split((double)p.omega / 12.0, p.c12);
   for (int a = 0; a < 3; ++a) p.force[a] = (float)cfg.fluid_body_force[a];
   for (int f = 0; f < 6; ++f)
     for (int i = 0; i < 19; ++i)

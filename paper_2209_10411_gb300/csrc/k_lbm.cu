@@ -57,6 +57,9 @@ __device__ __forceinline__ V inverse(V rho) {
 // them: a rounded omega w_i is the same relative error at every node and step,
 // a source of mass and momentum.  The states of the particles after 20 steps of
 // a 64^3 box, against 64 bits: 1.2e-10 off with pairs, 5e-10 with rounded products.
+// (1 - omega) h is h - omega h in one rounding: a rounded 1 - omega is off by up to
+// 2^-25 whatever omega is, at tau = 100 1e-6 and at tau = 10,000 2e-4 of the viscosity
+// (and the low half of a pair would be lost in the sum with the equilibrium).
 template <bool FORCE>
 __device__ __forceinline__ void collide_pairs(float (&h)[19], const CollideParams& P) {
   float s[10], d[10];  // pair k: h[2k - 1] + h[2k], h[2k - 1] - h[2k]
@@ -85,7 +88,7 @@ __device__ __forceinline__ void collide_pairs(float (&h)[19], const CollideParam
   const float om = P.omega;
   float uF = 0.f;
   if (FORCE) uF = vfma(P.force[0], u[0], vfma(P.force[1], u[1], vmul(P.force[2], u[2])));
-  const auto relax = [&](int i, float e) { h[i] = vfma(P.keep, h[i], e); };
+  const auto relax = [&](int i, float e) { h[i] = vadd(vfma(-om, h[i], h[i]), e); };
   {
     float e0 = vmul(12.0f, based);
     if (FORCE) e0 = vfma(-2.0f * (1.0f - 0.5f * om) * wq(0), uF, e0);
@@ -282,7 +285,7 @@ __device__ __forceinline__ void update_node(const typename Store<ST>::T* __restr
 // direction by direction these took 0.955 ms, 3.53 ms and 74 us.  Blocks of 64
 // threads measured best from 64^3 to 512^3 (32: up to 3 % more, 128: 1 %).  The
 // registers decide whether the 19 loads are issued together: 48 (40 with a body
-// force, 0.790 ms), where the compiler's own choices of 42 and 48 took 0.799 and 0.801.
+// force, 0.787 ms), where the compiler's own choices of 42 and 48 took 0.799 and 0.801.
 template <int ST, bool FORCE>
 __global__ void __launch_bounds__(256, FORCE ? 6 : 5) k_bulk(const typename Store<ST>::T* __restrict__ A,
                                               typename Store<ST>::T* __restrict__ B, LatticeGeom g,

@@ -177,8 +177,7 @@ struct LatticeGeom {
 
 struct CollideParams {
   float omega;            // 1 / tau
-  float keep;             // 1 - omega in FP32; the equilibrium's share is 1 - keep exactly:
-  float c36[2], c12[2];   // (1 - keep) / 36 and / 12 as float pairs (hi, lo)
+  float c36[2], c12[2];   // omega / 36 and omega / 12 as float pairs (hi, lo)
   float force[3];         // Guo body force density (zero unless set)
   float bb_wall[6][19];   // 6 w_i rho0 (e_i . u_wall[face]) per face and direction
   float rho0;

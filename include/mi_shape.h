@@ -49,8 +49,8 @@ size_t mi_shape_scratch_bytes(int n_particles, int max_n);
  * most max_n), out (MI_SHAPE_FIELDS doubles per particle), axes (9 floats per
  * particle: the unit axes, longest first, as rows; may be NULL), scratch
  * (mi_shape_scratch_bytes).  h > 0 and 0 < eps < 1 are the spacing and the
- * band half-width.  A particle without a solid cell, or with more than 4096
- * balls, gets NaN descriptors.
+ * band half-width.  A particle without a solid cell, with more than 4096 balls
+ * or with n outside 1 .. max_n gets NaN descriptors.
  * Errors: MI_EINVAL (sizes, h, eps, NULL arrays), MI_ECUDA. */
 mi_status mi_shape_descriptors(int n_particles, const int *ball_off, const float *balls, const float *grid_r,
                                const int *grid_n, int max_n, float h, float eps, double *out, float *axes,

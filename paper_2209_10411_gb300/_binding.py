@@ -319,7 +319,9 @@ def shape_descriptors(models, h, eps=0.1):
     c64 = rows[:, :3].astype(np.float64)
     far = np.maximum.reduceat(np.sqrt((c64 * c64).sum(1)), off[:-1])
     rg = (far + np.sqrt(ksum / (1.0 - eps))).astype(np.float32)
-    ng = np.ceil(2.0 * rg.astype(np.float64) / h).astype(np.int32)
+    # cell counts as Python integers: a radius that is not finite, or more cells than
+    # an int32 holds, is an error here (an array cast would pass it on as any number)
+    ng = np.array([int(np.ceil(2.0 * r / h)) for r in rg.tolist()], dtype=np.int32)
     balls = torch.from_numpy(rows).to(dev)
     offs = torch.from_numpy(off).to(dev)
     R = torch.from_numpy(rg).to(dev)

@@ -26,6 +26,7 @@ struct ShapeLaunch {
   const float* balls;
   const float* grid_r;
   const int* grid_n;
+  int max_n;                 // largest cell count a particle may have (sizes the bitmaps)
   float h, eps;
   int words;                 // bitmap words per particle
   unsigned long long* cnt;   // solid cells per particle
@@ -300,11 +301,12 @@ __global__ void __launch_bounds__(SH_THREADS) k_shape_pass1(ShapeLaunch S) {
   __shared__ float red[SH_THREADS / 32];
   const int p = blockIdx.y;
   const int b0 = S.ball_off[p], nb = S.ball_off[p + 1] - b0;
-  if (nb < 1 || nb > SH_MAX_BALLS) return;  // no solid cell counted: NaN descriptors
+  const int n = S.grid_n[p];
+  if (nb < 1 || nb > SH_MAX_BALLS || n < 1 || n > S.max_n) return;  // no solid cell counted: NaN descriptors
   const bool plain = sh_stage(S, b0, nb, sb, pairs);
   ShapeSums o = {0u, {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, 0.f};
-  if (nb <= SH_STAGED) sh_columns1(S, Staged{sb, pairs}, nb, plain, S.grid_n[p], -S.grid_r[p], zs[w], whose[w], o);
-  else sh_columns1(S, InPlace{S.balls + 4 * (size_t)b0}, nb, plain, S.grid_n[p], -S.grid_r[p], zs[w], whose[w], o);
+  if (nb <= SH_STAGED) sh_columns1(S, Staged{sb, pairs}, nb, plain, n, -S.grid_r[p], zs[w], whose[w], o);
+  else sh_columns1(S, InPlace{S.balls + 4 * (size_t)b0}, nb, plain, n, -S.grid_r[p], zs[w], whose[w], o);
   unsigned c = o.cnt;
 #pragma unroll
   for (int k = 16; k > 0; k >>= 1) c += __shfl_xor_sync(SH_FULL, c, k);
@@ -518,6 +520,7 @@ extern "C" mi_status mi_shape_descriptors(int n_particles, const int* ball_off, 
   S.balls = balls;
   S.grid_r = grid_r;
   S.grid_n = grid_n;
+  S.max_n = max_n;
   S.h = h;
   S.eps = eps;
   S.words = (int)words;

@@ -169,10 +169,13 @@ __device__ __forceinline__ void sh_add(float v, double* dst, float* red) {
   }
 }
 
-// The particle's balls into shared memory where they fit; whether every k is a
-// number >= 0 (the probes' bounds hold), the same in every thread.
-__device__ __forceinline__ bool sh_stage(const ShapeLaunch& S, int b0, int nb, float4* sb, float4* pairs) {
-  bool plain = true;
+// The particle's balls into shared memory where they fit; whether the probes' bounds
+// hold, the same in every thread: every k is a number >= 0, and the radius R lies
+// between 1e-8 and 1e8.  A probe's products of two squared distances are of the size
+// of R^4 near the surface, at most 144 R^4, and lose bits or overflow beyond (from
+// about 3e-10 down and 8e8 up); such models are decided cell by cell.
+__device__ __forceinline__ bool sh_stage(const ShapeLaunch& S, int b0, int nb, float R, float4* sb, float4* pairs) {
+  bool plain = R > 1e-8f && R < 1e8f;
   for (int j = threadIdx.x; j < nb; j += SH_THREADS) {
     const float4 v = make_float4(S.balls[4 * (b0 + j)], S.balls[4 * (b0 + j) + 1], S.balls[4 * (b0 + j) + 2],
                                  S.balls[4 * (b0 + j) + 3]);
@@ -303,7 +306,7 @@ __global__ void __launch_bounds__(SH_THREADS) k_shape_pass1(ShapeLaunch S) {
   const int b0 = S.ball_off[p], nb = S.ball_off[p + 1] - b0;
   const int n = S.grid_n[p];
   if (nb < 1 || nb > SH_MAX_BALLS || n < 1 || n > S.max_n) return;  // no solid cell counted: NaN descriptors
-  const bool plain = sh_stage(S, b0, nb, sb, pairs);
+  const bool plain = sh_stage(S, b0, nb, S.grid_r[p], sb, pairs);
   ShapeSums o = {0u, {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, 0.f};
   if (nb <= SH_STAGED) sh_columns1(S, Staged{sb, pairs}, nb, plain, n, -S.grid_r[p], zs[w], whose[w], o);
   else sh_columns1(S, InPlace{S.balls + 4 * (size_t)b0}, nb, plain, n, -S.grid_r[p], zs[w], whose[w], o);
@@ -426,7 +429,7 @@ __global__ void __launch_bounds__(SH_THREADS) k_shape_pass2(ShapeLaunch S) {
   const int p = blockIdx.y;
   const int b0 = S.ball_off[p], nb = S.ball_off[p + 1] - b0;
   if (S.cnt[p] == 0 || nb > SH_MAX_BALLS) return;
-  const bool plain = sh_stage(S, b0, nb, sb, pairs);
+  const bool plain = sh_stage(S, b0, nb, S.grid_r[p], sb, pairs);
   float mn[3] = {INFINITY, INFINITY, INFINITY}, mx[3] = {-INFINITY, -INFINITY, -INFINITY};
   if (nb <= SH_STAGED) sh_columns2(S, Staged{sb, pairs}, nb, plain, p, mn, mx);
   else sh_columns2(S, InPlace{S.balls + 4 * (size_t)b0}, nb, plain, p, mn, mx);

@@ -29,8 +29,10 @@ namespace mi {
 // Taylor series when a <= 1/64 (terms to a^8: the first omitted term is below
 // 2^-53 relative there), from the library functions otherwise.  1/|q| of a
 // quaternion whose squared norm n is within 2^-26 of 1 (every product made
-// here) is 1.5 - n / 2, off by 3/8 (n - 1)^2 < 2^-53; one that is handed in is
-// normalised when n is more than 64 ulps from 1.
+// here) is 1.5 - n / 2, off by 3/8 (n - 1)^2 < 2^-53.  A quaternion made here has
+// n within 6 ulps of 1 (the products' roundings and those of n itself), and one that is
+// loaded is normalised when n is more than 8 off: a handed-in one is, and what a
+// substep stored is taken as it is, as in the fused loop.
 //
 // Every operation is written out as a single rounding, so the substep kernel
 // and the fused loop give the same bits whatever the compiler hoists.
@@ -108,7 +110,7 @@ __device__ __forceinline__ RigidLane rigid_load(const IntegrateLaunch& L, int p,
   S.om = P.omega[S.a];
   S.q = P.quat[S.c < 3 ? S.c + 1 : 0];
   const double n = quad_norm2(S.q);
-  if (!near_one(n, 64)) S.q = __dmul_rn(S.q, __ddiv_rn(1.0, __dsqrt_rn(n)));
+  if (!near_one(n, 8)) S.q = __dmul_rn(S.q, __ddiv_rn(1.0, __dsqrt_rn(n)));
   double rb, rc;
   rigid_rotation(S, rb, rc);
   return S;

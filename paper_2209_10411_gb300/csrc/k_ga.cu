@@ -352,7 +352,8 @@ extern "C" mi_status mi_ga_run(int n_ind, int n_genes, const float* hull, int m,
   float* fnxt = fitB;
   const long long ng = (long long)n_ind * n_genes;
   const size_t gsm = sizeof(float4) * (size_t)n_genes;
-  if (gsm > 48 * 1024 &&
+  // with the reduction's static part: 48 KB is the limit of both together
+  if (gsm + sizeof(float) * GA_FIT_THREADS > 48 * 1024 &&
       (cudaFuncSetAttribute(k_ga_fitness, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm) != cudaSuccess ||
        cudaFuncSetAttribute(k_ga_children, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gsm) != cudaSuccess))
     return MI_ECUDA;

@@ -518,7 +518,17 @@ class Simulation:
         return v
 
     # -- timing -----------------------------------------------------------
-    def set_tuning(self, bulk_block_x=128, bulk_rows=1, bulk_pairs=False, list_blocks_per_sm=8):
+    def set_tuning(self, bulk_block_x=None, bulk_rows=None, bulk_pairs=None, list_blocks_per_sm=None):
+        """Launch shapes (mi_delbm_set_tuning); what is not given stays as it is,
+        but that paired nodes and more than 128 threads exclude each other: the one
+        that is not given gives way."""
+        now = self.get_tuning()
+        if bulk_pairs is None:
+            bulk_pairs = 0 if bulk_block_x is not None and int(bulk_block_x) > 128 else now["bulk_pairs"]
+        if bulk_block_x is None:
+            bulk_block_x = min(now["bulk_block_x"], 128) if bulk_pairs else now["bulk_block_x"]
+        bulk_rows = now["bulk_rows"] if bulk_rows is None else bulk_rows
+        list_blocks_per_sm = now["list_blocks_per_sm"] if list_blocks_per_sm is None else list_blocks_per_sm
         self._check(lib.mi_delbm_set_tuning(self.h, int(bulk_block_x), int(bulk_rows), int(bulk_pairs),
                                             int(list_blocks_per_sm)))
 

@@ -401,7 +401,7 @@ mi_status mi_delbm_set_graphs(mi_delbm *h, int enable);
  * fraction, refill and boundary-node kernels, from 2/4/8/16/32) by timing each candidate
  * with CUDA events on the handle's stream, and use the fastest from then on.
  * With cache_path != NULL, a line {"key": ..., "bulk_block_x": .., "list_blocks_per_sm": ..}
- * for this device, lattice, storage and particle count is read from that file
+ * for this device, lattice, storage, particle count and kernel revision is read from that file
  * if present (no timing), else appended after timing.  The list kernels are
  * tuned only when the last step produced boundary nodes, so call this after
  * at least one step.  The trial launches leave the populations untouched and

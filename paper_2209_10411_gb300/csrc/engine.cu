@@ -1268,12 +1268,16 @@ long long mi_delbm_launch_count(const mi_delbm* h) { return h ? h->launches : 0;
 // Autotuner: launch shapes of the bulk and list kernels, measured with CUDA
 // events and cached as one JSON object per line keyed by device and workload.
 // ---------------------------------------------------------------------------
+// Counted up when a kernel whose launch shape is tuned changes: shapes found for
+// other kernels are not taken for measured ones.
+static constexpr int TUNED_KERNELS = 3;
+
 std::string mi_delbm::tune_key() const {
   int major = 0, minor = 0;
   cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, cfg.device);
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, cfg.device);
   std::ostringstream k;
-  k << "sm_" << major << minor << "/" << sm_count << "sm/" << cfg.nx << "x" << cfg.ny << "x" << cfg.nz << "/st"
+  k << "kernels" << TUNED_KERNELS << "/sm_" << major << minor << "/" << sm_count << "sm/" << cfg.nx << "x" << cfg.ny << "x" << cfg.nz << "/st"
     << cfg.storage << "/np" << n_particles << "/bb" << cfg.bb_mode << (forcing() ? "/force" : "");
   return k.str();
 }

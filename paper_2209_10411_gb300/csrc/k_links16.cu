@@ -34,7 +34,8 @@
 // the accurate signs.  A step ends it when it is below 2e-5 or when the error
 // Newton's quadratic convergence leaves behind, |g''/2g'| step^2 with g'' in
 // FP32 from the same sums, is below 1e-7 (usually the first step); at most
-// four steps.  The largest error of q over 2.3 M links is 6.9e-7.
+// four steps.  The largest error of q over 2.3 M links is 6.9e-7; a link that grazes
+// the surface (both roots within 1e-3 of each other) can need more than four.
 #include "mi_internal.cuh"
 
 namespace mi {

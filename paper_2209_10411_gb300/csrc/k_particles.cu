@@ -764,7 +764,11 @@ cudaError_t launch_classify(const ParticleLaunch& L, cudaStream_t s) {
 // inside a bracket that starts at [0, 1] (the exact flags guarantee
 // g(0) < 0 <= g(1)) and moves with the accurate signs.  A step ends it when it
 // is below 2e-5 or when the error Newton's quadratic convergence leaves behind,
-// |h'' / 2 h'| step^2, is below 1e-7 (usually the first step); at most four steps.
+// |h'' / 2 h'| step^2, is below 1e-7 (usually the first step).  A link that
+// grazes the surface takes more: with both roots of a sphere within 1e-3 of each other
+// a step halves the error until it is as small as their distance, and one from
+// between them leaves the bracket (bisection), so that up to 24 steps are
+// allowed (four left 4e-4 at a depth of 1e-7 lu, 3e-5 at 1e-5).
 //
 // The residual: q = qh + ql with qh on the particle's grid, so that a link point
 // less a ball's centre is u + m, u a multiple of the grid (exact) and m below
@@ -883,7 +887,7 @@ __device__ __forceinline__ float link_root(const float4* __restrict__ bw, int nb
   lo = 0.f;
   hi = 1.f;
   const float ee = e[0] * e[0] + e[1] * e[1] + e[2] * e[2], inv_grid = 1.0f / grid;
-  for (int it = 0; it < 4; ++it) {
+  for (int it = 0; it < 24; ++it) {
     float gp, gpp;
     const float g = residual<EXACT>(bw, nb, n, e, q, grid, inv_grid, ee, gp, gpp);
     if (g >= 0.f) hi = q;

@@ -114,7 +114,7 @@ struct mi_delbm {
   bool unfused_dem = false;          // DEM substeps as separate launches even where the fused kernel applies
   bool cover_uncover = false;        // covered/uncovered-node momentum joins the hydrodynamic sums
   // blocks of the box kernels, sized per particle: device offsets (particle
-  // p owns blocks [off[p], off[p + 1])) of the flag and clear kernels, then of
+  // p owns blocks [off[p], off[p + 1])) of the flag kernel and the prologue's clear, then of
   // the classification, max_particles + 1 each; the totals are the grids
   int* dblk_off = nullptr;
   int flag_blocks = 1, classify_blocks = 1;

@@ -438,21 +438,22 @@ __global__ void __launch_bounds__(128, W == 4 ? 5 : (FORCE ? 7 : 8))
 
 template <int ST, bool FORCE, int W>
 static cudaError_t launch_bulk16_t(const BulkLaunch& L, cudaStream_t s) {
-  constexpr int S16 = ST == MI_STORE_F32 ? MI_STORE_F16_DEV : ST;
-  using T16 = typename Store<S16>::T;
+  using T = typename Store<ST>::T;
   const unsigned n = (unsigned)((long long)L.g.nx / W * L.g.ny * L.g.nz), bx = (unsigned)L.block_x;
-  k_bulk16<S16, FORCE, W><<<n / bx + (n % bx ? 1u : 0u), bx, 0, s>>>(
-      reinterpret_cast<const T16*>(L.A), reinterpret_cast<T16*>(L.B), L.g, L.p, fast_div((unsigned)L.g.nx / W),
+  k_bulk16<ST, FORCE, W><<<n / bx + (n % bx ? 1u : 0u), bx, 0, s>>>(
+      static_cast<const T*>(L.A), static_cast<T*>(L.B), L.g, L.p, fast_div((unsigned)L.g.nx / W),
       fast_div((unsigned)L.g.ny), n);
   return cudaGetLastError();
 }
 
 template <int ST>
 static cudaError_t launch_bulk_st(const BulkLaunch& L, cudaStream_t s) {
-  if (ST != MI_STORE_F32 && L.nodes == 4 && L.g.nx % 4 == 0)
-    return L.forcing ? launch_bulk16_t<ST, true, 4>(L, s) : launch_bulk16_t<ST, false, 4>(L, s);
-  if (ST != MI_STORE_F32 && L.nodes == 2 && L.g.nx % 2 == 0)
-    return L.forcing ? launch_bulk16_t<ST, true, 2>(L, s) : launch_bulk16_t<ST, false, 2>(L, s);
+  if constexpr (ST != MI_STORE_F32) {
+    if (L.nodes == 4 && L.g.nx % 4 == 0)
+      return L.forcing ? launch_bulk16_t<ST, true, 4>(L, s) : launch_bulk16_t<ST, false, 4>(L, s);
+    if (L.nodes == 2 && L.g.nx % 2 == 0)
+      return L.forcing ? launch_bulk16_t<ST, true, 2>(L, s) : launch_bulk16_t<ST, false, 2>(L, s);
+  }
   return L.forcing ? launch_bulk_t<ST, true>(L, s) : launch_bulk_t<ST, false>(L, s);
 }
 

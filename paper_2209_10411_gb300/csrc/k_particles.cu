@@ -12,13 +12,8 @@
 #include <cfloat>
 #include <climits>
 
-#include <cooperative_groups.h>
-#include <cooperative_groups/scan.h>
-
 #include "mi_internal.cuh"
 #include "rigid_dev.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace mi {
 

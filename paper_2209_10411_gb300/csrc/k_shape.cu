@@ -16,7 +16,7 @@ namespace {
 
 constexpr int SH_THREADS = 256;
 constexpr int SH_MAX_BALLS = 4096;  // balls of one particle
-constexpr int SH_STAGED = 512;      // staged in shared memory up to this many (8 KB), else read from global memory
+constexpr int SH_STAGED = 512;      // staged in shared memory up to this many (8 KB, and 8 KB by pairs), else read from global memory
 constexpr int SH_POOL = 64;          // band cells of a warp waiting for their gradients (at most 31 + 32)
 constexpr unsigned SH_FULL = 0xffffffffu;
 

@@ -103,13 +103,6 @@ template <> __device__ __forceinline__ float dev16<MI_STORE_F16_DEV>(unsigned sh
 template <> __device__ __forceinline__ float dev16<MI_STORE_BF16_DEV>(unsigned short u) {
   return __uint_as_float((unsigned)u << 16);
 }
-template <int ST> __device__ __forceinline__ unsigned short pack16(float h);
-template <> __device__ __forceinline__ unsigned short pack16<MI_STORE_F16_DEV>(float h) {
-  return __half_as_ushort(__float2half_rn(h));
-}
-template <> __device__ __forceinline__ unsigned short pack16<MI_STORE_BF16_DEV>(float h) {
-  return __bfloat16_as_ushort(__float2bfloat16_rn(h));
-}
 
 // ---------------------------------------------------------------------------
 // Packed FP32 pairs: one instruction for both values, each a single rounding
@@ -299,7 +292,7 @@ struct ParticleLaunch {
   unsigned cap_bc, cap_links, cap_new;
   int cover_uncover;
   // box kernels: particle p owns blocks [off[p], off[p + 1]) of a 1D grid,
-  // flag_off for the flag and clear kernels (flag_blocks in all), cls_off for
+  // flag_off for the flag kernel and the prologue's clear (flag_blocks in all), cls_off for
   // the row-per-warp classification (classify_blocks in all)
   const int* flag_off;
   const int* cls_off;

@@ -35,7 +35,7 @@ BYTES_PER_NODE = {0: 152, 1: 76, 2: 76}   # 19 loads + 19 stores of the stored t
 # processed (profiles/k_bulk.md);
 # keyed by (storage, four-node kernel).  Reported only for the kernel that
 # was captured.
-BULK_TRAFFIC = {(0, False): 4 * 1222.3e6, (1, True): 4 * 593.9e6}
+BULK_TRAFFIC = {(0, False): 4 * 1222.2e6, (1, True): 4 * 589.9e6}
 STORAGE = {"f32": 0, "f16": 1, "bf16": 2}
 DTYPE_NAME = {0: "f32", 1: "f16-dev/f32-compute", 2: "bf16-dev/f32-compute"}
 def _peaks():

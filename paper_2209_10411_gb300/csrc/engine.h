@@ -20,8 +20,8 @@ struct TuneChoice {
   int bulk_pairs = 0;         // 16-bit storages: 0 one node per thread; 1, 2: two x-adjacent nodes (nx even);
                               // 3: four (nx a multiple of 4)
   int list_blocks_per_sm = 4; // grid of the list kernels (links, refill, boundary, near) per SM: the boundary nodes of
-                              // 300 particles took 569 us with 4, 603 with 8, 575 with 32 (fewer nodes at a time share
-                              // more of the caches)
+                              // 300 particles take 509 us with 2, 446 with 4, 478 with 8, 442 with 32 (FP32; BF16 503,
+                              // 406, 422, 381), and few blocks leave more of the chip to the bulk kernel beside them
   bool tuned = false;
 };
 

@@ -665,7 +665,7 @@ __global__ void __launch_bounds__(128) k_near(BoundaryLaunch L) {
 // own, a 32-byte sector each.  One kernel per link (38 gathers: its own node's
 // too) that kept G for a second kernel per node took 497 + 320 us for 0.82 M
 // nodes and 3.35 M links in FP32 (300 particles, 512^3) and 27 + 22 us for
-// three cobbles' 32 k nodes; together they take 484 us (417 in 16 bits) and 24
+// three cobbles' 32 k nodes; together they take 467 us (408 in 16 bits) and 27
 // us (569 and 474 before the list came nearly in particle order).  (A thread per node that goes through its links in turn, with atomics of
 // its own where the particle changes, took 1200 us.)  The nodes around
 // uncovered ones (k_near) are recomputed by the same launch.

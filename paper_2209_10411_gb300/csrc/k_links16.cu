@@ -9,7 +9,7 @@
 // unit.  Each such unit is 2e-7 of a light particle's velocity (radius 3 lu,
 // BF16), so the states after 20 steps would depend on which kernel formed q: 1e-7 apart.
 // So 16-bit runs keep the arithmetic that they had: 300 particles, 3.35 M
-// links of balls 8 to 64 a particle take 842 us, 491 with k_links_q.
+// links of particles of 8 to 64 balls take 850 us, 494 with k_links_q.
 //
 // Inputs: the body-frame link origin p and direction e as float pairs hi + lo
 // (the prologue forms the particle's frame in FP64 once per step; each link
